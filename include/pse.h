@@ -479,7 +479,8 @@ enum {
     PSE_STAGE_NEIGHBOURS,     /* neighbour count, scan, fill                  */
     PSE_STAGE_MATVEC,         /* M_r q_j, all iterations                      */
     PSE_STAGE_LANCZOS_UPDATE, /* three-term update + ||w||, all iterations    */
-    PSE_STAGE_EIGEN,          /* FP64 T_j^{1/2} e_1 + stop test, all iterations */
+    PSE_STAGE_EIGEN,          /* 0: the FP64 T_j^{1/2} e_1 and the stop test are
+                                 a block of the update's launch               */
     PSE_STAGE_FINAL,          /* x = V y, + wave part, caller order           */
     PSE_STAGE_WAVE_NOISE,     /* k-space noise and B^{1/2} scaling (fused
                                  path: with the first FFT pass)               */

@@ -8,9 +8,10 @@
 //   update  alpha_j = q_j.u / beta_{j-1}^2,
 //           q_{j+1} = u/beta_{j-1} - alpha_j q_j/beta_{j-1} - beta_{j-1} q_{j-1}/beta_{j-2}
 //                                               (+ deterministic ||q_{j+1}||^2)
-//   eigen   y_j = T_j^{1/2} e_1 in FP64 (one warp), stop test
-//           ||y_j - [y_{j-1}; 0]|| / ||y_j|| < tol  (= ||x_j - x_{j-1}|| / ||x_j||
-//           for an orthonormal basis)
+//           and, in one more block of the same launch, y_j = T_j^{1/2} e_1 in
+//           FP64 (one warp; T_j needs alpha_j but not beta_j, so it runs beside
+//           the vector update), stop test ||y_j - [y_{j-1}; 0]|| / ||y_j|| < tol
+//           (= ||x_j - x_{j-1}|| / ||x_j|| for an orthonormal basis)
 // and finally x = beta_0 sum_i y_i q_i / beta_{i-1}.  Scalars are FP64; the
 // reducing kernels run persistent grids (a fixed multiple of the SM count)
 // and their per-block partial sums are added in block order by the last
@@ -73,14 +74,17 @@ __device__ __forceinline__ void lz_init_body(int64_t N, const SampleArgs<T> *arg
     const double bsum = block_total<T>(part, sh);
     double total;
     if (grid_sum_last(bsum, partials, &lz->counter_init, sh, &total, bidx, nblk) && threadIdx.x == 0) {
-        lz->beta[0] = sqrt(total);
+        const double bi = total > 0.0 ? rsqrt(total) : 0.0;
+        lz->beta[0] = total * bi;
+        lz->binv[0] = bi;
+        lz->tmax = 0.0;
         lz->iter = 1;
-        lz->jeig = 0;
         lz->J = 0;
         lz->converged = 0;
         lz->cont = 1;
         lz->active = 1;
-        lz->rel = 0.0;
+        lz->num = 0.0;
+        lz->den = 0.0;
     }
 }
 
@@ -97,6 +101,19 @@ __global__ void __launch_bounds__(256) k_lz_init_batch(const BSys *__restrict__ 
     const BSys &S = sys[tab[blockIdx.x]];
     lz_init_body<float>(S.N, S.d.args, S.system, S.d.pos_sorted, S.d.basis, S.d.rec, S.d.partials, S.d.lz, S.d.pc_on,
                         (int)blockIdx.x - S.b0[BK_INIT], S.nb[BK_INIT], sh);
+}
+
+// alpha_j = q_j.u / beta_{j-1}^2 and the coefficients of the update, by
+// multiplications with the stored 1/beta (an FP64 division costs about as much
+// as the rest of this tail).  beta_{j-1} = 0 (binv = 0): the Krylov space is
+// invariant and the loop has stopped.
+__device__ __forceinline__ void lz_alpha(LzState *lz, int j, double total) {
+    const double bi = lz->binv[j - 1];
+    const double alpha = total * bi * bi;
+    lz->alpha[j] = alpha;
+    lz->c_u = bi;
+    lz->c_q = alpha * bi;
+    lz->c_p = j >= 2 ? lz->beta[j - 1] * lz->binv[j - 2] : 0.0;
 }
 
 // ------------------------------------------------------------------ near-field matvec
@@ -360,13 +377,7 @@ __device__ __forceinline__ void lz_matvec_body(int64_t N, int K, const Geom<T> &
     const double bsum = block_total<T>(part, sh);
     double total;
     if (grid_sum_last(bsum, partials, &lz->counter_mv, sh, &total, bidx, nblk) && threadIdx.x == 0) {
-        const double b1 = lz->beta[j - 1];
-        const bool ok = b1 > 0.0;  // beta_{j-1} = 0: invariant subspace, the eigen kernel stops the loop
-        const double alpha = ok ? total / (b1 * b1) : 0.0;
-        lz->alpha[j] = alpha;
-        lz->c_u = ok ? (float)(1.0 / b1) : 0.f;
-        lz->c_q = ok ? (float)(alpha / b1) : 0.f;
-        lz->c_p = (ok && j >= 2) ? (float)(b1 / lz->beta[j - 2]) : 0.f;
+        lz_alpha(lz, j, total);
     }
 }
 
@@ -547,13 +558,7 @@ __global__ void __launch_bounds__(PSE_TILE_THREADS, 4) k_lz_matvec_tiled(
     const double bsum = block_sum_fw(part, sh);
     double total;
     if (grid_sum_last(bsum, partials, &lz->counter_mv, sh, &total) && threadIdx.x == 0) {
-        const double b1 = lz->beta[j - 1];
-        const bool ok = b1 > 0.0;
-        const double alpha = ok ? total / (b1 * b1) : 0.0;
-        lz->alpha[j] = alpha;
-        lz->c_u = ok ? (float)(1.0 / b1) : 0.f;
-        lz->c_q = ok ? (float)(alpha / b1) : 0.f;
-        lz->c_p = (ok && j >= 2) ? (float)(b1 / lz->beta[j - 2]) : 0.f;
+        lz_alpha(lz, j, total);
     }
 }
 
@@ -598,329 +603,325 @@ __global__ void __launch_bounds__(PSE_BATCH_MV_THREADS) k_lz_matvec_batch(const 
                                                      sh);
 }
 
+// ------------------------------------------------------------------ T_j^{1/2} e_1 and the stop test
+// One warp.  The matrix square root as an integral, discretised after Hale,
+// Higham & Trefethen, SIAM J. Numer. Anal. 46, 2505 (2008), method 3:
+//   T^{1/2} e_1 = sum_l w_l T (T + s_l I)^{-1} e_1,
+// nodes s_l and weights w_l from Jacobi elliptic functions for a spectrum in
+// [2^-18, 1], scaled by the power of four c >= ||T|| (exactly: shifts c s_l,
+// weights c^{1/2} w_l).  31 nodes leave a relative error of 1.5e-17 on that
+// interval (evaluated with 40 digits), so the result is T^{1/2} e_1 to
+// rounding (1-4e-15 against an eigendecomposition for j = 1..64).  Lane l
+// solves the system of node l through the trailing determinants
+//   phi_i = (alpha_i + s) phi_{i+1} - beta_i^2 phi_{i+2},
+//   x_i = (-1)^{i+1} beta_1 .. beta_{i-1} phi_{i+1} / phi_1,
+// j dependent multiply-adds and one division, where QL sweeps chain dozens of
+// divisions and square roots (FP64 latency is what this costs).  (T x)_i =
+// -s x_i for i >= 2, so no component cancels.  Lane 31 runs the recurrence at
+// the shift -2^-18 c: all phi_i > 0 there means that the spectrum lies above
+// it (Sylvester); otherwise (a zero mode of coincident spheres, or no
+// convergence) the QL route below is taken.
+// It was one launch of 12-19 us after each update (Newton-Schulz, QL); as a
+// block beside the update it takes 4 us, hidden behind the vectors.
+__constant__ double c_hht_s[32] = {
+    5.7983172601720927e-8, 5.4321516364628967e-7, 1.6334814437543627e-6, 3.5979661192943067e-6,
+    6.9216981084029469e-6, 1.2425309911265321e-5, 2.1467667841819654e-5, 3.6281423144883104e-5,
+    6.0524386131848248e-5, 0.00010018300523163798, 0.00016505141758121806, 0.00027115231705414841,
+    0.00044470021775750382, 0.00072859332384748145, 0.0011930574307098304, 0.001953125,
+    0.0031974129387513047, 0.0052357016469499542, 0.0085781322187369926, 0.014068466414259757,
+    0.023112175112024554, 0.038077289224902505, 0.063027442481034705, 0.10514188625930458,
+    0.17769500132631345, 0.30701023096143713, 0.55112158980091238, 1.0602371281842982,
+    2.3353171719278134, 7.0224425253874365, 65.789729924363965, -3.814697265625e-6};
+__constant__ double c_hht_w[32] = {
+    0.00030813623989951382, 0.00032687093299644554, 0.00036547944964625105, 0.00042630934808390455,
+    0.00051305944420673084, 0.00063100491451650686, 0.00078731848148126131, 0.0009915074693214191,
+    0.0012559938481394102, 0.0015968736736132673, 0.0020349044825956523, 0.002596785671713454,
+    0.0033168201568205391, 0.0042390802236798112, 0.0054202550989604143, 0.0069334495341588189,
+    0.0088733664177913662, 0.011363614366040764, 0.014567486387701018, 0.018704789507856225,
+    0.024079907193853152, 0.031131965811612131, 0.040530984970311739, 0.053375470369097509,
+    0.071630110008854434, 0.099187181846279507, 0.14477216591543603, 0.23141836745246686,
+    0.43699734258975575, 1.1752613581759009, 10.379366401483795, 0.0};
+
+// y[0..k-1] = T_k^{1/2} e_1 by the QL eigendecomposition (Golub & Van Loan,
+// Sec. 8.3): every lane runs the scalar recurrences redundantly and applies
+// each plane rotation to its own rows of the eigenvector matrix, then
+// y = Q diag(sqrt(max(lambda, 0))) Q^T e_1.  ws: PSE_QL_WORK doubles.
+__device__ __noinline__ void tri_sqrt_e1_ql(int k, const double *alpha, const double *beta, double *y, double *ws) {
+    double *Q = ws, *d = ws + PSE_MAXIT * (PSE_MAXIT + 1), *e = d + PSE_MAXIT + 1;
+    constexpr int LD = PSE_MAXIT + 1;
+    const int lane = threadIdx.x & 31;
+    for (int i = lane; i < k; i += 32) {
+        d[i] = alpha[i + 1];
+        e[i] = (i + 1 < k) ? beta[i + 1] : 0.0;
+        for (int c = 0; c < k; ++c) Q[i * LD + c] = (i == c) ? 1.0 : 0.0;
+    }
+    __syncwarp();
+    const double eps = 2.220446049250313e-16;
+    for (int l = 0; l < k; ++l) {
+        for (int sweep = 0; sweep < 60; ++sweep) {
+            int m = l;
+            for (; m < k - 1; ++m) {
+                const double dd = fabs(d[m]) + fabs(d[m + 1]);
+                if (fabs(e[m]) <= eps * dd) break;
+            }
+            if (m == l) break;
+            // shift from the leading 2x2 block (entries are O(mobility), far
+            // from overflow, so plain square roots replace hypot)
+            double g = (d[l + 1] - d[l]) / (2.0 * e[l]);
+            double r = sqrt(fma(g, g, 1.0));
+            g = d[m] - d[l] + e[l] / (g + (g >= 0 ? r : -r));
+            double s = 1.0, c = 1.0, p = 0.0;
+            int i = m - 1;
+            bool deflated = false;
+            for (; i >= l; --i) {
+                const double f = s * e[i], b = c * e[i];
+                r = sqrt(fma(f, f, g * g));
+                __syncwarp();
+                if (lane == 0) e[i + 1] = r;
+                __syncwarp();
+                if (r == 0.0) {
+                    if (lane == 0) { d[i + 1] -= p; e[m] = 0.0; }
+                    __syncwarp();
+                    deflated = true;
+                    break;
+                }
+                const double rinv = 1.0 / r;  // one division per rotation
+                s = f * rinv;
+                c = g * rinv;
+                g = d[i + 1] - p;
+                r = (d[i] - g) * s + 2.0 * c * b;
+                p = s * r;
+                __syncwarp();
+                if (lane == 0) d[i + 1] = g + p;
+                __syncwarp();
+                g = c * r - b;
+                for (int row = lane; row < k; row += 32) {
+                    const double qa = Q[row * LD + i], qb = Q[row * LD + i + 1];
+                    Q[row * LD + i + 1] = s * qa + c * qb;
+                    Q[row * LD + i] = c * qa - s * qb;
+                }
+                __syncwarp();
+            }
+            if (deflated && i >= l) continue;
+            __syncwarp();
+            if (lane == 0) { d[l] -= p; e[l] = g; e[m] = 0.0; }
+            __syncwarp();
+        }
+    }
+    __syncwarp();
+    for (int c = lane; c < k; c += 32) e[c] = sqrt(fmax(d[c], 0.0)) * Q[c];
+    __syncwarp();
+    for (int row = lane; row < k; row += 32) {
+        double acc = 0.0;
+        for (int c = 0; c < k; ++c) acc += Q[row * LD + c] * e[c];
+        y[row] = acc;
+    }
+    __syncwarp();
+}
+
+// T_k^{1/2} e_1 into sm->y (one warp) by the rational sum, QL where the
+// spectrum is too wide for it.
+// phi_i (then the terms of y_i) of each lane's node lie in shared memory for
+// j <= 8 and in the global workspace above: the 19 KB that j = 64 needs would
+// change the SMs' split between L1 and shared memory, which costs the kernels
+// of the wave branch beside this one (64-system batch 0.5% slower).
+#define PSE_EIG_ROWS 8
+struct EigSmem {
+    double ph[PSE_EIG_ROWS][33];
+    double a[PSE_MAXIT + 2], b[PSE_MAXIT + 2], y[PSE_MAXIT + 2];
+};
+static_assert(PSE_QL_WORK >= PSE_MAXIT * 33, "the rational sum's terms fit the QL workspace");
+__device__ __forceinline__ void tri_sqrt_e1(int k, double bound, EigSmem *sm, const double *alpha,
+                                            const double *beta, double *qlws) {
+    const int lane = threadIdx.x & 31;
+    for (int i = lane + 1; i <= k; i += 32) {
+        sm->a[i] = alpha[i];
+        sm->b[i] = i < k ? beta[i] : 0.0;
+    }
+    // c = 4^p >= bound: exponent of the bound rounded up to an even one
+    int ex = 0;
+    frexp(bound, &ex);
+    const int p = (ex + 1) >> 1;
+    const double c = ldexp(1.0, 2 * p);
+    const double s = c_hht_s[lane] * c;
+    __syncwarp();
+    double(*ph)[33] = k <= PSE_EIG_ROWS ? sm->ph : reinterpret_cast<double(*)[33]>(qlws);
+    double p1 = 1.0, p2 = 0.0;  // phi_{i+1}, phi_{i+2}
+    bool pos = bound > 0.0 && isfinite(bound);
+    for (int i = k; i >= 1; --i) {
+        ph[i - 1][lane] = p1;  // phi_{i+1}, the minor of x_i
+        const double bi = sm->b[i];
+        const double t = fma(sm->a[i] + s, p1, -bi * bi * p2);
+        p2 = p1;
+        p1 = t;
+        pos = pos && t > 0.0;
+    }
+    if (!__all_sync(0xffffffffu, pos)) {
+        tri_sqrt_e1_ql(k, alpha, beta, sm->y, qlws);
+        return;
+    }
+    double f = ldexp(c_hht_w[lane], p) / p1;  // w_l / phi_1, times the running beta product with its sign
+    {
+        const double x1 = f * ph[0][lane];
+        double v = sm->a[1] * x1;
+        if (k > 1) v -= sm->b[1] * sm->b[1] * f * ph[1][lane];
+        ph[0][lane] = v;
+    }
+    f *= -s;
+    for (int i = 2; i <= k; ++i) {
+        f *= -sm->b[i - 1];
+        ph[i - 1][lane] *= f;
+    }
+    __syncwarp();
+    // row sums, 32 / parts rows at a time, `parts` lanes per row
+    const int parts = k <= 8 ? 4 : (k <= 16 ? 2 : 1), span = 32 / parts;
+    for (int r0 = 0; r0 < k; r0 += span) {
+        const int row = r0 + lane / parts, part = lane % parts;
+        double v0 = 0.0, v1 = 0.0;
+        if (row < k)
+            for (int l = part * span; l < (part + 1) * span; l += 2) {
+                v0 += ph[row][l];
+                v1 += ph[row][l + 1];
+            }
+        v0 += v1;
+        for (int o = 1; o < parts; o <<= 1) v0 += __shfl_xor_sync(0xffffffffu, v0, o);
+        if (row < k && part == 0) sm->y[row] = v0;
+    }
+    __syncwarp();
+}
+
+// The T_j block of one update launch (its first warp): y_j, the stop test
+// without beta_j (||y_j - y_{j-1}||^2 < tol^2 ||y_j||^2), and the
+// coefficients of the final combination once it passes.
+__device__ __forceinline__ void lz_eig_body(LzState *lz, int k, const LzStop &st, EigSmem *sm, double *qlws) {
+    const int lane = threadIdx.x & 31;
+    // rows 1..k of T_k: |T| row sums of rows < k already include their beta
+    const double bk1 = k > 1 ? lz->beta[k - 1] : 0.0, ak = lz->alpha[k];
+    double tmax = lz->tmax;
+    if (k > 1) tmax = fmax(tmax, lz->alpha[k - 1] + bk1 + (k > 2 ? lz->beta[k - 2] : 0.0));
+    tmax = fmax(tmax, ak + bk1);
+    tri_sqrt_e1(k, tmax, sm, lz->alpha, lz->beta, qlws);
+    double num = 0.0, den = 0.0;
+    for (int row = lane; row < k; row += 32) {
+        const double yr = sm->y[row], prev = row < k - 1 ? lz->y[row] : 0.0;
+        num += (yr - prev) * (yr - prev);
+        den += yr * yr;
+    }
+    for (int o = k <= 8 ? 4 : 16; o > 0; o >>= 1) {
+        num += __shfl_xor_sync(0xffffffffu, num, o);
+        den += __shfl_xor_sync(0xffffffffu, den, o);
+    }
+    num = __shfl_sync(0xffffffffu, num, 0);
+    den = __shfl_sync(0xffffffffu, den, 0);
+    int conv, stop;
+    if (st.fixed_iter > 0) {
+        stop = conv = k >= st.fixed_iter;
+    } else {
+        conv = k >= 2 && den > 0.0 && num < st.tol * st.tol * den;
+        stop = conv || k >= st.max_iter;
+    }
+    __syncwarp();
+    for (int row = lane; row < k; row += 32) lz->y[row] = sm->y[row];
+    if (lane == 0) {
+        lz->tmax = tmax;
+        lz->num = num;
+        lz->den = k >= 2 ? den : 0.0;
+        lz->stop_y = stop;
+        lz->converged = conv;
+    }
+}
+
+// Lanczos update of one system: block 0 is its T_j block (first, so that it is
+// placed at once in a launch of several waves), blocks 1 .. nblk do the vectors.
 template <typename T>
 __device__ __forceinline__ void lz_update_body(int64_t N, V4<T> *basis, Rec<T> *rec, const V4<T> *u, double *partials,
-                                               LzState *lz, const float *__restrict__ pc, int bidx, int nblk,
-                                               double *sh) {
+                                               LzState *lz, double *qlws, const float *__restrict__ pc,
+                                               const LzStop &st, int bidx, int nblk, double *sh, EigSmem *esm) {
     const int j = lz->iter;
     if (j > PSE_MAXIT || !lz->active) return;
-    // coefficients in the working precision; the FP64 path recomputes them exactly
-    T cu, cq, cp;
-    if constexpr (sizeof(T) == 4) {
-        cu = lz->c_u; cq = lz->c_q; cp = lz->c_p;
+    double bsum = 0.0;
+    if (bidx == 0) {
+        if (threadIdx.x < 32) lz_eig_body(lz, j, st, esm, qlws);
+        __threadfence();
+        __syncthreads();
     } else {
-        const double b1 = lz->beta[j - 1];
-        const bool ok = b1 > 0.0;
-        cu = ok ? 1.0 / b1 : 0.0;
-        cq = ok ? lz->alpha[j] / b1 : 0.0;
-        cp = (ok && j >= 2) ? b1 / lz->beta[j - 2] : 0.0;
-    }
-    const V4<T> *qj = basis + (int64_t)(j - 1) * N;
-    const V4<T> *qp = basis + (int64_t)(j - 2) * N;
-    V4<T> *qn = basis + (int64_t)j * N;
-    typename Part<T>::type part = 0;
-    for (int64_t s = bidx * (int64_t)blockDim.x + threadIdx.x; s < N; s += (int64_t)nblk * blockDim.x) {
-        const V4<T> us = u[s];
-        const V4<T> a = qj[s];
-        V4<T> w;
-        w.x = cu * us.x - cq * a.x;
-        w.y = cu * us.y - cq * a.y;
-        w.z = cu * us.z - cq * a.z;
-        w.w = T(0);
-        if (j >= 2) {
-            const V4<T> b = qp[s];
-            w.x -= cp * b.x;
-            w.y -= cp * b.y;
-            w.z -= cp * b.z;
-        }
-        qn[s] = w;
-        if constexpr (sizeof(T) == 4) {
-            if (pc) {
-                V4<T> p;
-                sym3_apply(pc + s * 16, w.x, w.y, w.z, p.x, p.y, p.z);
-                p.w = T(0);
-                rec[s].q = p;
+        const T cu = (T)lz->c_u, cq = (T)lz->c_q, cp = (T)lz->c_p;
+        const V4<T> *qj = basis + (int64_t)(j - 1) * N;
+        const V4<T> *qp = basis + (int64_t)(j - 2) * N;
+        V4<T> *qn = basis + (int64_t)j * N;
+        typename Part<T>::type part = 0;
+        for (int64_t s = (bidx - 1) * (int64_t)blockDim.x + threadIdx.x; s < N; s += (int64_t)nblk * blockDim.x) {
+            const V4<T> us = u[s];
+            const V4<T> a = qj[s];
+            V4<T> w;
+            w.x = cu * us.x - cq * a.x;
+            w.y = cu * us.y - cq * a.y;
+            w.z = cu * us.z - cq * a.z;
+            w.w = T(0);
+            if (j >= 2) {
+                const V4<T> b = qp[s];
+                w.x -= cp * b.x;
+                w.y -= cp * b.y;
+                w.z -= cp * b.z;
+            }
+            qn[s] = w;
+            if constexpr (sizeof(T) == 4) {
+                if (pc) {
+                    V4<T> p;
+                    sym3_apply(pc + s * 16, w.x, w.y, w.z, p.x, p.y, p.z);
+                    p.w = T(0);
+                    rec[s].q = p;
+                } else {
+                    rec[s].q = w;
+                }
             } else {
                 rec[s].q = w;
             }
-        } else {
-            rec[s].q = w;
+            part += w.x * w.x + w.y * w.y + w.z * w.z;
         }
-        part += w.x * w.x + w.y * w.y + w.z * w.z;
+        bsum = block_total<T>(part, sh);
     }
-    const double bsum = block_total<T>(part, sh);
     double total;
-    if (grid_sum_last(bsum, partials, &lz->counter_up, sh, &total, bidx, nblk) && threadIdx.x == 0) {
-        lz->beta[j] = sqrt(total);
-        lz->iter = j + 1;
+    if (grid_sum_last(bsum, partials, &lz->counter_up, sh, &total, bidx, nblk + 1)) {
+        // every block is done: join beta_j with the T_j block's decision
+        __shared__ int s_stop;
+        if (threadIdx.x == 0) {
+            const double bi = total > 0.0 ? rsqrt(total) : 0.0;
+            lz->beta[j] = total * bi;
+            lz->binv[j] = bi;
+            lz->iter = j + 1;
+            // beta_j = 0: the Krylov space is invariant and T_j^{1/2} e_1 is exact
+            const bool breakdown = st.fixed_iter <= 0 && !(total > 0.0);
+            const int stop = __ldcg(&lz->stop_y) || breakdown;
+            if (breakdown) lz->converged = 1;
+            if (stop) lz->J = j;
+            lz->cont = stop ? 0 : 1;
+            s_stop = stop;
+            if (st.h) cudaGraphSetConditional(st.h, stop ? 0u : 1u);
+        }
+        __syncthreads();
+        if (s_stop)  // coefficients of the final combination
+            for (int i = threadIdx.x; i < j; i += blockDim.x)
+                lz->coef[i] = (float)(__ldcg(&lz->beta[0]) * __ldcg(&lz->y[i]) * __ldcg(&lz->binv[i]));
     }
 }
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_lz_update(int64_t N, V4<T> *basis, Rec<T> *rec, const V4<T> *u,
-                                                   double *partials, LzState *lz, const float *__restrict__ pc) {
+                                                   double *partials, LzState *lz, double *qlws,
+                                                   const float *__restrict__ pc, LzStop st) {
     __shared__ double sh[32];
-    lz_update_body<T>(N, basis, rec, u, partials, lz, pc, blockIdx.x, gridDim.x, sh);
+    __shared__ EigSmem esm;
+    lz_update_body<T>(N, basis, rec, u, partials, lz, qlws, pc, st, blockIdx.x, gridDim.x - 1, sh, &esm);
 }
 
-__global__ void __launch_bounds__(256) k_lz_update_batch(const LzSys *__restrict__ sys, const int *__restrict__ blk2sys) {
+// (five blocks per SM, as the lone form has)
+__global__ void __launch_bounds__(256, 5) k_lz_update_batch(const LzSys *__restrict__ sys, const int *__restrict__ blk2sys) {
     __shared__ double sh[32];
+    __shared__ EigSmem esm;
     const LzSys &S = sys[blk2sys[blockIdx.x]];
-    lz_update_body<float>(S.N, S.basis, S.rec, S.u, S.part_up, S.lz, S.pc, blockIdx.x - S.blk_up, S.nblk_up, sh);
-}
-
-// ------------------------------------------------------------------ FP64 tridiagonal eigen-solve
-// One warp.  T_k (diag alpha_1..alpha_k, off-diag beta_1..beta_{k-1}) is
-// diagonalised by implicit QL sweeps with Wilkinson-type shifts (Golub & Van
-// Loan, Sec. 8.3); every lane runs the scalar recurrences redundantly and
-// applies each plane rotation to its own rows of the eigenvector matrix.
-// Then y = Q diag(sqrt(lambda)) Q^T e_1.
-__device__ __forceinline__ double warp_max_d(double v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
-    return v;
-}
-
-// T_k^{1/2} e_1 for a small SPD tridiagonal T_k (k <= KP, KP * KP <= 64) by
-// the coupled Newton-Schulz iteration for the matrix square root: with
-// A = T_k / c, where c = the Gershgorin bound >= lambda_max, Y_0 = A,
-// Z_0 = I and W_n = (3 I - Z_n Y_n) / 2, the iterates Y_{n+1} = Y_n W_n and
-// Z_{n+1} = W_n Z_n converge to A^{1/2} and A^{-1/2}; the residual
-// R_n = I - Z_n Y_n obeys R_{n+1} = (3 R_n^2 + R_n^3) / 4 and starts below
-// 1 - lambda_min / c < 1.  Only multiply-adds (no FP64 divisions or square
-// roots per step), the KP^2 entries spread over the warp's lanes; rows and
-// columns k..KP-1 are padded with the identity, which stays its own root.
-// Once max|R_n| < 1e-8 one more product gives Y to rounding (the next
-// residual is ~1e-16).  Writes y = c^{1/2} Y e_1 and returns true, or false
-// (y untouched) if the residual has not fallen below 1e-8 in 60 steps.
-template <int KP>
-__device__ bool tri_sqrt_e1_ns(int k, const double *alpha, const double *beta, double *y, double *sm) {
-    constexpr int NE = KP * KP, PER = (NE + 31) / 32;
-    double *Y = sm, *Z = sm + NE, *W = sm + 2 * NE;
-    const int lane = threadIdx.x;
-    double c = 0.0;
-    for (int i = lane; i < k; i += 32) {
-        const double r = alpha[i + 1] + (i > 0 ? fabs(beta[i]) : 0.0) + (i + 1 < k ? fabs(beta[i + 1]) : 0.0);
-        c = fmax(c, r);
-    }
-    c = warp_max_d(c);
-    if (!(c > 0.0)) return false;
-    const double ic = 1.0 / c;
-#pragma unroll
-    for (int u = 0; u < PER; ++u) {
-        const int q = lane + 32 * u;
-        if (q < NE) {
-            const int i = q / KP, j = q % KP;
-            double a = i == j ? 1.0 : 0.0;
-            if (i < k && j < k) {
-                if (i == j) a = alpha[i + 1] * ic;
-                else if (i - j == 1 || j - i == 1) a = beta[i > j ? i : j] * ic;
-                else a = 0.0;
-            }
-            Y[q] = a;
-            Z[q] = i == j ? 1.0 : 0.0;
-        }
-    }
-    __syncwarp();
-    for (int it = 0; it < 60; ++it) {
-        double res = 0.0;
-#pragma unroll
-        for (int u = 0; u < PER; ++u) {
-            const int q = lane + 32 * u;
-            if (q < NE) {
-                const int i = q / KP, j = q % KP;
-                double zy = 0.0;
-#pragma unroll
-                for (int l = 0; l < KP; ++l) zy = fma(Z[i * KP + l], Y[l * KP + j], zy);
-                const double r = (i == j ? 1.0 : 0.0) - zy;
-                res = fmax(res, fabs(r));
-                W[q] = 0.5 * ((i == j ? 3.0 : 0.0) - zy);
-            }
-        }
-        res = warp_max_d(res);
-        if (!(res < 1.0)) return false;  // diverging (not SPD) or NaN
-        __syncwarp();
-        const bool last = res < 1e-8;
-        double yn[PER], zn[PER];
-#pragma unroll
-        for (int u = 0; u < PER; ++u) {
-            const int q = lane + 32 * u;
-            yn[u] = zn[u] = 0.0;
-            if (q < NE) {
-                const int i = q / KP, j = q % KP;
-#pragma unroll
-                for (int l = 0; l < KP; ++l) {
-                    yn[u] = fma(Y[i * KP + l], W[l * KP + j], yn[u]);
-                    zn[u] = fma(W[i * KP + l], Z[l * KP + j], zn[u]);
-                }
-            }
-        }
-        __syncwarp();
-#pragma unroll
-        for (int u = 0; u < PER; ++u) {
-            const int q = lane + 32 * u;
-            if (q < NE) {
-                Y[q] = yn[u];
-                Z[q] = zn[u];
-            }
-        }
-        __syncwarp();
-        if (last) {
-            const double sc = sqrt(c);
-            for (int i = lane; i < k; i += 32) y[i] = sc * Y[i * KP];
-            __syncwarp();
-            return true;
-        }
-    }
-    return false;
-}
-
-__device__ __forceinline__ void lz_eig_body(LzState *lz, int max_iter, int fixed_iter, double tol,
-                                            cudaGraphConditionalHandle handle) {
-    __shared__ double Q[PSE_MAXIT][PSE_MAXIT + 1];
-    __shared__ double d[PSE_MAXIT + 1], e[PSE_MAXIT + 1], y[PSE_MAXIT + 1];
-    __shared__ double nsm[3 * 64];
-    const int lane = threadIdx.x;
-    if (!lz->active) return;  // this system has stopped (batched loop)
-    const int k = lz->iter - 1;  // T_k is complete: alpha_k from the matvec, beta_k from the update
-    // Every FP64 warp instruction costs many cycles of this GPU's FP64 pipe,
-    // active lanes or not, so T_1 and T_2 take closed forms: T_1^{1/2} e_1 =
-    // sqrt(alpha_1); for the SPD 2x2 T = [[a, b], [b, c]], T^{1/2} =
-    // (T + s I) / t with s = sqrt(det T), t = sqrt(tr T + 2 s) (Cayley-Hamilton),
-    // the same matrix the eigendecomposition gives, to rounding.
-    if (k <= 2) {
-        if (lane == 0) {
-            const double a = lz->alpha[1];
-            if (k == 1) {
-                y[0] = sqrt(fmax(a, 0.0));
-            } else {
-                const double c = lz->alpha[2], b = lz->beta[1];
-                const double sd = sqrt(fmax(fma(a, c, -b * b), 0.0)), t = sqrt(a + c + 2.0 * sd);
-                y[0] = (a + sd) / t;
-                y[1] = b / t;
-            }
-        }
-        __syncwarp();
-    } else if ((k <= 4 && tri_sqrt_e1_ns<4>(k, lz->alpha, lz->beta, y, nsm)) ||
-               (k > 4 && k <= 8 && tri_sqrt_e1_ns<8>(k, lz->alpha, lz->beta, y, nsm))) {
-        // T_3 .. T_8: multiply-add iteration (k_lz_eig's FP64 QL sweeps took
-        // ~20 and ~38 us for k = 3 and 4: divisions and square roots per rotation)
-    } else {
-        for (int i = lane; i < k; i += 32) {
-            d[i] = lz->alpha[i + 1];
-            e[i] = (i + 1 < k) ? lz->beta[i + 1] : 0.0;
-            for (int c = 0; c < k; ++c) Q[i][c] = (i == c) ? 1.0 : 0.0;
-        }
-        __syncwarp();
-        const double eps = 2.220446049250313e-16;
-        for (int l = 0; l < k; ++l) {
-            for (int sweep = 0; sweep < 60; ++sweep) {
-                int m = l;
-                for (; m < k - 1; ++m) {
-                    const double dd = fabs(d[m]) + fabs(d[m + 1]);
-                    if (fabs(e[m]) <= eps * dd) break;
-                }
-                if (m == l) break;
-                // shift from the leading 2x2 block (entries are O(mobility), far
-                // from overflow, so plain square roots replace hypot)
-                double g = (d[l + 1] - d[l]) / (2.0 * e[l]);
-                double r = sqrt(fma(g, g, 1.0));
-                g = d[m] - d[l] + e[l] / (g + (g >= 0 ? r : -r));
-                double s = 1.0, c = 1.0, p = 0.0;
-                int i = m - 1;
-                bool deflated = false;
-                for (; i >= l; --i) {
-                    const double f = s * e[i], b = c * e[i];
-                    r = sqrt(fma(f, f, g * g));
-                    __syncwarp();
-                    if (lane == 0) e[i + 1] = r;
-                    __syncwarp();
-                    if (r == 0.0) {
-                        if (lane == 0) { d[i + 1] -= p; e[m] = 0.0; }
-                        __syncwarp();
-                        deflated = true;
-                        break;
-                    }
-                    const double rinv = 1.0 / r;  // one division per rotation
-                    s = f * rinv;
-                    c = g * rinv;
-                    g = d[i + 1] - p;
-                    r = (d[i] - g) * s + 2.0 * c * b;
-                    p = s * r;
-                    __syncwarp();
-                    if (lane == 0) d[i + 1] = g + p;
-                    __syncwarp();
-                    g = c * r - b;
-                    for (int row = lane; row < k; row += 32) {
-                        const double qa = Q[row][i], qb = Q[row][i + 1];
-                        Q[row][i + 1] = s * qa + c * qb;
-                        Q[row][i] = c * qa - s * qb;
-                    }
-                    __syncwarp();
-                }
-                if (deflated && i >= l) continue;
-                __syncwarp();
-                if (lane == 0) { d[l] -= p; e[l] = g; e[m] = 0.0; }
-                __syncwarp();
-            }
-        }
-        __syncwarp();
-        // y = Q diag(sqrt(max(lambda, 0))) Q^T e_1, each square root taken once
-        for (int c = lane; c < k; c += 32) e[c] = sqrt(fmax(d[c], 0.0)) * Q[0][c];
-        __syncwarp();
-        for (int row = lane; row < k; row += 32) {
-            double acc = 0.0;
-            for (int c = 0; c < k; ++c) acc += Q[row][c] * e[c];
-            y[row] = acc;
-        }
-        __syncwarp();
-    }
-    double num = 0.0, den = 0.0;
-    for (int row = lane; row < k; row += 32) {
-        const double prev = (row < k - 1) ? lz->y[row] : 0.0;
-        num += (y[row] - prev) * (y[row] - prev);
-        den += y[row] * y[row];
-    }
-    num = warp_sum(num);
-    den = warp_sum(den);
-    const double rel = (k >= 2 && den > 0) ? sqrt(num / den) : 1.0;
-    bool stop;
-    int conv = 0;
-    if (fixed_iter > 0) {
-        stop = (k >= fixed_iter);
-        conv = stop;
-    } else {
-        // beta_k = 0: the Krylov space is invariant and T_k^{1/2} e_1 is exact
-        const bool breakdown = !(lz->beta[k] > 0.0);
-        conv = breakdown || (k >= 2 && rel < tol);
-        stop = conv || (k >= max_iter);
-    }
-    const double b0 = lz->beta[0];
-    __syncwarp();
-    for (int row = lane; row < k; row += 32) {
-        lz->y[row] = y[row];
-        lz->coef[row] = (float)(b0 * y[row] / lz->beta[row]);
-    }
-    if (lane == 0) {
-        lz->rel = rel;
-        if (stop) {
-            lz->J = k;
-            lz->converged = conv;
-        }
-        lz->cont = stop ? 0 : 1;
-        if (handle) cudaGraphSetConditional(handle, stop ? 0u : 1u);
-    }
-}
-
-__global__ void __launch_bounds__(32) k_lz_eig(LzState *lz, int max_iter, int fixed_iter, double tol,
-                                               cudaGraphConditionalHandle handle) {
-    lz_eig_body(lz, max_iter, fixed_iter, tol, handle);
-}
-
-// One warp per system of a batch.
-__global__ void __launch_bounds__(32) k_lz_eig_batch(const LzSys *__restrict__ sys) {
-    const LzSys &S = sys[blockIdx.x];
-    lz_eig_body(S.lz, S.max_iter, S.fixed_iter, S.tol, 0);
+    lz_update_body<float>(S.N, S.basis, S.rec, S.u, S.part_up, S.lz, S.qlws, S.pc, S.stop, blockIdx.x - S.blk_up,
+                          S.nblk_up, sh, &esm);
 }
 
 // One thread per system: the systems whose stop test passed in this loop
@@ -1337,13 +1338,12 @@ template <typename T> void launch_lz_matvec(int64_t N, Geom<T> g, const Dev<T> &
         default: mv_launch<T, 4, 4>(N, g, d, s); break;
     }
 }
-template <typename T> void launch_lz_update(int64_t N, int, const Dev<T> &d, cudaStream_t s) {
-    k_lz_update<T><<<pgrid(N, 256, up_blocks_per_sm<T>()), 256, 0, s>>>(N, d.basis, d.rec, d.u, d.partials + num_sms() * 16 + 32, d.lz,
-                                                    sizeof(T) == 4 ? d.pc_on : nullptr);
-}
-void launch_lz_eig(LzState *lz, int max_iter, int fixed_iter, double tol, cudaGraphConditionalHandle h,
-                   cudaStream_t s) {
-    k_lz_eig<<<1, 32, 0, s>>>(lz, max_iter, fixed_iter, tol, h);
+// one block more than the vector update needs: the T_j^{1/2} e_1 block
+template <typename T>
+void launch_lz_update(int64_t N, const LzStop &stop, const Dev<T> &d, cudaStream_t s) {
+    k_lz_update<T><<<pgrid(N, 256, up_blocks_per_sm<T>()) + 1, 256, 0, s>>>(
+        N, d.basis, d.rec, d.u, d.partials + num_sms() * 16 + 32, d.lz, d.qlws, sizeof(T) == 4 ? d.pc_on : nullptr,
+        stop);
 }
 void launch_batch_cond(LzState *const *lzs, int nsys, cudaGraphConditionalHandle h, cudaStream_t s, int *any_out) {
     k_batch_cond<<<1, 256, 0, s>>>(lzs, nsys, h, any_out);
@@ -1354,7 +1354,6 @@ void launch_lz_matvec_batch(const LzSys *sys, const int *blk2sys, int nblocks, c
 void launch_lz_update_batch(const LzSys *sys, const int *blk2sys, int nblocks, cudaStream_t s) {
     k_lz_update_batch<<<nblocks, 256, 0, s>>>(sys, blk2sys);
 }
-void launch_lz_eig_batch(const LzSys *sys, int nsys, cudaStream_t s) { k_lz_eig_batch<<<nsys, 32, 0, s>>>(sys); }
 void launch_batch_init(const BSys *sys, int *const *tab, const int *nblk, cudaStream_t s) {
     k_lz_init_batch<<<nblk[BK_INIT], 256, 0, s>>>(sys, tab[BK_INIT]);
 }
@@ -1403,7 +1402,7 @@ void launch_matvec_caller(int64_t N, const SampleArgs<T> *args, Geom<T> g, const
 #define PSE_INST(T)                                                                                          \
     template void launch_lz_init<T>(int64_t, const SampleArgs<T> *, int, const Dev<T> &, cudaStream_t);        \
     template void launch_lz_matvec<T>(int64_t, Geom<T>, const Dev<T> &, cudaStream_t);                       \
-    template void launch_lz_update<T>(int64_t, int, const Dev<T> &, cudaStream_t);                           \
+    template void launch_lz_update<T>(int64_t, const LzStop &, const Dev<T> &, cudaStream_t);                \
     template void launch_lz_final<T>(int64_t, const SampleArgs<T> *, const Dev<T> &, bool, cudaStream_t);    \
     template void launch_lz_final_forces<T>(int64_t, const SampleArgs<T> *, const Dev<T> &, cudaStream_t);   \
     template void launch_det_final<T>(int64_t, const SampleArgs<T> *, const Dev<T> &, cudaStream_t);         \

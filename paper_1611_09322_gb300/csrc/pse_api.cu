@@ -562,6 +562,7 @@ template <typename T> pse_status ensure(pse_ctx *c, int64_t N) {
     A(d.bd_force, sizeof(T) * 3 * N);
     A(d.bd_dx, sizeof(T) * 3 * N);
     A(d.partials, sizeof(double) * (2 * num_sms() * 16 + 64));
+    A(d.qlws, sizeof(double) * PSE_QL_WORK);
     A(c->stage_pos, sizeof(T) * 3 * N);
     A(c->stage_out, sizeof(T) * 3 * N);
     A(c->stage_pos2, sizeof(T) * 3 * N);
@@ -694,13 +695,16 @@ template <typename T> pse_status capture_pre(pse_ctx *c, int mode) {
     return wst;
 }
 
+static LzStop lz_stop(const pse_ctx *c, cudaGraphConditionalHandle h) {
+    return LzStop{c->max_iter, c->params.fixed_iter, c->params.lanczos_tol > 0 ? c->params.lanczos_tol : c->plan.tol,
+                  h};
+}
+
 template <typename T>
 void capture_body(pse_ctx *c, cudaStream_t sa, cudaGraphConditionalHandle h) {
     Dev<T> &d = dev<T>(c);
-    const double ltol = c->params.lanczos_tol > 0 ? c->params.lanczos_tol : c->plan.tol;
     launch_lz_matvec<T>(c->N, geom<T>(c), d, sa);
-    launch_lz_update<T>(c->N, c->max_iter, d, sa);
-    launch_lz_eig(d.lz, c->max_iter, c->params.fixed_iter, ltol, h, sa);
+    launch_lz_update<T>(c->N, lz_stop(c, h), d, sa);
 }
 
 template <typename T> void capture_post(pse_ctx *c, int mode) {
@@ -770,7 +774,6 @@ template <typename T> pse_status full_step(pse_ctx *c, cudaStream_t s, cudaGraph
     Dev<T> &d = dev<T>(c);
     const WaveGeom<T> &w = wgeom<T>(c);
     const int64_t M3 = (int64_t)w.M * w.M * w.M;
-    const double ltol = c->params.lanczos_tol > 0 ? c->params.lanczos_tol : c->plan.tol;
     CK(cudaMemsetAsync(d.grid, 0, sizeof(T) * 3 * M3, s));
     CK(run_spread<T>(c, c->spread, s, d.rec));
     CKF(cufftSetStream(c->fft_r2c, s));
@@ -790,8 +793,7 @@ template <typename T> pse_status full_step(pse_ctx *c, cudaStream_t s, cudaGraph
     Dev<T> da = d;
     da.mv_add = d.uwave;
     launch_lz_matvec<T>(N, geom<T>(c), da, s);
-    launch_lz_update<T>(N, c->max_iter, d, s);
-    launch_lz_eig(d.lz, c->max_iter, c->params.fixed_iter, ltol, h, s);
+    launch_lz_update<T>(N, lz_stop(c, h), d, s);
     return PSE_OK;
 }
 
@@ -846,7 +848,6 @@ template <typename T> pse_status build_graph(pse_ctx *c, int mode) {
 template <typename T> pse_status run_plain(pse_ctx *c, cudaStream_t s, int mode) {
     const int64_t N = c->N;
     Dev<T> &d = dev<T>(c);
-    const double ltol = c->params.lanczos_tol > 0 ? c->params.lanczos_tol : c->plan.tol;
     pre<T>(c, N, s);
     launch_nbr<T>(N, geom<T>(c), d, s);
     if (gm_bd(mode)) launch_repulsion<T>(N, geom<T>(c), d, s);
@@ -864,8 +865,7 @@ template <typename T> pse_status run_plain(pse_ctx *c, cudaStream_t s, int mode)
     real_setup<T>(c, N, s);
     for (int it = 0; it < c->max_iter + 2; ++it) {
         launch_lz_matvec<T>(N, geom<T>(c), d, s);
-        launch_lz_update<T>(N, c->max_iter, d, s);
-        launch_lz_eig(d.lz, c->max_iter, c->params.fixed_iter, ltol, 0, s);
+        launch_lz_update<T>(N, lz_stop(c, 0), d, s);
         int cont = 0;
         CK(cudaMemcpyAsync(&cont, &d.lz->cont, sizeof(int), cudaMemcpyDeviceToHost, s));
         CK(cudaStreamSynchronize(s));
@@ -1519,7 +1519,6 @@ pse_status pse_profile_stages(pse_ctx *c, int64_t N, const float *d_pos, uint64_
     a.c_noise = 1.0;
     CK(push_args(c, d.args, &a, sizeof(a), s));
     if (c->params.wave_noise == 1 && (st = ensure_r2c<float>(c)) != PSE_OK) return st;
-    const double ltol = c->params.lanczos_tol > 0 ? c->params.lanczos_tol : c->plan.tol;
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
@@ -1582,9 +1581,8 @@ pse_status pse_profile_stages(pse_ctx *c, int64_t N, const float *d_pos, uint64_
         return PSE_OK; });
     for (int it = 0; r == PSE_OK && it < c->max_iter + 2; ++it) {
         r = timed(PSE_STAGE_MATVEC, 1, [&] { launch_lz_matvec<float>(N, c->gf, d, s); return PSE_OK; });
-        if (r == PSE_OK) r = timed(PSE_STAGE_LANCZOS_UPDATE, 1, [&] { launch_lz_update<float>(N, c->max_iter, d, s); return PSE_OK; });
-        if (r == PSE_OK) r = timed(PSE_STAGE_EIGEN, 1, [&] {
-            launch_lz_eig(d.lz, c->max_iter, c->params.fixed_iter, ltol, 0, s);
+        if (r == PSE_OK) r = timed(PSE_STAGE_LANCZOS_UPDATE, 1, [&] {
+            launch_lz_update<float>(N, lz_stop(c, 0), d, s);
             return PSE_OK; });
         int cont = 0;
         if (r == PSE_OK && cudaMemcpy(&cont, &d.lz->cont, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) r = PSE_ECUDA;
@@ -1873,7 +1871,7 @@ pse_status pse_get_stats(pse_ctx *c, pse_stats *out) {
     const int64_t np = (int64_t)lz.n_pairs;
     out->lanczos_iters = lz.J;
     out->converged = lz.converged;
-    out->lanczos_rel_change = lz.rel;
+    out->lanczos_rel_change = lz.den > 0.0 ? sqrt(lz.num / lz.den) : 1.0;
     out->n_pairs = np;
     out->overflow = lz.overflow;
     out->matvec_shape = (c->plan.precision == PSE_FP64 ? c->gd.mv : c->gf.mv) + 1;
@@ -2139,10 +2137,8 @@ static pse_status batch_descriptors(pse_batch *b) {
         d.blk_up = (int)blk_up.size();
         d.nblk_up = blocks(256, cap_up);
         blk_mv.insert(blk_mv.end(), d.nblk_mv, k);
-        blk_up.insert(blk_up.end(), d.nblk_up, k);
-        d.max_iter = c->max_iter;
-        d.fixed_iter = c->params.fixed_iter;
-        d.tol = c->params.lanczos_tol > 0 ? c->params.lanczos_tol : c->plan.tol;
+        blk_up.insert(blk_up.end(), d.nblk_up + 1, k);  // and the T_j block
+        d.stop = lz_stop(c, 0);
         d.g = c->gf;
         d.rec = c->df.rec;
         d.count = c->df.nbr_count;
@@ -2152,6 +2148,7 @@ static pse_status batch_descriptors(pse_batch *b) {
         d.u = c->df.u;
         d.part_mv = c->df.partials;
         d.part_up = c->df.partials + num_sms() * 16 + 32;
+        d.qlws = c->df.qlws;
         d.lz = c->df.lz;
         d.pc = c->df.pc_on;
         d.basis = c->df.basis;
@@ -2274,7 +2271,6 @@ static void batch_step(pse_batch *b, cudaStream_t s, cudaGraphConditionalHandle 
     const int S = (int)b->sys.size();
     launch_lz_matvec_batch(b->d_sys, b->d_blk_mv, b->nblk_mv, s);
     launch_lz_update_batch(b->d_sys, b->d_blk_up, b->nblk_up, s);
-    launch_lz_eig_batch(b->d_sys, S, s);
     launch_batch_cond(b->d_lzs, S, h, s, any_out);
 }
 

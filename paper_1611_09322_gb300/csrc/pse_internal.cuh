@@ -158,21 +158,32 @@ struct SpreadTile {
 struct LzState {
     double alpha[PSE_MAXIT + 2];
     double beta[PSE_MAXIT + 2];     // beta[0] = ||z1||
+    double binv[PSE_MAXIT + 2];     // 1 / beta (0 where beta = 0)
     double y[PSE_MAXIT + 2];        // T_j^{1/2} e_1 of the last checked j
     float coef[PSE_MAXIT + 2];      // beta0 * y_i / beta_{i-1}, i = 1..J (float for the final pass)
-    float c_u, c_q, c_p;            // update coefficients of the current iteration
+    double c_u, c_q, c_p;           // update coefficients of the current iteration
+    double tmax;                    // largest row sum |T| so far: a bound of the spectrum of T_j
     int iter;                       // iteration the matvec/update kernels run next
-    int jeig;                       // T_j the eigen kernel processes next
+    int stop_y;                     // the T_j block's decision, joined by the update's last block
     int J;                          // accepted iteration count
     int converged;
     int cont;                       // loop continues (host-loop mode reads this)
-    int active;                     // matvec/update/eigen still run; changes only between loop bodies
-    double rel;                     // last ||y_j - y_{j-1}|| / ||y_j||
+    int active;                     // matvec/update still run; changes only between loop bodies
+    double num, den;                // last ||y_j - y_{j-1}||^2 and ||y_j||^2 (den = 0: no y_{j-1})
     unsigned int counter_mv, counter_up, counter_init;
     int overflow;                   // neighbour list capacity exceeded
     int pad_;
     unsigned long long n_pairs;     // directed pairs found by the neighbour search
 };
+
+// Stop rule of one Lanczos iteration; h != 0: the WHILE node it controls.
+struct LzStop {
+    int max_iter, fixed_iter;
+    double tol;
+    cudaGraphConditionalHandle h;
+};
+// FP64 workspace of the QL route of T_j^{1/2} e_1 (eigenvectors, diagonals)
+#define PSE_QL_WORK (PSE_MAXIT * (PSE_MAXIT + 1) + 2 * (PSE_MAXIT + 1))
 
 // Appendix A, cases 1 and 2 (FP64): 6 pi eta a M^(r) = F (I - rr) + G rr.
 // Used by the host table builder and by the FP64 device matvec.
@@ -367,6 +378,7 @@ template <typename T> struct Dev {
     T *bd_force;         // 3N, caller order: forces of a Brownian step
     T *bd_dx;            // 3N, caller order: displacement of a Brownian step
     double *partials;    // per-block partial sums
+    double *qlws;        // PSE_QL_WORK
     LzState *lz;
     V4<T> *table;        // PSE_TABLE_N: (F, G - F, dF, d(G-F)) / (6 pi a)
     V4<T> *table_c;      // PSE_TABLEC_N, same columns, on the two-segment knots
@@ -399,9 +411,7 @@ inline int nbr_k(int64_t N, int64_t cap) {
 template <typename T> void launch_lz_init(int64_t N, const SampleArgs<T> *args, int system, const Dev<T> &d,
                                           cudaStream_t s);
 template <typename T> void launch_lz_matvec(int64_t N, Geom<T> g, const Dev<T> &d, cudaStream_t s);
-template <typename T> void launch_lz_update(int64_t N, int max_iter, const Dev<T> &d, cudaStream_t s);
-void launch_lz_eig(LzState *lz, int max_iter, int fixed_iter, double tol, cudaGraphConditionalHandle h,
-                   cudaStream_t s);
+template <typename T> void launch_lz_update(int64_t N, const LzStop &stop, const Dev<T> &d, cudaStream_t s);
 // batch loop condition: active_k = cont_k for every system, continue while any is active
 void launch_batch_cond(LzState *const *lzs, int nsys, cudaGraphConditionalHandle h, cudaStream_t s,
                        int *any_out = nullptr);
@@ -413,9 +423,8 @@ struct LzSys {
     int64_t N;
     int K;                       // ELL capacity per particle
     int blk_mv, nblk_mv;         // first block and block count in the fused matvec
-    int blk_up, nblk_up;         // same in the fused update
-    int max_iter, fixed_iter;
-    double tol;
+    int blk_up, nblk_up;         // same in the fused update (plus one T_j block)
+    LzStop stop;
     Geom<float> g;
     Rec<float> *rec;
     const int *count;
@@ -424,6 +433,7 @@ struct LzSys {
     const V4<float> *table_c;    // compact table (staged in shared memory by the matvec)
     V4<float> *u;
     double *part_mv, *part_up;   // per-block partial sums of the matvec and the update
+    double *qlws;
     LzState *lz;
     const float *pc;
     V4<float> *basis;
@@ -465,7 +475,6 @@ void launch_batch_interp(const BSys *sys, int *const *tab, const int *nblk, int 
 void launch_batch_pc_infer(const BSys *sys, int *const *tab, const int *nblk, cudaStream_t s);
 void launch_lz_matvec_batch(const LzSys *sys, const int *blk2sys, int nblocks, cudaStream_t s);
 void launch_lz_update_batch(const LzSys *sys, const int *blk2sys, int nblocks, cudaStream_t s);
-void launch_lz_eig_batch(const LzSys *sys, int nsys, cudaStream_t s);
 template <typename T> void launch_lz_final(int64_t N, const SampleArgs<T> *args, const Dev<T> &d, bool with_wave,
                                            cudaStream_t s);
 // plain matvec of a caller vector (sorted gather -> M_r -> scatter back)
