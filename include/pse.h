@@ -92,8 +92,10 @@ typedef struct {
                             forces call if it does not fit shared memory)      */
     int matvec_shape;    /* 0 (default): near-field matvec with 2 threads x 4
                             gathers per particle in blocks of 1024 threads
-                            (FP32; 4 x 4 in blocks of 128 in FP64), or timed
-                            with autotune bit 2;
+                            (FP32), pair blocks evaluated once per sample and
+                            streamed by every product (FP64; reported as
+                            shape 1, whose list they follow), or timed with
+                            autotune bit 2;
                             1..10 force threads x gathers, block size: 4x4
                             128, 8x2 128, 16x1 128, 4x2 128, 4x4 1024, 4x4
                             512, 8x2 1024, 4x2 1024, 1x4 1024, 2x4 1024;

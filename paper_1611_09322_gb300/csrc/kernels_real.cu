@@ -16,6 +16,8 @@
 // reducing kernels run persistent grids (a fixed multiple of the SM count)
 // and their per-block partial sums are added in block order by the last
 // block to arrive, so results do not depend on scheduling.
+#include <type_traits>
+
 #include "pse_internal.cuh"
 
 namespace pse {
@@ -63,10 +65,10 @@ __device__ __forceinline__ void lz_init_body(int64_t N, const SampleArgs<T> *arg
                 sym3_apply(pc + s * 16, v.x, v.y, v.z, p.x, p.y, p.z);
                 p.w = T(0);
                 rec[s].q = p;
-            } else {
+            } else if (rec) {
                 rec[s].q = v;
             }
-        } else {
+        } else if (rec) {
             rec[s].q = v;
         }
         part += v.x * v.x + v.y * v.y + v.z * v.z;
@@ -99,7 +101,7 @@ __global__ void __launch_bounds__(256) k_lz_init(int64_t N, const SampleArgs<T> 
 __global__ void __launch_bounds__(256) k_lz_init_batch(const BSys *__restrict__ sys, const int *__restrict__ tab) {
     __shared__ double sh[32];
     const BSys &S = sys[tab[blockIdx.x]];
-    lz_init_body<float>(S.N, S.d.args, S.system, S.d.pos_sorted, S.d.basis, S.d.rec, S.d.partials, S.d.lz, S.d.pc_on,
+    lz_init_body<float>(S.N, S.d.args, S.system, S.d.pos_sorted, S.d.basis, rec_q(S.d), S.d.partials, S.d.lz, S.d.pc_on,
                         (int)blockIdx.x - S.b0[BK_INIT], S.nb[BK_INIT], sh);
 }
 
@@ -404,6 +406,192 @@ __global__ void __launch_bounds__(BS) k_lz_matvec(int64_t N, int K, Geom<T> g, c
         lz_matvec_body<T, TPP, ILP, false>(N, K, g, rec, count, nbr, table, u, partials, lz, pc, basis, add,
                                            blockIdx.x, gridDim.x, sh);
     }
+}
+
+// ------------------------------------------------------------------ stored pair blocks (FP64)
+// The block of a pair, F (I - rr) + G rr = F I + sign(g) w w^T with g = G - F
+// and w = |g|^{1/2} r^, is the same in every product of one sample, and in
+// FP64 its closed form (three exponentials, three complementary error
+// functions, a dozen divisions) costs far more than streaming it: k_pairs
+// evaluates it once per directed pair, one pair per thread at a time, and the
+// products read a 4-byte entry (neighbour, the sign of g in bit 31) and a
+// 32-byte record (w, F) in order and gather the neighbour's q.  N = 1000
+// (phi = 0.1, J = 4): four products of 125 us each -> k_pairs 39 us and four
+// of 9 us.  In FP32 the list form stays: a record costs 16 bytes more per pair
+// and product than it saves in table lookups (N = 1e6: products 78 -> 69 us,
+// but 143 us for k_pairs).
+// Layout: slices of 32 consecutive particles, column k of a slice = 32
+// entries (records) side by side, `cols` columns of room per slice.
+// Columns past `cols` (lists about twice as long as the mean) are not stored:
+// pair_far evaluates those pairs in each product.
+__device__ __forceinline__ void pair_scalars(const V4<double> &li, const V4<double> &lt, int e, const Geom<double> &g,
+                                             const V4<double> *table, double &F, double &GmF, double &hx, double &hy,
+                                             double &hz) {
+    const int ox = ((e >> 4) & 3) - 1, oy = ((e >> 2) & 3) - 1, oz = (e & 3) - 1;
+    const double dx = (li.x - lt.x) - (double(ox) * g.cs + double(ox) * g.cs_lo);
+    const double dy = (li.y - lt.y) - (double(oy) * g.cs + double(oy) * g.cs_lo);
+    const double dz = (li.z - lt.z) - (double(oz) * g.cs + double(oz) * g.cs_lo);
+    const double r2 = dx * dx + dy * dy + dz * dz;
+    const double rinv = r2 > 0.0 ? 1.0 / sqrt(r2) : 0.0;
+    pair_fg(r2 * rinv, g, table, F, GmF);
+    hx = dx * rinv;
+    hy = dy * rinv;
+    hz = dz * rinv;
+}
+
+// Stored entry (record) k of particle s.
+__device__ __forceinline__ uint32_t pair_at(uint32_t s, uint32_t k, uint32_t cols) {
+    return ((s >> 5) * cols + k) * 32u + (s & 31u);
+}
+
+// TPP lanes share a particle: a warp works on SP = 32 / TPP consecutive
+// particles, lanes of equal lane / SP on the same column; a block's share of
+// these row groups is contiguous and its warps take consecutive groups.
+template <int TPP> struct RowShare {
+    static constexpr int SP = 32 / TPP;
+    int p, c;  // this lane's particle of the group, column offset
+    int64_t i, end;
+    int step;
+    __device__ RowShare(int64_t N) : p((threadIdx.x & 31) % SP), c((threadIdx.x & 31) / SP) {
+        const int64_t groups = (N + SP - 1) / SP;
+        i = blockIdx.x * groups / gridDim.x + (threadIdx.x >> 5);
+        end = (blockIdx.x + 1) * groups / gridDim.x;
+        step = blockDim.x >> 5;
+    }
+};
+
+#define PSE_STORED_THREADS 256
+template <int TPP>
+__global__ void __launch_bounds__(PSE_STORED_THREADS) k_pairs(int64_t N, int cols, Geom<double> g,
+                                                              const V4<double> *__restrict__ loc,
+                                                              const int *__restrict__ count,
+                                                              const int *__restrict__ nbr,
+                                                              const V4<double> *__restrict__ table,
+                                                              V4<double> *__restrict__ pair, int *__restrict__ pent) {
+    for (RowShare<TPP> R(N); R.i < R.end; R.i += R.step) {
+        const int64_t s = R.i * R.SP + R.p;
+        if (s >= N) continue;
+        const int n = min(count[s], cols);
+        const V4<double> li = loc[s];
+        for (int k = R.c; k < n; k += TPP) {
+            const int e = nbr[(int64_t)k * N + s];
+            V4<double> r;
+            r.x = r.y = r.z = r.w = 0.0;
+            int t = (int)s;  // a removed entry: a zero block
+            if (e >= 0) {
+                double F, g2, hx, hy, hz;
+                pair_scalars(li, loc[e >> 6], e, g, table, F, g2, hx, hy, hz);
+                const double c = sqrt(fabs(g2));
+                r.x = c * hx; r.y = c * hy; r.z = c * hz; r.w = F;
+                t = (e >> 6) | (g2 < 0.0 ? (int)0x80000000 : 0);
+            }
+            const uint32_t at = pair_at((uint32_t)s, (uint32_t)k, (uint32_t)cols);
+            pair[at] = r;
+            pent[at] = t;
+        }
+    }
+}
+
+// One pair past the stored columns.
+__device__ __noinline__ V4<double> pair_far(int64_t s, int e, const Geom<double> *g,
+                                            const V4<double> *__restrict__ loc, const V4<double> *__restrict__ table,
+                                            V4<double> q) {
+    double F, g2, hx, hy, hz;
+    pair_scalars(loc[s], loc[e >> 6], e, *g, table, F, g2, hx, hy, hz);
+    const double dot = g2 * (hx * q.x + hy * q.y + hz * q.z);
+    V4<double> r;
+    r.x = F * q.x + dot * hx;
+    r.y = F * q.y + dot * hy;
+    r.z = F * q.z + dot * hz;
+    r.w = 0.0;
+    return r;
+}
+
+// u = M_r q (+ add) over this block's particles; returns this thread's share
+// of q.u.
+template <int TPP>
+__device__ __forceinline__ double stored_rows(int64_t N, int cols, const Geom<double> &g,
+                                              const V4<double> *__restrict__ q, const V4<double> *__restrict__ loc,
+                                              const int *__restrict__ count, const int *__restrict__ nbr,
+                                              const V4<double> *__restrict__ pair, const int *__restrict__ pent,
+                                              const V4<double> *__restrict__ table, V4<double> *__restrict__ u,
+                                              const V4<double> *__restrict__ add) {
+    double part = 0.0;
+    for (RowShare<TPP> R(N); R.i < R.end; R.i += R.step) {
+        const int64_t s = R.i * R.SP + R.p;
+        const bool active = s < N;
+        const int cnt = active ? count[s] : 0;
+        const int n = cnt < cols ? cnt : cols;
+        double ax = 0.0, ay = 0.0, az = 0.0;
+        const uint32_t b = pair_at((uint32_t)s, 0, (uint32_t)cols);
+#pragma unroll 2
+        for (int k = R.c; k < n; k += TPP) {
+            const int e = pent[b + 32u * k];
+            const V4<double> r = pair[b + 32u * k], qt = q[e & 0x7fffffff];
+            double dot = r.x * qt.x + r.y * qt.y + r.z * qt.z;
+            dot = e < 0 ? -dot : dot;
+            ax += r.w * qt.x + dot * r.x;
+            ay += r.w * qt.y + dot * r.y;
+            az += r.w * qt.z + dot * r.z;
+        }
+        for (int k = n + R.c; k < cnt; k += TPP) {
+            const int e = nbr[(int64_t)k * N + s];
+            if (e < 0) continue;
+            const V4<double> f = pair_far(s, e, &g, loc, table, q[e >> 6]);
+            ax += f.x;
+            ay += f.y;
+            az += f.z;
+        }
+#pragma unroll
+        for (int o = R.SP; o < 32; o <<= 1) {
+            ax += __shfl_xor_sync(0xffffffffu, ax, o);
+            ay += __shfl_xor_sync(0xffffffffu, ay, o);
+            az += __shfl_xor_sync(0xffffffffu, az, o);
+        }
+        if (active && R.c == 0) {
+            const V4<double> qs = q[s];
+            V4<double> o;
+            o.x = ax + g.self_m * qs.x;
+            o.y = ay + g.self_m * qs.y;
+            o.z = az + g.self_m * qs.z;
+            o.w = 0.0;
+            if (add) {  // full-mobility Lanczos: the wave product M_w q_j of the same vector
+                const V4<double> aw = add[s];
+                o.x += aw.x;
+                o.y += aw.y;
+                o.z += aw.z;
+            }
+            u[s] = o;
+            part += qs.x * o.x + qs.y * o.y + qs.z * o.z;
+        }
+    }
+    return part;
+}
+
+template <int TPP>
+__global__ void __launch_bounds__(PSE_STORED_THREADS) k_lz_matvec_stored(
+    int64_t N, int cols, const __grid_constant__ Geom<double> g, const V4<double> *__restrict__ basis,
+    const V4<double> *__restrict__ loc, const int *__restrict__ count, const int *__restrict__ nbr,
+    const V4<double> *__restrict__ pair, const int *__restrict__ pent, const V4<double> *__restrict__ table,
+    V4<double> *u, double *partials, LzState *lz, const V4<double> *__restrict__ add) {
+    __shared__ double sh[32];
+    const int j = lz->iter;
+    if (j > PSE_MAXIT || !lz->active) return;  // uniform across the launch
+    const double part = stored_rows<TPP>(N, cols, g, basis + (int64_t)(j - 1) * N, loc, count, nbr, pair, pent, table,
+                                         u, add);
+    const double bsum = block_sum(part, sh);
+    double total;
+    if (grid_sum_last(bsum, partials, &lz->counter_mv, sh, &total) && threadIdx.x == 0) lz_alpha(lz, j, total);
+}
+
+// M_r v of a sorted vector (forces path).
+template <int TPP>
+__global__ void __launch_bounds__(PSE_STORED_THREADS) k_matvec_stored(
+    int64_t N, int cols, const __grid_constant__ Geom<double> g, const V4<double> *__restrict__ v,
+    const V4<double> *__restrict__ loc, const int *__restrict__ count, const int *__restrict__ nbr,
+    const V4<double> *__restrict__ pair, const int *__restrict__ pent, const V4<double> *__restrict__ table,
+    V4<double> *out) {
+    stored_rows<TPP>(N, cols, g, v, loc, count, nbr, pair, pent, table, out, nullptr);
 }
 
 // ------------------------------------------------------------------ brick-tiled matvec
@@ -871,10 +1059,10 @@ __device__ __forceinline__ void lz_update_body(int64_t N, V4<T> *basis, Rec<T> *
                     sym3_apply(pc + s * 16, w.x, w.y, w.z, p.x, p.y, p.z);
                     p.w = T(0);
                     rec[s].q = p;
-                } else {
+                } else if (rec) {
                     rec[s].q = w;
                 }
-            } else {
+            } else if (rec) {
                 rec[s].q = w;
             }
             part += w.x * w.x + w.y * w.y + w.z * w.z;
@@ -1053,19 +1241,19 @@ __global__ void k_det_final(int64_t N, const SampleArgs<T> *args, const V4<T> *p
 // s closer than 2a (pair vectors from cell-local offsets, as in the matvec),
 // plus the external force, written in caller order.
 template <typename T>
-__global__ void k_repulsion(int64_t N, Geom<T> g, const SampleArgs<T> *args, const Rec<T> *__restrict__ rec,
+__global__ void k_repulsion(int64_t N, Geom<T> g, const SampleArgs<T> *args, const V4<T> *__restrict__ loc,
                             const int *__restrict__ count, const int *__restrict__ nbr,
                             const V4<T> *__restrict__ pos_sorted, T *F) {
     const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= N) return;
-    const V4<T> li = rec[s].l;
+    const V4<T> li = loc[s];
     const T two_a = T(2) * g.a, k = (T)args->k_rep;
     T fx = 0, fy = 0, fz = 0;
     const int cnt = count[s];
     for (int q = 0; q < cnt; ++q) {
         const int e = nbr[(int64_t)q * N + s];
         if (e < 0) continue;  // a pair removed by the float64 decision at r_cut
-        const V4<T> lt = rec[e >> 6].l;
+        const V4<T> lt = loc[e >> 6];
         const int ox = ((e >> 4) & 3) - 1, oy = ((e >> 2) & 3) - 1, oz = (e & 3) - 1;
         const T dx = (li.x - lt.x) - (T(ox) * g.cs + T(ox) * g.cs_lo);
         const T dy = (li.y - lt.y) - (T(oy) * g.cs + T(oy) * g.cs_lo);
@@ -1102,13 +1290,14 @@ template <typename T> __global__ void k_advance(int64_t N, Geom<T> g, const Samp
 
 // ------------------------------------------------------------------ caller-vector matvec
 template <typename T>
-__global__ void k_gather_vec(int64_t N, const SampleArgs<T> *args, const V4<T> *pos_sorted, Rec<T> *rec) {
+__global__ void k_gather_vec(int64_t N, const SampleArgs<T> *args, const V4<T> *pos_sorted, Rec<T> *rec, V4<T> *vec) {
     const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (s >= N) return;
     const int64_t o = 3 * w_bits_r(pos_sorted[s].w);
     V4<T> v;
     v.x = args->vin[o]; v.y = args->vin[o + 1]; v.z = args->vin[o + 2]; v.w = T(0);
-    rec[s].q = v;
+    if (vec) vec[s] = v;
+    else rec[s].q = v;
 }
 
 template <typename T, int TPP, bool POLY = false>
@@ -1164,7 +1353,7 @@ static constexpr int kMvTpp = 4;
 
 template <typename T>
 void launch_lz_init(int64_t N, const SampleArgs<T> *args, int system, const Dev<T> &d, cudaStream_t s) {
-    k_lz_init<T><<<pgrid(N, 256, 8), 256, 0, s>>>(N, args, system, d.pos_sorted, d.basis, d.rec, d.partials, d.lz,
+    k_lz_init<T><<<pgrid(N, 256, 8), 256, 0, s>>>(N, args, system, d.pos_sorted, d.basis, rec_q(d), d.partials, d.lz,
                                                   sizeof(T) == 4 ? d.pc_on : nullptr);
 }
 // Matvec launch shapes (threads per particle, independent gathers per thread),
@@ -1288,12 +1477,14 @@ template <typename T> void mv_prepare_all() {
         mv_nolist_blocks_per_sm();
     }
 }
+static void stored_prepare();
 void matvec_prepare() {
     tile_prepare();
     mv_prepare_all<float>();
     mv_prepare_all<double>();
     up_blocks_per_sm<float>(); up_blocks_per_sm<double>();
     matvec_blocks_per_sm();
+    stored_prepare();
 }
 
 template <typename T, int TPP, int ILP, int BS = 128>
@@ -1302,7 +1493,55 @@ void mv_launch(int64_t N, Geom<T> g, const Dev<T> &d, cudaStream_t s) {
         N, nbr_k(N, d.nbr_cap), g, d.rec, d.nbr_count, d.nbr, d.table, d.table_c, d.u, d.partials, d.lz,
         sizeof(T) == 4 ? d.pc_on : nullptr, d.basis, d.mv_add);
 }
+// Stored pair blocks: threads per particle by N (few particles need more
+// threads each to fill the GPU and to shorten the chain of columns).
+template <typename F> static void with_stored_tpp(int64_t N, F &&f) {
+    using std::integral_constant;
+    if (N >= 60000) f(integral_constant<int, 2>{});
+    else if (N >= 15000) f(integral_constant<int, 4>{});
+    else f(integral_constant<int, 16>{});
+}
+// one wave of resident blocks (at most 8 per SM)
+template <int TPP> static int stored_per_sm() {
+    static int per_sm = 0;
+    if (per_sm == 0) {
+        int nb = 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, k_lz_matvec_stored<TPP>, PSE_STORED_THREADS, 0) !=
+                cudaSuccess ||
+            nb < 1) {
+            cudaGetLastError();
+            nb = 1;
+        }
+        per_sm = nb < 8 ? nb : 8;
+    }
+    return per_sm;
+}
+static void stored_prepare() {
+    stored_per_sm<2>();
+    stored_per_sm<4>();
+    stored_per_sm<16>();
+}
+template <typename T> void launch_pairs(int64_t N, Geom<T> g, const Dev<T> &d, cudaStream_t s) {
+    if constexpr (sizeof(T) == 8) {
+        if (!stored(d)) return;
+        with_stored_tpp(N, [&](auto tpp) {
+            k_pairs<tpp()><<<nb(N * tpp(), PSE_STORED_THREADS), PSE_STORED_THREADS, 0, s>>>(
+                N, d.pair_cols, g, d.loc_sorted, d.nbr_count, d.nbr, d.table, d.pair, d.pent);
+        });
+    }
+}
 template <typename T> void launch_lz_matvec(int64_t N, Geom<T> g, const Dev<T> &d, cudaStream_t s) {
+    if constexpr (sizeof(T) == 8) {
+        if (stored(d)) {
+            with_stored_tpp(N, [&](auto tpp) {
+                k_lz_matvec_stored<tpp()>
+                    <<<pgrid(N, PSE_STORED_THREADS / tpp(), stored_per_sm<tpp()>()), PSE_STORED_THREADS, 0, s>>>(
+                        N, d.pair_cols, g, d.basis, d.loc_sorted, d.nbr_count, d.nbr, d.pair, d.pent, d.table, d.u,
+                        d.partials, d.lz, d.mv_add);
+            });
+            return;
+        }
+    }
     if constexpr (sizeof(T) == 4) {
         if (g.mv == PSE_MV_TILED && g.nspec <= 1 && !d.pc_on && g_sm_smem) {
             const int cap = tile_cap(N, g.nc);
@@ -1342,7 +1581,7 @@ template <typename T> void launch_lz_matvec(int64_t N, Geom<T> g, const Dev<T> &
 template <typename T>
 void launch_lz_update(int64_t N, const LzStop &stop, const Dev<T> &d, cudaStream_t s) {
     k_lz_update<T><<<pgrid(N, 256, up_blocks_per_sm<T>()) + 1, 256, 0, s>>>(
-        N, d.basis, d.rec, d.u, d.partials + num_sms() * 16 + 32, d.lz, d.qlws, sizeof(T) == 4 ? d.pc_on : nullptr,
+        N, d.basis, rec_q(d), d.u, d.partials + num_sms() * 16 + 32, d.lz, d.qlws, sizeof(T) == 4 ? d.pc_on : nullptr,
         stop);
 }
 void launch_batch_cond(LzState *const *lzs, int nsys, cudaGraphConditionalHandle h, cudaStream_t s, int *any_out) {
@@ -1371,7 +1610,7 @@ void launch_lz_final_forces(int64_t N, const SampleArgs<T> *args, const Dev<T> &
                                              sizeof(T) == 4 ? d.pc_on : nullptr, d.udet);
 }
 template <typename T> void launch_repulsion(int64_t N, Geom<T> g, const Dev<T> &d, cudaStream_t s) {
-    k_repulsion<T><<<nb(N, 128), 128, 0, s>>>(N, g, d.args, d.rec, d.nbr_count, d.nbr, d.pos_sorted, d.bd_force);
+    k_repulsion<T><<<nb(N, 128), 128, 0, s>>>(N, g, d.args, d.loc_sorted, d.nbr_count, d.nbr, d.pos_sorted, d.bd_force);
 }
 template <typename T> void launch_advance(int64_t N, Geom<T> g, const Dev<T> &d, cudaStream_t s) {
     k_advance<T><<<nb(3 * N, 256), 256, 0, s>>>(N, g, d.args);
@@ -1379,16 +1618,27 @@ template <typename T> void launch_advance(int64_t N, Geom<T> g, const Dev<T> &d,
 template <typename T> void launch_det_final(int64_t N, const SampleArgs<T> *args, const Dev<T> &d, cudaStream_t s) {
     k_det_final<T><<<nb(N, 256), 256, 0, s>>>(N, args, d.pos_sorted, d.udet, d.uwave);
 }
+// the vector goes to the records, or to d.u for the stored pair blocks
 template <typename T> void launch_gather_vec(int64_t N, const SampleArgs<T> *args, const Dev<T> &d, cudaStream_t s) {
-    k_gather_vec<T><<<nb(N, 256), 256, 0, s>>>(N, args, d.pos_sorted, d.rec);
+    k_gather_vec<T><<<nb(N, 256), 256, 0, s>>>(N, args, d.pos_sorted, d.rec, stored(d) ? d.u : nullptr);
 }
 template <typename T> void launch_matvec_sorted(int64_t N, Geom<T> g, const Dev<T> &d, cudaStream_t s) {
+    if constexpr (sizeof(T) == 8) {
+        if (stored(d)) {
+            with_stored_tpp(N, [&](auto tpp) {
+                k_matvec_stored<tpp()>
+                    <<<pgrid(N, PSE_STORED_THREADS / tpp(), stored_per_sm<tpp()>()), PSE_STORED_THREADS, 0, s>>>(
+                        N, d.pair_cols, g, d.u, d.loc_sorted, d.nbr_count, d.nbr, d.pair, d.pent, d.table, d.udet);
+            });
+            return;
+        }
+    }
     k_matvec_sorted<T, kMvTpp><<<nb(N * kMvTpp, 128), 128, 0, s>>>(N, nbr_k(N, d.nbr_cap), g, d.rec, d.nbr_count,
                                                                     d.nbr, d.table, d.udet);
 }
 template <typename T>
 void launch_matvec_caller(int64_t N, const SampleArgs<T> *args, Geom<T> g, const Dev<T> &d, cudaStream_t s) {
-    k_gather_vec<T><<<nb(N, 256), 256, 0, s>>>(N, args, d.pos_sorted, d.rec);
+    k_gather_vec<T><<<nb(N, 256), 256, 0, s>>>(N, args, d.pos_sorted, d.rec, nullptr);
     if (g.nspec > 1)
         k_matvec_scatter<T, kMvTpp, true><<<nb(N * kMvTpp, 128), 128, 0, s>>>(N, nbr_k(N, d.nbr_cap), args, g, d.rec,
                                                                               d.nbr_count, d.nbr, d.table,
@@ -1402,6 +1652,7 @@ void launch_matvec_caller(int64_t N, const SampleArgs<T> *args, Geom<T> g, const
 #define PSE_INST(T)                                                                                          \
     template void launch_lz_init<T>(int64_t, const SampleArgs<T> *, int, const Dev<T> &, cudaStream_t);        \
     template void launch_lz_matvec<T>(int64_t, Geom<T>, const Dev<T> &, cudaStream_t);                       \
+    template void launch_pairs<T>(int64_t, Geom<T>, const Dev<T> &, cudaStream_t);                           \
     template void launch_lz_update<T>(int64_t, const LzStop &, const Dev<T> &, cudaStream_t);                \
     template void launch_lz_final<T>(int64_t, const SampleArgs<T> *, const Dev<T> &, bool, cudaStream_t);    \
     template void launch_lz_final_forces<T>(int64_t, const SampleArgs<T> *, const Dev<T> &, cudaStream_t);   \

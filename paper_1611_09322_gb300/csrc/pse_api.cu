@@ -569,6 +569,27 @@ template <typename T> pse_status ensure(pse_ctx *c, int64_t N) {
     A(c->stage_out2, sizeof(T) * 3 * N);
     c->host_used[0] = c->host_used[1] = false;
 #undef A
+    // stored pair blocks (FP64): 1.5 times the mean list and 24 more, so that
+    // only rare long lists (clusters) have pairs beyond.  Last, and only from a
+    // quarter of what is left: without them the products read the list, so
+    // they must not take the memory that something else cannot do without.
+    d.pair = nullptr;
+    d.pent = nullptr;
+    d.pair_cols = 0;
+    d.use_pair = sizeof(T) == 8 && c->params.matvec_shape == 0;
+    d.want_rec = false;
+    if (d.use_pair) {
+        const double mean = (double)N * 4.18879020478639 * p.r_cut * p.r_cut * p.r_cut / (p.L * p.L * p.L);
+        const int64_t K = nbr_k(N, cap), want = (int64_t)ceil(1.5 * mean) + 24;
+        d.pair_cols = (int)(want < K ? want : K);
+        const size_t slots = (size_t)((N + 31) / 32 * 32) * d.pair_cols;
+        size_t left = 0, all = 0;
+        CK(cudaMemGetInfo(&left, &all));
+        if (slots >= (1ull << 31) || (sizeof(V4<T>) + sizeof(int)) * slots > left / 4 ||
+            alloc(c->per_n, (void **)&d.pent, sizeof(int) * slots) != PSE_OK ||
+            alloc(c->per_n, (void **)&d.pair, sizeof(V4<T>) * slots) != PSE_OK)
+            d.pair = nullptr;
+    }
     c->N = N;
     return PSE_OK;
 }
@@ -686,6 +707,7 @@ template <typename T> pse_status capture_pre(pse_ctx *c, int mode) {
         cudaEventRecord(c->ev_init, c->s_init);
     }
     if (!gm_bd(mode) && !nolist_sample<T>(c, mode)) launch_nbr<T>(N, geom<T>(c), d, s);
+    launch_pairs<T>(N, geom<T>(c), d, s);
     if (mode != GM_SAMPLE) {  // M_r F into udet (the records are overwritten by q_1 next)
         launch_gather_vec<T>(N, d.args, d, s);
         launch_matvec_sorted<T>(N, geom<T>(c), d, s);
@@ -792,8 +814,9 @@ template <typename T> pse_status full_step(pse_ctx *c, cudaStream_t s, cudaGraph
     interp<T>(c, N, s);
     Dev<T> da = d;
     da.mv_add = d.uwave;
+    da.want_rec = true;  // the next step spreads q_{j+1} from the records
     launch_lz_matvec<T>(N, geom<T>(c), da, s);
-    launch_lz_update<T>(N, lz_stop(c, h), d, s);
+    launch_lz_update<T>(N, lz_stop(c, h), da, s);
     return PSE_OK;
 }
 
@@ -806,7 +829,10 @@ template <typename T> pse_status capture_full(pse_ctx *c) {
     cudaStream_t s = c->s_main;
     pre<T>(c, N, s);
     launch_nbr<T>(N, geom<T>(c), d, s);
-    launch_lz_init<T>(N, d.args, c->params.system, d, s);
+    launch_pairs<T>(N, geom<T>(c), d, s);
+    Dev<T> da = d;
+    da.want_rec = true;
+    launch_lz_init<T>(N, d.args, c->params.system, da, s);
     cudaGraph_t body = nullptr;
     pse_status st = PSE_OK;
     cudaError_t e = add_while(s, &c->cond[GM_FULL], &body);
@@ -851,6 +877,7 @@ template <typename T> pse_status run_plain(pse_ctx *c, cudaStream_t s, int mode)
     pre<T>(c, N, s);
     launch_nbr<T>(N, geom<T>(c), d, s);
     if (gm_bd(mode)) launch_repulsion<T>(N, geom<T>(c), d, s);
+    launch_pairs<T>(N, geom<T>(c), d, s);
     pse_status st = wave_branch<T>(c, N, s, mode);
     if (st != PSE_OK) return st;
     if (mode != GM_SAMPLE) {
@@ -884,7 +911,10 @@ template <typename T> pse_status run_full_plain(pse_ctx *c, cudaStream_t s) {
     Dev<T> &d = dev<T>(c);
     pre<T>(c, N, s);
     launch_nbr<T>(N, geom<T>(c), d, s);
-    launch_lz_init<T>(N, d.args, c->params.system, d, s);
+    launch_pairs<T>(N, geom<T>(c), d, s);
+    Dev<T> da = d;
+    da.want_rec = true;
+    launch_lz_init<T>(N, d.args, c->params.system, da, s);
     for (int it = 0; it < c->max_iter + 2; ++it) {
         const pse_status st = full_step<T>(c, s, 0);
         if (st != PSE_OK) return st;
@@ -913,6 +943,9 @@ template <typename T> pse_status tune_matvec(pse_ctx *c, cudaStream_t s) {
     float t[PSE_MV_VARIANTS];
     for (int v = 0; v < PSE_MV_VARIANTS; ++v) t[v] = 1e30f;
     Geom<T> g = geom<T>(c);
+    const bool had_pair = d.use_pair;
+    d.use_pair = false;  // the list shapes first
+    real_setup<T>(c, N, s);  // (q_1 into the records they read)
     for (int sweep = 0; sweep < 2; ++sweep)
         for (int v = 0; v < PSE_MV_VARIANTS; ++v) {
             g.mv = v;
@@ -929,6 +962,27 @@ template <typename T> pse_status tune_matvec(pse_ctx *c, cudaStream_t s) {
     int keep = 0;
     for (int v = 1; v < PSE_MV_VARIANTS; ++v)
         if (t[v] < t[keep]) keep = v;
+    // the stored pair blocks (the default) against the fastest list shape: 8
+    // products and two pair evaluations (one per four products)
+    d.use_pair = had_pair;
+    if (stored(d)) {
+        float best = 1e30f;
+        launch_pairs<T>(N, geom<T>(c), d, s);
+        for (int sweep = 0; sweep < 2; ++sweep) {
+            for (int rep = 0; rep < 10; ++rep) {
+                if (rep == 2) cudaEventRecord(e0, s);
+                if (rep == 2 || rep == 6) launch_pairs<T>(N, geom<T>(c), d, s);
+                launch_lz_matvec<T>(N, geom<T>(c), d, s);
+            }
+            cudaEventRecord(e1, s);
+            float ms = 0.f;
+            if (cudaEventSynchronize(e1) != cudaSuccess) continue;
+            cudaEventElapsedTime(&ms, e0, e1);
+            best = ms < best ? ms : best;
+        }
+        if (best >= t[keep]) d.use_pair = false;
+        else keep = geom<T>(c).mv;
+    }
     geom<T>(c).mv = keep;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);

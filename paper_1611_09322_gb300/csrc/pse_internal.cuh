@@ -370,6 +370,11 @@ template <typename T> struct Dev {
     float *pc;           // N x 16: preconditioner blocks S (0..5), S^{-1} (8..13), sorted order
     const float *pc_on;  // == pc while the learned preconditioner is active, else null
     float *pc_theta;     // network parameters (PSE_PRECOND_NPARAM)
+    V4<T> *pair;         // FP64: stored pair blocks (w, F), slices of 32 particles, pair_cols columns each; or null
+    int *pent;           // their entries: neighbour, bit 31 the sign of G - F
+    int pair_cols;
+    bool use_pair;       // the sample's products read them (launch_pairs filled them)
+    bool want_rec;       // q_j also goes to the records (full-mobility Lanczos spreads from there)
     V4<T> *u;            // matvec output
     const V4<T> *mv_add; // added to every Lanczos matvec row (the wave product of the
                          // full-mobility Lanczos), or null
@@ -387,6 +392,13 @@ template <typename T> struct Dev {
     V4<T> *grid4;        // M^3 node-major copy (x, y, z, 0) of grid for the interpolation (float)
     SampleArgs<T> *args;
 };
+
+// Whether the Lanczos products of a sample read stored pair blocks (FP64).
+template <typename T> PSE_HD inline bool stored(const Dev<T> &d) { return d.pair && d.use_pair; }
+// Where q_j is written besides the basis: the records the list products read.
+template <typename T> PSE_HD inline Rec<T> *rec_q(const Dev<T> &d) {
+    return stored(d) && !d.want_rec ? nullptr : d.rec;
+}
 
 // SM count of the current device (cached): persistent grids of the
 // reducing kernels are sized from it.
@@ -411,6 +423,7 @@ inline int nbr_k(int64_t N, int64_t cap) {
 template <typename T> void launch_lz_init(int64_t N, const SampleArgs<T> *args, int system, const Dev<T> &d,
                                           cudaStream_t s);
 template <typename T> void launch_lz_matvec(int64_t N, Geom<T> g, const Dev<T> &d, cudaStream_t s);
+template <typename T> void launch_pairs(int64_t N, Geom<T> g, const Dev<T> &d, cudaStream_t s);
 template <typename T> void launch_lz_update(int64_t N, const LzStop &stop, const Dev<T> &d, cudaStream_t s);
 // batch loop condition: active_k = cont_k for every system, continue while any is active
 void launch_batch_cond(LzState *const *lzs, int nsys, cudaGraphConditionalHandle h, cudaStream_t s,

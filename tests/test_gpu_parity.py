@@ -429,3 +429,29 @@ def test_pipelined_host_buffers(torch):
     s.host_sync()
     assert torch.equal(o2, s.sample(torch.from_numpy(pos[:1000].copy()).cuda(), SEED, 3).cpu())
     s.close()
+
+
+@pytest.mark.parametrize("N", [1, 5, 700, 15500])
+def test_fp64_stored_pair_blocks(torch, N):
+    """FP64 products over stored pair blocks (matvec_shape 0) against the list
+    form (shape 1): a dilute box with a clump whose lists run past the stored
+    columns, coincident pairs included, at the sizes of the two thread layouts.
+    The two evaluate the same blocks in another order of summation: 1e-12 is
+    over 1000 times the rounding of lists of a few hundred pairs."""
+    rng = np.random.default_rng(N)
+    L = 60.0
+    pos = rng.uniform(0, L, (N, 3))
+    m = min(N, 120)
+    pos[:m] = 30.0 + rng.uniform(-1.2, 1.2, (m, 3))
+    if N > 10:
+        pos[1] = pos[0]
+    d = torch.from_numpy(pos).cuda()
+    outs = []
+    for sh in (0, 1):
+        s = _sampler(L, xi=0.5, tol=1e-3, precision=1, fixed_iter=3, matvec_shape=sh)
+        _, r, _ = s.sample(d, SEED, 4, parts=True)
+        F = torch.from_numpy(np.random.default_rng(1).standard_normal((N, 3))).cuda()
+        outs.append((r.cpu().numpy(), s.mobility_apply(d, F).cpu().numpy(), s.sample_full_lanczos(d, SEED, 2).cpu().numpy()))
+        s.close()
+    for a, b in zip(*outs):
+        assert _rel(a, b) < 1e-12, _rel(a, b)
