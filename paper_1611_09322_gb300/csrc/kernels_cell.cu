@@ -249,6 +249,185 @@ __global__ void __launch_bounds__(256) k_nbr(int64_t N, Geom<T> g, const V4<T> *
     if ((threadIdx.x & 31) == 0 && tot) atomicAdd(n_pairs, (unsigned long long)tot);
 }
 
+// ------------------------------------------------------------------ search for few particles
+// Up to PSE_NBR_COOP particles one thread per particle leaves most of the GPU
+// idle and walks its 27 cells one after another, a chain of ~80 dependent
+// candidate loads.  Here Q lanes share a particle (27: one stencil cell each;
+// 9: one column of three cells in z): a lane tests its cells' particles and
+// keeps the accepted ones as bits; an exclusive sum over the particle's lanes
+// gives its first list slot, so the list is the one-thread walk's, entry by
+// entry.  Search (with the float64 decision) at N = 1000 35 -> 10 us, 4000
+// (phi = 0.2) 50 -> 14, 16000 48 -> 20, 16000 at tol 1e-5 (81 neighbours)
+// 102 -> 44, 30000 53 -> 30, a gel of 60000 53 -> 40; at 100000 (phi = 0.4)
+// 58 -> 74 and at 1e6 185 -> 331, where the lanes of a warp on different cells
+// cost the loads their broadcasts.  27 lanes below 10000 (10.2 against 12.1 us
+// at 1000, 13.9 against 16.3 at 4000; 22 against 20 at 16000).
+#define PSE_NBR_COOP 70000
+#define PSE_NBR_COOP27 10000
+template <typename T> struct NbrArgs {
+    int64_t N;
+    const V4<T> *loc, *pos;
+    const int *cell_start;
+    int *count, *nbr;
+    int K;
+    int *overflow;
+    unsigned long long *n_pairs;
+    int4 *edge;
+    int *edge_n;
+    int edge_cap;
+};
+
+// Range [b, e) and stencil code of the lane's cells, and the particle's
+// offset seen from them.
+template <typename T, int Q> struct NbrCells {
+    static constexpr int Z = 27 / Q;  // cells per lane
+    int b[Z], n[Z];
+    T px, py, pz[Z];
+    int code0;  // of the first cell; the next ones follow by 1 (z)
+};
+
+template <typename T>
+__device__ __forceinline__ bool nbr_hit(const V4<T> &lt, T px, T py, T pz, const Geom<T> &g, T &r2) {
+    const T dx = px - lt.x, dy = py - lt.y, dz = pz - lt.z;
+    r2 = dx * dx + dy * dy + dz * dz;
+    return r2 < g.rc2_hi;
+}
+
+// The second walk of a lane that met a pair in the band.
+template <typename T, int Q>
+__device__ __noinline__ void nbr_record_band_lane(int s, int slot, NbrCells<T, Q> C, const Geom<T> *g,
+                                             const NbrArgs<T> *a) {
+    for (int z = 0; z < C.Z; ++z)
+        for (int i = 0; i < C.n[z]; ++i) {
+            const int t = C.b[z] + i, code = C.code0 + z;
+            T r2;
+            if (!nbr_hit(a->loc[t], C.px, C.py, C.pz[z], *g, r2) || (t == s && code == 21)) continue;
+            if (r2 >= g->rc2_lo) {
+                const int k = atomicAdd(a->edge_n, 1);
+                if (k < a->edge_cap) a->edge[k] = make_int4(s, t, code, slot < a->K ? slot : -2);
+            }
+            ++slot;
+        }
+}
+
+// The lists of the warp's 32 / Q particles s0, s0 + 1, ...; returns the
+// warp's pair count (valid in every lane).
+template <typename T, int Q>
+__device__ __forceinline__ int nbr_warp(int64_t s0, const Geom<T> &g, const NbrArgs<T> &a) {
+    constexpr int R = 32 / Q, Z = 27 / Q;
+    const int lane = threadIdx.x & 31, grp = lane / Q, q = lane - grp * Q;
+    const int64_t s = s0 + grp;
+    const bool on = grp < R && s < a.N;
+    NbrCells<T, Q> C;
+    unsigned mask[Z];
+    int cnt = 0;
+    bool band = false;
+    if (on) {
+        const V4<T> li = a.loc[s], xi = a.pos[s];
+        // the binning's own arithmetic, cheaper than taking the cell id apart
+        const int cx = cell_coord(xi.x, g.inv_cs, g.nc), cy = cell_coord(xi.y, g.inv_cs, g.nc),
+                  cz = cell_coord(xi.z, g.inv_cs, g.nc);
+        const int col = Q == 27 ? q / 3 : q;
+        const int ox = col / 3 - 1, oy = col % 3 - 1, oz0 = Q == 27 ? q % 3 - 1 : -1;
+        int ax = cx + ox, ay = cy + oy;
+        ax += ax < 0 ? g.nc : 0;
+        ax -= ax >= g.nc ? g.nc : 0;
+        ay += ay < 0 ? g.nc : 0;
+        ay -= ay >= g.nc ? g.nc : 0;
+        C.px = li.x - (T(ox) * g.cs + T(ox) * g.cs_lo);
+        C.py = li.y - (T(oy) * g.cs + T(oy) * g.cs_lo);
+        C.code0 = ((ox + 1) << 4) | ((oy + 1) << 2) | (oz0 + 1);
+#pragma unroll
+        for (int z = 0; z < Z; ++z) {
+            int az = cz + oz0 + z;
+            az += az < 0 ? g.nc : 0;
+            az -= az >= g.nc ? g.nc : 0;
+            const int c2 = cell_id(ax, ay, az, g.nb);
+            C.b[z] = a.cell_start[c2];
+            C.n[z] = a.cell_start[c2 + 1] - C.b[z];
+            C.pz[z] = li.z - (T(oz0 + z) * g.cs + T(oz0 + z) * g.cs_lo);
+        }
+#pragma unroll
+        for (int z = 0; z < Z; ++z) {
+            const int self = C.code0 + z == 21 ? (int)s - C.b[z] : -1;  // the particle itself, in its own cell
+            const V4<T> *lz = a.loc + C.b[z];
+            unsigned m = 0, bit = 1;  // bits of the first 32 candidates
+#pragma unroll 2
+            for (int i = 0; i < C.n[z]; ++i) {
+                T r2;
+                if (nbr_hit(lz[i], C.px, C.py, C.pz[z], g, r2) && i != self) {
+                    m |= bit;
+                    ++cnt;
+                    if constexpr (sizeof(T) == 4) {
+                        if (r2 >= g.rc2_lo) band = true;
+                    }
+                }
+                bit <<= 1;
+            }
+            mask[z] = m;
+        }
+    }
+    // exclusive sums over the warp's lanes, less the particle's first
+    int inc = cnt;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += v;
+    }
+    const int first = __shfl_sync(0xffffffffu, inc - cnt, grp < R ? grp * Q : 0);
+    const int total = __shfl_sync(0xffffffffu, inc, grp < R ? grp * Q + Q - 1 : 0) - first;
+    if (on) {
+        int k = inc - cnt - first;
+        const int K = a.K;
+        if constexpr (sizeof(T) == 4) {
+            if (band) nbr_record_band_lane<T, Q>((int)s, k, C, &g, &a);
+        }
+#pragma unroll
+        for (int z = 0; z < Z; ++z) {
+            const int code = C.code0 + z;
+            for (unsigned m = mask[z]; m; m &= m - 1, ++k)
+                if (k < K) a.nbr[(int64_t)k * a.N + s] = ((C.b[z] + __ffs(m) - 1) << 6) | code;
+            for (int i = 32; i < C.n[z]; ++i) {  // a cell of more than 32 particles
+                const int t = C.b[z] + i;
+                T r2;
+                if (!nbr_hit(a.loc[t], C.px, C.py, C.pz[z], g, r2) || (code == 21 && t == s)) continue;
+                if (k < K) a.nbr[(int64_t)k * a.N + s] = (t << 6) | code;
+                ++k;
+            }
+        }
+        if (q == 0) {
+            if (total > K) atomicExch(a.overflow, 1);
+            a.count[s] = total < K ? total : K;
+        }
+    }
+    return __shfl_sync(0xffffffffu, inc, 31);
+}
+
+// A block's share of the particles is contiguous, its warps take consecutive
+// ones together.
+template <typename T, int Q>
+__device__ __forceinline__ void nbr_body(const Geom<T> &g, const NbrArgs<T> &a, int bidx, int nblk, int *sh) {
+    constexpr int R = 32 / Q;
+    if (threadIdx.x == 0) *sh = 0;
+    __syncthreads();
+    const int64_t groups = (a.N + R - 1) / R, end = (bidx + 1) * groups / nblk;
+    int tot = 0;
+    for (int64_t i = bidx * groups / nblk + (threadIdx.x >> 5); i < end; i += blockDim.x >> 5)
+        tot += nbr_warp<T, Q>(i * R, g, a);
+    // pair total for the statistics: one atomic per block
+    if ((threadIdx.x & 31) == 0 && tot) atomicAdd(sh, tot);
+    __syncthreads();
+    if (threadIdx.x == 0 && *sh) atomicAdd(a.n_pairs, (unsigned long long)*sh);
+}
+
+#define PSE_NBR_THREADS 256
+template <typename T, int Q>
+__global__ void __launch_bounds__(PSE_NBR_THREADS) k_nbr_coop(const __grid_constant__ Geom<T> g,
+                                                         const __grid_constant__ NbrArgs<T> a) {
+    __shared__ int sh;
+    nbr_body<T, Q>(g, a, blockIdx.x, gridDim.x, &sh);
+}
+
 // The float64 decision for the pairs k_nbr recorded within rounding of
 // r_cut (one block; a few per 10^5 particles).  Entry (s, t, code, slot):
 // slot >= 0 the float search stored the pair there, -2 it accepted it with a
@@ -356,7 +535,7 @@ __global__ void k_place_batch(const BSys *__restrict__ sys, const int *__restric
         place_elem<float>(k, S.d.args, S.g, S.d.cell_of, S.d.cell_start, S.d.perm, S.d.pos_sorted, S.d.loc_sorted,
                           S.d.rec);
 }
-__global__ void __launch_bounds__(256) k_nbr_batch(const BSys *__restrict__ sys, const int *__restrict__ tab) {
+__global__ void __launch_bounds__(256, 6) k_nbr_batch(const BSys *__restrict__ sys, const int *__restrict__ tab) {
     PSE_BATCH_SYS(BK_NBR);
     for (int64_t s0 = lb * (int64_t)blockDim.x; s0 < S.N; s0 += stride) {  // uniform per block
         const int64_t s = s0 + threadIdx.x;
@@ -491,8 +670,19 @@ void launch_place(int64_t N, const SampleArgs<T> *args, Geom<T> g, const Dev<T> 
                                             d.loc_sorted, d.rec);
 }
 
+template <typename T, int Q> static void nbr_coop(const Geom<T> &g, const NbrArgs<T> &a, cudaStream_t s) {
+    const int64_t groups = (a.N + 32 / Q - 1) / (32 / Q), warps = PSE_NBR_THREADS / 32;
+    const int64_t blocks = (groups + warps - 1) / warps, most = (int64_t)num_sms() * 32;
+    k_nbr_coop<T, Q><<<(unsigned)(blocks < most ? blocks : most), PSE_NBR_THREADS, 0, s>>>(g, a);
+}
 template <typename T> void launch_nbr(int64_t N, Geom<T> g, const Dev<T> &d, cudaStream_t s) {
-    k_nbr<T><<<nblk(N, 256), 256, 0, s>>>(N, g, d.loc_sorted, d.cell_start, d.nbr_count, d.nbr,
+    if (N < PSE_NBR_COOP) {
+        const NbrArgs<T> a{N, d.loc_sorted, d.pos_sorted, d.cell_start, d.nbr_count, d.nbr, nbr_k(N, d.nbr_cap),
+                           &d.lz->overflow, &d.lz->n_pairs, d.edge, d.edge_n, d.edge_cap};
+        if (N < PSE_NBR_COOP27) nbr_coop<T, 27>(g, a, s);
+        else nbr_coop<T, 9>(g, a, s);
+    } else
+        k_nbr<T><<<nblk(N, 256), 256, 0, s>>>(N, g, d.loc_sorted, d.cell_start, d.nbr_count, d.nbr,
                                           nbr_k(N, d.nbr_cap), &d.lz->overflow, &d.lz->n_pairs, d.edge, d.edge_n,
                                           d.edge_cap);
     if constexpr (sizeof(T) == 4)

@@ -455,3 +455,25 @@ def test_fp64_stored_pair_blocks(torch, N):
         s.close()
     for a, b in zip(*outs):
         assert _rel(a, b) < 1e-12, _rel(a, b)
+
+
+@pytest.mark.parametrize("N,L,kind", [(1, 20.0, "u"), (3, 20.0, "u"), (700, 14.0, "u"), (9999, 60.0, "clump"),
+                                      (10000, 60.0, "clump"), (10001, 45.0, "u"), (69999, 90.0, "u")])
+def test_neighbour_search_lane_groups(torch, N, L, kind):
+    """The searches with 27 and 9 lanes per particle, at the sizes where one
+    takes over from the other, in boxes of 2 and more cells per side and with
+    a clump that puts over 32 particles in one cell: the near-field product is
+    the oracle's over all pairs (1e-5, as test_real_matvec: FP32 sums of up
+    to a few hundred terms)."""
+    from oracle import ewald, pse
+    rng = np.random.default_rng(N)
+    pos = rng.uniform(0, L, (N, 3)).astype(np.float32)
+    if kind == "clump":
+        pos[:150] = (20.0 + rng.uniform(-1.5, 1.5, (150, 3))).astype(np.float32)
+    v = rng.standard_normal((N, 3)).astype(np.float32)
+    s = _sampler(L, xi=0.5, tol=1e-3)
+    got = s.real_matvec(torch.from_numpy(pos).cuda(), torch.from_numpy(v).cuda()).cpu().numpy()
+    s.close()
+    plan = ewald.plan(L, 1.0, 0.5, 1e-3)
+    ref = pse.RealOperator(pos.astype(np.float64), plan)(v.astype(np.float64))
+    assert _rel(got, ref) < 1e-5, _rel(got, ref)
