@@ -90,10 +90,10 @@ typedef struct {
                             autotune bit 1); 1, 2 or 4: tiles of that many
                             cells per side (PSE_ENOTSUPPORTED at the first
                             forces call if it does not fit shared memory)      */
-    int matvec_shape;    /* 0 (default): near-field matvec with 2 threads x 4
-                            gathers per particle in blocks of 1024 threads
-                            (FP32), pair blocks evaluated once per sample and
-                            streamed by every product (FP64; reported as
+    int matvec_shape;    /* 0 (default): a launch shape chosen by the number of
+                            particles and neighbours (FP32; pse_get_stats
+                            reports it), pair blocks evaluated once per sample
+                            and streamed by every product (FP64; reported as
                             shape 1, whose list they follow), or timed with
                             autotune bit 2;
                             1..10 force threads x gathers, block size: 4x4

@@ -208,6 +208,27 @@ template <typename T> void build_scale_table(const pse_plan_info &p, double a, s
     }
 }
 
+// Default matvec launch shape (index into the shapes of Geom::mv).  FP64: 4 x 4
+// in blocks of 128.  FP32 by particles and mean list length, us per product
+// with the launch's events (2 x 4 in blocks of 1024 in parentheses):
+//   N = 1e3: 8 x 2 in 128 11.1 (17.5); 4e3 at phi = 0.2 12.8 (20.9)
+//   N = 1.6e4: 4 x 4 in 512 13.1 (18.9), 81 neighbours 19.0 (34.9);
+//   3e4 15.9 (20.4); 6e4 18.2 (18.6)
+//   N = 1e5, 33 neighbours: 4 x 2 in 1024 28.5 (32.9); 1.25e5, 14
+//   neighbours 24.6 (23.8)
+//   N = 2e5, 35 neighbours: 47.3 (45.1); 4e5 45.7 (44.7); 1e6 92.5 (80.2)
+// Few particles want more threads each (a shorter chain of gathers, and no
+// second pass of a block for a few of them); many want 2 x 4 and one copy of
+// the shared-memory table per SM, which leaves more of it to the L1.
+template <typename T> int default_matvec_shape(const pse_plan_info &p, int64_t N) {
+    if (sizeof(T) == 8) return 0;
+    const double mean = (double)N * 4.18879020478639 * p.r_cut * p.r_cut * p.r_cut / (p.L * p.L * p.L);
+    if (N < 6000) return 1;
+    if (N < 70000) return 5;
+    if (N < 150000 && mean > 20) return 7;
+    return 9;
+}
+
 template <typename T> void fill_geom(pse_ctx *c) {
     const pse_plan_info &p = c->plan;
     Geom<T> g{};
@@ -227,11 +248,7 @@ template <typename T> void fill_geom(pse_ctx *c) {
     g.xi = (T)p.xi;
     g.nc = p.ncell;
     g.nb = bricks_per_side(p.ncell);
-    // default launch shape: FP32 2 threads x 4 gathers per particle in blocks
-    // of 1024 threads (one copy of the shared-memory table per SM leaves more
-    // of it to the L1: 81 us per matvec at N = 1e6 against 86 for 4 x 4 and 95
-    // for 4 x 4 in blocks of 128), FP64 4 x 4 in blocks of 128
-    g.mv = c->params.matvec_shape > 0 ? c->params.matvec_shape - 1 : (sizeof(T) == 4 ? 9 : 0);
+    g.mv = c->params.matvec_shape > 0 ? c->params.matvec_shape - 1 : default_matvec_shape<T>(p, 1 << 30);
     g.rc2_d = p.r_cut * p.r_cut;
     g.L_d = p.L;
     g.invL_d = 1.0 / p.L;
@@ -522,6 +539,7 @@ template <typename T> pse_status ensure(pse_ctx *c, int64_t N) {
     cudaDeviceSynchronize();
     drop_graph(c);
     free_list(c->per_n);
+    if (c->params.matvec_shape == 0 && !c->mv_tuned) geom<T>(c).mv = default_matvec_shape<T>(c->plan, N);
     c->N = 0;
     Dev<T> &d = dev<T>(c);
     const pse_plan_info &p = c->plan;
