@@ -76,7 +76,7 @@ __device__ __forceinline__ void lz_init_body(int64_t N, const SampleArgs<T> *arg
     const double bsum = block_total<T>(part, sh);
     double total;
     if (grid_sum_last(bsum, partials, &lz->counter_init, sh, &total, bidx, nblk) && threadIdx.x == 0) {
-        const double bi = total > 0.0 ? rsqrt(total) : 0.0;
+        const double bi = total > 0.0 ? rsqrt_f64(total) : 0.0;
         lz->beta[0] = total * bi;
         lz->binv[0] = bi;
         lz->tmax = 0.0;
@@ -108,14 +108,22 @@ __global__ void __launch_bounds__(256) k_lz_init_batch(const BSys *__restrict__ 
 // alpha_j = q_j.u / beta_{j-1}^2 and the coefficients of the update, by
 // multiplications with the stored 1/beta (an FP64 division costs about as much
 // as the rest of this tail).  beta_{j-1} = 0 (binv = 0): the Krylov space is
-// invariant and the loop has stopped.
-__device__ __forceinline__ void lz_alpha(LzState *lz, int j, double total) {
-    const double bi = lz->binv[j - 1];
-    const double alpha = total * bi * bi;
+// invariant and the loop has stopped.  What thread 0 of the last block will
+// need is fetched by thread 0 of every block before its rows.
+struct LzPrev {
+    double bi, cp;
+};
+__device__ __forceinline__ void lz_prev(const LzState *lz, int j, LzPrev *sp) {
+    if (threadIdx.x) return;
+    sp->bi = lz->binv[j - 1];
+    sp->cp = j >= 2 ? lz->beta[j - 1] * lz->binv[j - 2] : 0.0;
+}
+__device__ __forceinline__ void lz_alpha(LzState *lz, int j, double total, const LzPrev &sp) {
+    const double bi = sp.bi, cu = total * bi, alpha = cu * bi;
     lz->alpha[j] = alpha;
     lz->c_u = bi;
     lz->c_q = alpha * bi;
-    lz->c_p = j >= 2 ? lz->beta[j - 1] * lz->binv[j - 2] : 0.0;
+    lz->c_p = sp.cp;
 }
 
 // ------------------------------------------------------------------ near-field matvec
@@ -333,6 +341,8 @@ __device__ __forceinline__ void lz_matvec_body(int64_t N, int K, const Geom<T> &
                                                const V4<T> *__restrict__ pos_sorted = nullptr) {
     const int j = lz->iter;
     if (j > PSE_MAXIT || !lz->active) return;  // uniform across the system's blocks
+    __shared__ LzPrev prev;
+    lz_prev(lz, j, &prev);
     typename Part<T>::type part = 0;
     const int lane_g = threadIdx.x % TPP;
     const int64_t per_block = blockDim.x / TPP;
@@ -379,7 +389,7 @@ __device__ __forceinline__ void lz_matvec_body(int64_t N, int K, const Geom<T> &
     const double bsum = block_total<T>(part, sh);
     double total;
     if (grid_sum_last(bsum, partials, &lz->counter_mv, sh, &total, bidx, nblk) && threadIdx.x == 0) {
-        lz_alpha(lz, j, total);
+        lz_alpha(lz, j, total, prev);
     }
 }
 
@@ -577,11 +587,13 @@ __global__ void __launch_bounds__(PSE_STORED_THREADS) k_lz_matvec_stored(
     __shared__ double sh[32];
     const int j = lz->iter;
     if (j > PSE_MAXIT || !lz->active) return;  // uniform across the launch
+    __shared__ LzPrev prev;
+    lz_prev(lz, j, &prev);
     const double part = stored_rows<TPP>(N, cols, g, basis + (int64_t)(j - 1) * N, loc, count, nbr, pair, pent, table,
                                          u, add);
     const double bsum = block_sum(part, sh);
     double total;
-    if (grid_sum_last(bsum, partials, &lz->counter_mv, sh, &total) && threadIdx.x == 0) lz_alpha(lz, j, total);
+    if (grid_sum_last(bsum, partials, &lz->counter_mv, sh, &total) && threadIdx.x == 0) lz_alpha(lz, j, total, prev);
 }
 
 // M_r v of a sorted vector (forces path).
@@ -623,6 +635,8 @@ __global__ void __launch_bounds__(PSE_TILE_THREADS, 4) k_lz_matvec_tiled(
     for (int i = threadIdx.x; i < PSE_TABLEC_N; i += blockDim.x) tab_s[i] = table_c[i];
     const int j = lz->iter;
     if (j > PSE_MAXIT || !lz->active) return;  // uniform across the launch
+    __shared__ LzPrev prev;
+    lz_prev(lz, j, &prev);
     float part = 0.f;
     const int nb = g.nb, nc = g.nc;
     const int lane_g = threadIdx.x % TPP;
@@ -746,7 +760,7 @@ __global__ void __launch_bounds__(PSE_TILE_THREADS, 4) k_lz_matvec_tiled(
     const double bsum = block_sum_fw(part, sh);
     double total;
     if (grid_sum_last(bsum, partials, &lz->counter_mv, sh, &total) && threadIdx.x == 0) {
-        lz_alpha(lz, j, total);
+        lz_alpha(lz, j, total, prev);
     }
 }
 
@@ -809,9 +823,8 @@ __global__ void __launch_bounds__(PSE_BATCH_MV_THREADS) k_lz_matvec_batch(const 
 // the shift -2^-18 c: all phi_i > 0 there means that the spectrum lies above
 // it (Sylvester); otherwise (a zero mode of coincident spheres, or no
 // convergence) the QL route below is taken.
-// It was one launch of 12-19 us after each update (Newton-Schulz, QL); as a
-// block beside the update it takes 4 us, hidden behind the vectors.
-__constant__ double c_hht_s[32] = {
+// It was one launch of 12-19 us after each update (Newton-Schulz, QL).
+__device__ const double c_hht_s[32] = {
     5.7983172601720927e-8, 5.4321516364628967e-7, 1.6334814437543627e-6, 3.5979661192943067e-6,
     6.9216981084029469e-6, 1.2425309911265321e-5, 2.1467667841819654e-5, 3.6281423144883104e-5,
     6.0524386131848248e-5, 0.00010018300523163798, 0.00016505141758121806, 0.00027115231705414841,
@@ -820,7 +833,7 @@ __constant__ double c_hht_s[32] = {
     0.023112175112024554, 0.038077289224902505, 0.063027442481034705, 0.10514188625930458,
     0.17769500132631345, 0.30701023096143713, 0.55112158980091238, 1.0602371281842982,
     2.3353171719278134, 7.0224425253874365, 65.789729924363965, -3.814697265625e-6};
-__constant__ double c_hht_w[32] = {
+__device__ const double c_hht_w[32] = {
     0.00030813623989951382, 0.00032687093299644554, 0.00036547944964625105, 0.00042630934808390455,
     0.00051305944420673084, 0.00063100491451650686, 0.00078731848148126131, 0.0009915074693214191,
     0.0012559938481394102, 0.0015968736736132673, 0.0020349044825956523, 0.002596785671713454,
@@ -907,110 +920,138 @@ __device__ __noinline__ void tri_sqrt_e1_ql(int k, const double *alpha, const do
     __syncwarp();
 }
 
-// T_k^{1/2} e_1 into sm->y (one warp) by the rational sum, QL where the
-// spectrum is too wide for it.
-// phi_i (then the terms of y_i) of each lane's node lie in shared memory for
-// j <= 8 and in the global workspace above: the 19 KB that j = 64 needs would
-// change the SMs' split between L1 and shared memory, which costs the kernels
-// of the wave branch beside this one (64-system batch 0.5% slower).
+// phi_{i+1} (then its share of the sums) of each lane's node lie in shared
+// memory for j <= 8 and in the global workspace above: the 17 KB that j = 64
+// needs would change the SMs' split between L1 and shared memory, which costs
+// the kernels of the wave branch beside this one (64-system batch 0.5% slower).
 #define PSE_EIG_ROWS 8
 struct EigSmem {
     double ph[PSE_EIG_ROWS][33];
-    double a[PSE_MAXIT + 2], b[PSE_MAXIT + 2], y[PSE_MAXIT + 2];
+    double a[PSE_MAXIT + 2], b[PSE_MAXIT + 2], p[PSE_MAXIT + 2], y[PSE_MAXIT + 2];
 };
 static_assert(PSE_QL_WORK >= PSE_MAXIT * 33, "the rational sum's terms fit the QL workspace");
-__device__ __forceinline__ void tri_sqrt_e1(int k, double bound, EigSmem *sm, const double *alpha,
-                                            const double *beta, double *qlws) {
-    const int lane = threadIdx.x & 31;
-    for (int i = lane + 1; i <= k; i += 32) {
-        sm->a[i] = alpha[i];
-        sm->b[i] = i < k ? beta[i] : 0.0;
-    }
-    // c = 4^p >= bound: exponent of the bound rounded up to an even one
-    int ex = 0;
-    frexp(bound, &ex);
-    const int p = (ex + 1) >> 1;
-    const double c = ldexp(1.0, 2 * p);
-    const double s = c_hht_s[lane] * c;
-    __syncwarp();
-    double(*ph)[33] = k <= PSE_EIG_ROWS ? sm->ph : reinterpret_cast<double(*)[33]>(qlws);
-    double p1 = 1.0, p2 = 0.0;  // phi_{i+1}, phi_{i+2}
-    bool pos = bound > 0.0 && isfinite(bound);
-    for (int i = k; i >= 1; --i) {
-        ph[i - 1][lane] = p1;  // phi_{i+1}, the minor of x_i
-        const double bi = sm->b[i];
-        const double t = fma(sm->a[i] + s, p1, -bi * bi * p2);
-        p2 = p1;
-        p1 = t;
-        pos = pos && t > 0.0;
-    }
-    if (!__all_sync(0xffffffffu, pos)) {
-        tri_sqrt_e1_ql(k, alpha, beta, sm->y, qlws);
-        return;
-    }
-    double f = ldexp(c_hht_w[lane], p) / p1;  // w_l / phi_1, times the running beta product with its sign
-    {
-        const double x1 = f * ph[0][lane];
-        double v = sm->a[1] * x1;
-        if (k > 1) v -= sm->b[1] * sm->b[1] * f * ph[1][lane];
-        ph[0][lane] = v;
-    }
-    f *= -s;
-    for (int i = 2; i <= k; ++i) {
-        f *= -sm->b[i - 1];
-        ph[i - 1][lane] *= f;
-    }
-    __syncwarp();
-    // row sums, 32 / parts rows at a time, `parts` lanes per row
-    const int parts = k <= 8 ? 4 : (k <= 16 ? 2 : 1), span = 32 / parts;
-    for (int r0 = 0; r0 < k; r0 += span) {
-        const int row = r0 + lane / parts, part = lane % parts;
-        double v0 = 0.0, v1 = 0.0;
-        if (row < k)
-            for (int l = part * span; l < (part + 1) * span; l += 2) {
-                v0 += ph[row][l];
-                v1 += ph[row][l + 1];
-            }
-        v0 += v1;
-        for (int o = 1; o < parts; o <<= 1) v0 += __shfl_xor_sync(0xffffffffu, v0, o);
-        if (row < k && part == 0) sm->y[row] = v0;
-    }
-    __syncwarp();
-}
 
-// The T_j block of one update launch (its first warp): y_j, the stop test
-// without beta_j (||y_j - y_{j-1}||^2 < tol^2 ||y_j||^2), and the
-// coefficients of the final combination once it passes.
-__device__ __forceinline__ void lz_eig_body(LzState *lz, int k, const LzStop &st, EigSmem *sm, double *qlws) {
+// What the T_j warp reads, fetched at once and before j is known (one round
+// of loads instead of three): alpha_{l+1}, beta_{l+1}, y_l of lane l and its
+// node.
+struct EigIn {
+    double a, b, y, s, w, tmax;
+    __device__ __forceinline__ void fetch(const LzState *lz, int lane) {
+        a = lz->alpha[lane + 1];
+        b = lz->beta[lane + 1];
+        y = lz->y[lane];
+        s = __ldg(c_hht_s + lane);
+        w = __ldg(c_hht_w + lane);
+        tmax = lz->tmax;
+    }
+};
+
+// The T_j block of one update launch (its first warp): y_j = T_k^{1/2} e_1
+// (k = j) by the rational sum, QL where the spectrum is too wide for it, the
+// stop test without beta_j (||y_j - y_{j-1}||^2 < tol^2 ||y_j||^2), the state.
+// Every step of the chain is one dependent FP64 operation of ~70 cycles: the
+// recurrence takes one per row (its other term a step ahead), the reciprocal
+// of phi_1 three instead of a division's ~3500 cycles, the beta products run
+// beside it and scale the row sums at the end: 13000 -> 4500 cycles at k = 4.
+__device__ __forceinline__ void lz_eig_body(LzState *lz, int k, const LzStop &st, EigSmem *sm, double *qlws,
+                                            const EigIn &in) {
     const int lane = threadIdx.x & 31;
-    // rows 1..k of T_k: |T| row sums of rows < k already include their beta
-    const double bk1 = k > 1 ? lz->beta[k - 1] : 0.0, ak = lz->alpha[k];
-    double tmax = lz->tmax;
-    if (k > 1) tmax = fmax(tmax, lz->alpha[k - 1] + bk1 + (k > 2 ? lz->beta[k - 2] : 0.0));
-    tmax = fmax(tmax, ak + bk1);
-    tri_sqrt_e1(k, tmax, sm, lz->alpha, lz->beta, qlws);
-    double num = 0.0, den = 0.0;
-    for (int row = lane; row < k; row += 32) {
-        const double yr = sm->y[row], prev = row < k - 1 ? lz->y[row] : 0.0;
-        num += (yr - prev) * (yr - prev);
-        den += yr * yr;
+    sm->a[lane + 1] = in.a;
+    sm->b[lane + 1] = in.b;
+    for (int i = lane + 33; i <= k; i += 32) {
+        sm->a[i] = lz->alpha[i];
+        sm->b[i] = lz->beta[i];
     }
-    for (int o = k <= 8 ? 4 : 16; o > 0; o >>= 1) {
-        num += __shfl_xor_sync(0xffffffffu, num, o);
-        den += __shfl_xor_sync(0xffffffffu, den, o);
-    }
-    num = __shfl_sync(0xffffffffu, num, 0);
-    den = __shfl_sync(0xffffffffu, den, 0);
-    int conv, stop;
-    if (st.fixed_iter > 0) {
-        stop = conv = k >= st.fixed_iter;
-    } else {
-        conv = k >= 2 && den > 0.0 && num < st.tol * st.tol * den;
-        stop = conv || k >= st.max_iter;
-    }
+    if (lane == 0) sm->b[0] = 0.0;
     __syncwarp();
-    for (int row = lane; row < k; row += 32) lz->y[row] = sm->y[row];
+    // largest row sum of |T|: rows < k with their beta, row k without beta_k
+    double tmax = in.tmax;
+    {
+        const double b1 = sm->b[k - 1], b2 = k > 1 ? sm->b[k - 2] : 0.0;
+        if (k > 1) tmax = fmax(tmax, sm->a[k - 1] + b1 + b2);
+        tmax = fmax(tmax, sm->a[k] + b1);
+    }
+    // c = 4^p >= tmax
+    const int thi = __double2hiint(tmax), p = ((thi >> 20) - 1023 + 2) >> 1;
+    bool pos = thi > 0 && normal_f64(thi) && p > -400 && p < 400;
+    const double s = in.s * __hiloint2double((1023 + 2 * p) << 20, 0);
+    double(*ph)[33] = k <= PSE_EIG_ROWS ? sm->ph : reinterpret_cast<double(*)[33]>(qlws);
+    {
+        double p1 = 1.0, u = 0.0, as = sm->a[k] + s;  // phi_{i+1}, beta_i^2 phi_{i+2}, alpha_i + s
+        double bp = 1.0;                              // (-1)^{i+1} beta_1 .. beta_{i-1}
+        for (int i = k, r = 1; i >= 1; --i, ++r) {
+            ph[i - 1][lane] = p1;
+            const double b = sm->b[i - 1];
+            const double t = fma(as, p1, -u);
+            u = b * b * p1;
+            as = sm->a[i > 1 ? i - 1 : 1] + s;
+            p1 = t;
+            const int hi = __double2hiint(t);
+            pos = pos && hi > 0 && normal_f64(hi);
+            if (lane == 0) sm->p[r] = bp;
+            bp *= -sm->b[r];
+        }
+        if (__all_sync(0xffffffffu, pos)) {
+            const double f = in.w * __hiloint2double((1023 + p) << 20, 0) * rcp_f64(p1);  // w_l / phi_1
+            double v = sm->a[1] * ph[0][lane];
+            if (k > 1) v = fma(-sm->b[1] * sm->b[1], ph[1][lane], v);
+            ph[0][lane] = v * f;
+            const double g = -s * f;
+            for (int i = 1; i < k; ++i) ph[i][lane] *= g;
+            __syncwarp();
+        } else {
+            tri_sqrt_e1_ql(k, lz->alpha, lz->beta, sm->y, qlws);
+            pos = false;
+        }
+        pos = __all_sync(0xffffffffu, pos);
+    }
+    double num = 0.0, den = 0.0;
+    if (pos && k <= PSE_EIG_ROWS) {  // four lanes per row
+        const int row = lane >> 2, l0 = (lane & 3) * 8;
+        double y = 0.0;
+        if (row < k) {
+            const double *q = ph[row] + l0;
+            y = ((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7]));
+        }
+        y += __shfl_xor_sync(0xffffffffu, y, 1);
+        y += __shfl_xor_sync(0xffffffffu, y, 2);
+        const double prev = __shfl_sync(0xffffffffu, in.y, row);
+        if (row < k) {
+            y *= sm->p[row + 1];
+            const double d = row < k - 1 ? y - prev : y;
+            num = d * d;
+            den = y * y;
+            if ((lane & 3) == 0) lz->y[row] = y;
+        }
+#pragma unroll
+        for (int o = 4; o < 32; o <<= 1) {
+            num += __shfl_xor_sync(0xffffffffu, num, o);
+            den += __shfl_xor_sync(0xffffffffu, den, o);
+        }
+    } else {
+        for (int row = lane; row < k; row += 32) {
+            double y = sm->y[row];
+            if (pos) {
+                y = 0.0;
+                for (int l = 0; l < 32; ++l) y += ph[row][l];
+                y *= sm->p[row + 1];
+            }
+            const double d = row < k - 1 ? y - lz->y[row] : y;
+            num += d * d;
+            den += y * y;
+            lz->y[row] = y;
+        }
+        num = warp_sum(num);
+        den = warp_sum(den);
+    }
     if (lane == 0) {
+        int conv, stop;
+        if (st.fixed_iter > 0) {
+            stop = conv = k >= st.fixed_iter;
+        } else {
+            conv = k >= 2 && den > 0.0 && num < st.tol * st.tol * den;
+            stop = conv || k >= st.max_iter;
+        }
         lz->tmax = tmax;
         lz->num = num;
         lz->den = k >= 2 ? den : 0.0;
@@ -1025,13 +1066,14 @@ template <typename T>
 __device__ __forceinline__ void lz_update_body(int64_t N, V4<T> *basis, Rec<T> *rec, const V4<T> *u, double *partials,
                                                LzState *lz, double *qlws, const float *__restrict__ pc,
                                                const LzStop &st, int bidx, int nblk, double *sh, EigSmem *esm) {
+    EigIn in;
+    if (bidx == 0 && threadIdx.x < 32) in.fetch(lz, threadIdx.x);
     const int j = lz->iter;
     if (j > PSE_MAXIT || !lz->active) return;
     double bsum = 0.0;
     if (bidx == 0) {
-        if (threadIdx.x < 32) lz_eig_body(lz, j, st, esm, qlws);
-        __threadfence();
-        __syncthreads();
+        if (threadIdx.x < 32) lz_eig_body(lz, j, st, esm, qlws, in);
+        __syncthreads();  // its writes are the ticket's to release
     } else {
         const T cu = (T)lz->c_u, cq = (T)lz->c_q, cp = (T)lz->c_p;
         const V4<T> *qj = basis + (int64_t)(j - 1) * N;
@@ -1074,7 +1116,7 @@ __device__ __forceinline__ void lz_update_body(int64_t N, V4<T> *basis, Rec<T> *
         // every block is done: join beta_j with the T_j block's decision
         __shared__ int s_stop;
         if (threadIdx.x == 0) {
-            const double bi = total > 0.0 ? rsqrt(total) : 0.0;
+            const double bi = total > 0.0 ? rsqrt_f64(total) : 0.0;
             lz->beta[j] = total * bi;
             lz->binv[j] = bi;
             lz->iter = j + 1;
@@ -1094,8 +1136,9 @@ __device__ __forceinline__ void lz_update_body(int64_t N, V4<T> *basis, Rec<T> *
     }
 }
 
+// (five FP32 blocks per SM)
 template <typename T>
-__global__ void __launch_bounds__(256) k_lz_update(int64_t N, V4<T> *basis, Rec<T> *rec, const V4<T> *u,
+__global__ void __launch_bounds__(256, sizeof(T) == 4 ? 5 : 1) k_lz_update(int64_t N, V4<T> *basis, Rec<T> *rec, const V4<T> *u,
                                                    double *partials, LzState *lz, double *qlws,
                                                    const float *__restrict__ pc, LzStop st) {
     __shared__ double sh[32];
@@ -1103,7 +1146,6 @@ __global__ void __launch_bounds__(256) k_lz_update(int64_t N, V4<T> *basis, Rec<
     lz_update_body<T>(N, basis, rec, u, partials, lz, qlws, pc, st, blockIdx.x, gridDim.x - 1, sh, &esm);
 }
 
-// (five blocks per SM, as the lone form has)
 __global__ void __launch_bounds__(256, 5) k_lz_update_batch(const LzSys *__restrict__ sys, const int *__restrict__ blk2sys) {
     __shared__ double sh[32];
     __shared__ EigSmem esm;
@@ -1577,10 +1619,13 @@ template <typename T> void launch_lz_matvec(int64_t N, Geom<T> g, const Dev<T> &
         default: mv_launch<T, 4, 4>(N, g, d, s); break;
     }
 }
-// one block more than the vector update needs: the T_j^{1/2} e_1 block
+// the T_j^{1/2} e_1 block and the vector blocks, together one wave of resident
+// blocks at most (one block more than that trailed it by a block's time: 19.5
+// -> 22 us at N = 1e6)
 template <typename T>
 void launch_lz_update(int64_t N, const LzStop &stop, const Dev<T> &d, cudaStream_t s) {
-    k_lz_update<T><<<pgrid(N, 256, up_blocks_per_sm<T>()) + 1, 256, 0, s>>>(
+    const unsigned most = (unsigned)num_sms() * up_blocks_per_sm<T>(), vec = (unsigned)((N + 255) / 256);
+    k_lz_update<T><<<vec < most ? vec + 1 : most, 256, 0, s>>>(
         N, d.basis, rec_q(d), d.u, d.partials + num_sms() * 16 + 32, d.lz, d.qlws, sizeof(T) == 4 ? d.pc_on : nullptr,
         stop);
 }

@@ -282,43 +282,57 @@ __device__ __forceinline__ float warp_sum_f(float v) {
     return v;
 }
 
-// Block-wide sum of per-thread float partials: float inside each warp (the
-// operands are float products), double across warps and blocks.  Result
-// valid in all threads.
-__device__ __forceinline__ double block_sum_fw(float v, double *sh) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    v = warp_sum_f(v);
-    __syncthreads();
-    if (lane == 0) sh[wid] = (double)v;
-    __syncthreads();
-    double t = (threadIdx.x < nw) ? sh[threadIdx.x] : 0.0;
-    if (wid == 0) t = warp_sum(t);
-    if (threadIdx.x == 0) sh[0] = t;
-    __syncthreads();
-    const double r = sh[0];
-    __syncthreads();
-    return r;
+// 1/x and x^{-1/2} in FP64 for the scalar tails of the Lanczos kernels, where
+// one thread's chain of dependent FP64 operations is what is waited for: such
+// an operation takes ~70 cycles here and a compiled division ~3500.  Seed: the
+// FP32 approximation of the significand (relative error < 2^-22); one
+// third-order step, r (1 + e + e^2) with e = 1 - x r, or r (1 + e/2 + 3 e^2/8)
+// with e = 1 - x r^2 (the binomial series), leaves e^3 ~ 2^-66, so the result
+// is rounded to 1-2 ulp.  Zero, denormals, infinities and NaN take the
+// ordinary operations.
+__device__ __forceinline__ bool normal_f64(int hi) { return (unsigned)((hi & 0x7fffffff) - 0x00100000) < 0x7fe00000u; }
+__device__ __forceinline__ double rcp_f64(double x) {
+    const int hi = __double2hiint(x), E = ((hi >> 20) & 0x7ff) - 1023;
+    if (!normal_f64(hi) || E > 1000 || E < -1000) return 1.0 / x;
+    const double m = __hiloint2double(hi - E * 0x100000, __double2loint(x));  // +-[1, 2)
+    const double r = (double)__frcp_rn((float)m);
+    const double e = fma(-m, r, 1.0);
+    const double y = fma(r, fma(e, e, e), r);
+    return __hiloint2double(__double2hiint(y) - E * 0x100000, __double2loint(y));
+}
+__device__ __forceinline__ double rsqrt_f64(double x) {
+    const int hi = __double2hiint(x), E = (((hi >> 20) & 0x7ff) - 1023) & ~1;  // even: m in [1, 4)
+    if (hi < 0 || !normal_f64(hi)) return rsqrt(x);
+    const double m = __hiloint2double(hi - E * 0x100000, __double2loint(x));
+    const double r = (double)rsqrtf((float)m);
+    const double e = fma(-m * r, r, 1.0);
+    const double y = fma(r, e * fma(0.375, e, 0.5), r);
+    return __hiloint2double(__double2hiint(y) - (E >> 1) * 0x100000, __double2loint(y));
 }
 
-// Block-wide sum (blockDim.x a multiple of 32, <= 1024); result valid in all threads.
-__device__ __forceinline__ double block_sum(double v, double *sh) {
+// Block-wide sums, valid in thread 0 (blockDim.x = 32 times a power of two).
+// Per-thread float partials: float inside each warp (the operands are float
+// products), double across warps and blocks.
+__device__ __forceinline__ double block_sum_warps(double v, double *sh) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    v = warp_sum(v);
-    __syncthreads();
+    __syncthreads();  // an earlier sum's readers of sh are done
     if (lane == 0) sh[wid] = v;
     __syncthreads();
-    double t = (threadIdx.x < nw) ? sh[threadIdx.x] : 0.0;
-    if (wid == 0) t = warp_sum(t);
-    if (threadIdx.x == 0) sh[0] = t;
-    __syncthreads();
-    const double r = sh[0];
-    __syncthreads();
-    return r;
+    if (wid) return 0.0;
+    double t = lane < nw ? sh[lane] : 0.0;
+    for (int o = nw >> 1; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    return t;
 }
+__device__ __forceinline__ double block_sum_fw(float v, double *sh) {
+    return block_sum_warps((double)warp_sum_f(v), sh);
+}
+__device__ __forceinline__ double block_sum(double v, double *sh) { return block_sum_warps(warp_sum(v), sh); }
 
-// Deterministic grid-wide sum: every block stores its partial, the last block
-// to arrive (atomic ticket, no waiting) adds the partials in block order.
-// Returns true in the last block, with *total valid in all its threads.
+// Deterministic grid-wide sum: every block's thread 0 stores its partial, the
+// last block to arrive (atomic ticket, no waiting) adds the partials in a
+// fixed order.  Returns true in the last block, with *total valid in its
+// thread 0.  The ticket releases the block's earlier writes and acquires the
+// other blocks'.
 // bidx / nblk: this block's index among the nblk blocks reducing together
 // (the launch's grid, or one system's share of a fused multi-system launch).
 __device__ __forceinline__ bool grid_sum_last(double partial, double *partials, unsigned int *counter,
@@ -326,16 +340,22 @@ __device__ __forceinline__ bool grid_sum_last(double partial, double *partials, 
     __shared__ int s_last;
     if (threadIdx.x == 0) {
         partials[bidx] = partial;
-        __threadfence();
-        const unsigned int t = atomicAdd(counter, 1u);
+        unsigned int t;
+        asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(t) : "l"(counter) : "memory");
         s_last = (t == nblk - 1);
     }
     __syncthreads();
     if (!s_last) return false;
-    __threadfence();
     double acc = 0.0;
-    for (unsigned int b = threadIdx.x; b < nblk; b += blockDim.x) acc += __ldcg(partials + b);
-    *total = block_sum(acc, sh);
+    if (nblk <= 128) {  // one warp
+        if (threadIdx.x < 32) {
+            for (unsigned int b = threadIdx.x; b < nblk; b += 32) acc += __ldcg(partials + b);
+            *total = warp_sum(acc);
+        }
+    } else {
+        for (unsigned int b = threadIdx.x; b < nblk; b += blockDim.x) acc += __ldcg(partials + b);
+        *total = block_sum(acc, sh);
+    }
     if (threadIdx.x == 0) *counter = 0u;
     return true;
 }
