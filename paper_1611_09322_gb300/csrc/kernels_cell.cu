@@ -64,24 +64,12 @@ template <typename T> __device__ __forceinline__ long long w_bits(T w) {
     else return __double_as_longlong(w);
 }
 
-// Placement of counting-sort slot k: its particle i goes to position
-// b + rank in its cell [b, e), rank = the number of the cell's members with
-// a smaller caller index, so each cell is ordered by caller index whatever
-// the atomics did (one thread per particle, no serial per-cell sort).  The
-// position there gets the wrapped position (w = caller index bits), the
-// offsets from the cell corner (w = cell id, species in the high bits) and
-// the offsets half of the matvec record.
+// Particle i of cell c goes to sorted position dst: the wrapped position (w =
+// caller index bits), the offsets from the cell corner (w = cell id, species
+// in the high bits) and the offsets half of the matvec record.
 template <typename T>
-__device__ __forceinline__ void place_elem(int64_t k, const SampleArgs<T> *args, const Geom<T> &g,
-                                           const int *__restrict__ cell_of, const int *__restrict__ start,
-                                           const int *__restrict__ perm, V4<T> *pos_sorted, V4<T> *loc_sorted,
-                                           Rec<T> *rec) {
-    const int i = perm[k];
-    const int c = cell_of[i];
-    const int b = start[c], e = start[c + 1];
-    int rank = 0;
-    for (int t = b; t < e; ++t) rank += perm[t] < i;
-    const int64_t dst = b + rank;
+__device__ __forceinline__ void place_at(int i, int c, int64_t dst, const SampleArgs<T> *args, const Geom<T> &g,
+                                         V4<T> *pos_sorted, V4<T> *loc_sorted, Rec<T> *rec) {
     const T *p = args->pos + 3 * (int64_t)i;
     const T x = wrap_box(p[0], g.L), y = wrap_box(p[1], g.L), z = wrap_box(p[2], g.L);
     int cx, cy, cz;
@@ -109,12 +97,143 @@ __device__ __forceinline__ void place_elem(int64_t k, const SampleArgs<T> *args,
     rec[dst].l = l;
 }
 
+// Placement of counting-sort slot k: its particle i goes to position
+// b + rank in its cell [b, e), rank = the number of the cell's members with
+// a smaller caller index, so each cell is ordered by caller index whatever
+// the atomics did (one thread per particle, no serial per-cell sort).
+template <typename T>
+__device__ __forceinline__ void place_elem(int64_t k, const SampleArgs<T> *args, const Geom<T> &g,
+                                           const int *__restrict__ cell_of, const int *__restrict__ start,
+                                           const int *__restrict__ perm, V4<T> *pos_sorted, V4<T> *loc_sorted,
+                                           Rec<T> *rec) {
+    const int i = perm[k];
+    const int c = cell_of[i];
+    const int b = start[c], e = start[c + 1];
+    int rank = 0;
+    for (int t = b; t < e; ++t) rank += perm[t] < i;
+    place_at<T>(i, c, b + rank, args, g, pos_sorted, loc_sorted, rec);
+}
+
 template <typename T>
 __global__ void k_place(int64_t N, const SampleArgs<T> *args, Geom<T> g, const int *__restrict__ cell_of,
                         const int *__restrict__ start, const int *__restrict__ perm, V4<T> *pos_sorted,
                         V4<T> *loc_sorted, Rec<T> *rec) {
     const int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
     if (k < N) place_elem<T>(k, args, g, cell_of, start, perm, pos_sorted, loc_sorted, rec);
+}
+
+// ------------------------------------------------------------------ cell list of few particles
+// Binning, scan, scatter and placement in one launch: a cluster of 8 blocks
+// whose barrier takes the place of seven launches and four clears (each costs
+// a few microseconds of latency, more than its work here).  A thread keeps its
+// particles' cells and counting-sort slots in registers; after the scatter it
+// finds each particle's rank in its cell by caller index, as place_elem does.
+// Up to PSE_CELLS_FEW particles (one per thread) and PSE_CELLS_SLOTS cell
+// slots: sample of 1000 particles 115 -> 103 us, FP64 202 -> 194 (with the
+// search's float64 decisions in its last block).  With four particles per
+// thread the 8 SMs of the cluster take longer than the whole GPU's launches
+// (N = 30000: Brownian step 222 -> 240 us).
+#define PSE_CELLS_BLOCKS 8
+#define PSE_CELLS_THREADS 1024
+#define PSE_CELLS_PER 1     // particles per thread
+#define PSE_CELLS_SCAN 8    // cell slots per thread
+#define PSE_CELLS_FEW (PSE_CELLS_BLOCKS * PSE_CELLS_THREADS * PSE_CELLS_PER)
+#define PSE_CELLS_SLOTS (PSE_CELLS_BLOCKS * PSE_CELLS_THREADS * PSE_CELLS_SCAN)
+
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+
+// What other blocks of the cluster wrote is read through L2 (__ldcg).
+template <typename T>
+__global__ void __cluster_dims__(PSE_CELLS_BLOCKS, 1, 1) __launch_bounds__(PSE_CELLS_THREADS)
+    k_cells_few(int N, const SampleArgs<T> *args, const __grid_constant__ Geom<T> g, int nslots, int *count, int *start,
+                int *perm, int *sums, V4<T> *pos_sorted, V4<T> *loc_sorted, Rec<T> *rec, int *overflow,
+                unsigned long long *n_pairs) {
+    constexpr int ALL = PSE_CELLS_BLOCKS * PSE_CELLS_THREADS;
+    __shared__ int wsum[32];
+    const int blk = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    const int id = blk * PSE_CELLS_THREADS + threadIdx.x;
+    for (int c = id; c < nslots; c += ALL) count[c] = 0;
+    if (id == 0) {
+        *overflow = 0;
+        *n_pairs = 0ull;
+    }
+    int cell[PSE_CELLS_PER], slot[PSE_CELLS_PER];
+    const T *pos = args->pos;
+#pragma unroll
+    for (int u = 0; u < PSE_CELLS_PER; ++u) {
+        const int i = id + u * ALL;
+        cell[u] = 0;
+        if (i < N) {
+            const T x = wrap_box(pos[3 * i], g.L), y = wrap_box(pos[3 * i + 1], g.L), z = wrap_box(pos[3 * i + 2], g.L);
+            cell[u] = cell_id(cell_coord(x, g.inv_cs, g.nc), cell_coord(y, g.inv_cs, g.nc),
+                              cell_coord(z, g.inv_cs, g.nc), g.nb);
+        }
+    }
+    cluster_sync();
+#pragma unroll
+    for (int u = 0; u < PSE_CELLS_PER; ++u) slot[u] = id + u * ALL < N ? atomicAdd(count + cell[u], 1) : 0;
+    cluster_sync();
+    // exclusive scan: block `blk` has the slots [blk chunk, (blk + 1) chunk),
+    // a thread `per` consecutive ones
+    const int chunk = (nslots + PSE_CELLS_BLOCKS - 1) / PSE_CELLS_BLOCKS;
+    const int per = (chunk + PSE_CELLS_THREADS - 1) / PSE_CELLS_THREADS;  // at most PSE_CELLS_SCAN
+    const int c0 = blk * chunk + threadIdx.x * per, cend = min(nslots, (blk + 1) * chunk);
+    int v[PSE_CELLS_SCAN], tot = 0;
+#pragma unroll
+    for (int k = 0; k < PSE_CELLS_SCAN; ++k) {
+        v[k] = k < per && c0 + k < cend ? __ldcg(count + c0 + k) : 0;
+        tot += v[k];
+    }
+    int inc = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int n = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += n;
+    }
+    if (lane == 31) wsum[wid] = inc;
+    __syncthreads();
+    if (wid == 0) {
+        int w = wsum[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int n = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += n;
+        }
+        wsum[lane] = w;
+        if (lane == 31) sums[blk] = w;
+    }
+    cluster_sync();
+    int run = inc - tot + (wid ? wsum[wid - 1] : 0);
+    for (int b = 0; b < blk; ++b) run += __ldcg(sums + b);
+#pragma unroll
+    for (int k = 0; k < PSE_CELLS_SCAN; ++k) {
+        if (k < per && c0 + k < cend) start[c0 + k] = run;
+        run += v[k];
+    }
+    if (id == 0) start[nslots] = N;
+    cluster_sync();
+    int b[PSE_CELLS_PER];
+#pragma unroll
+    for (int u = 0; u < PSE_CELLS_PER; ++u) {
+        const int i = id + u * ALL;
+        b[u] = 0;
+        if (i < N) {
+            b[u] = __ldcg(start + cell[u]);
+            perm[b[u] + slot[u]] = i;
+        }
+    }
+    cluster_sync();
+#pragma unroll
+    for (int u = 0; u < PSE_CELLS_PER; ++u) {
+        const int i = id + u * ALL;
+        if (i >= N) continue;
+        const int c = cell[u], n = __ldcg(count + c);
+        int rank = 0;
+        for (int t = 0; t < n; ++t) rank += __ldcg(perm + b[u] + t) < i;
+        place_at<T>(i, c, b[u] + rank, args, g, pos_sorted, loc_sorted, rec);
+    }
 }
 
 // One thread per sorted particle, one pass: every neighbour within r_cut over
@@ -249,6 +368,39 @@ __global__ void __launch_bounds__(256) k_nbr(int64_t N, Geom<T> g, const V4<T> *
     if ((threadIdx.x & 31) == 0 && tot) atomicAdd(n_pairs, (unsigned long long)tot);
 }
 
+// The float64 decision for the pairs k_nbr recorded within rounding of
+// r_cut (one block; a few per 10^5 particles).  Entry (s, t, code, slot):
+// slot >= 0 the float search stored the pair there, -2 it accepted it with a
+// full list, -1 it rejected it.  Clears the edge count for the next search.
+__device__ __forceinline__ void nbr_edges_body(int64_t N, const Geom<float> &g, const V4<float> *__restrict__ pos,
+                                               int *count, int *nbr, int K, int *overflow,
+                                               unsigned long long *n_pairs, const int4 *edge, int *edge_n,
+                                               int edge_cap) {
+    const int n = min(__ldcg(edge_n), edge_cap);
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const int4 e = __ldcg(edge + i);
+        const int64_t s = e.x;
+        const bool in32 = e.w != -1, in64 = pair_inside_f64(pos[s], pos[e.y], g);
+        if (in32 && !in64) {
+            if (e.w >= 0) {
+                nbr[(int64_t)e.w * N + s] = -1;
+                atomicAdd(n_pairs, ~0ull);  // - 1
+            }
+        } else if (!in32 && in64) {
+            const int k = atomicAdd(count + s, 1);
+            if (k < K) {
+                nbr[(int64_t)k * N + s] = (e.y << 6) | e.z;
+                atomicAdd(n_pairs, 1ull);
+            } else {
+                atomicSub(count + s, 1);
+                atomicExch(overflow, 1);
+            }
+        }
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) *edge_n = 0;
+}
+
 // ------------------------------------------------------------------ search for few particles
 // Up to PSE_NBR_COOP particles one thread per particle leaves most of the GPU
 // idle and walks its 27 cells one after another, a chain of ~80 dependent
@@ -275,6 +427,7 @@ template <typename T> struct NbrArgs {
     int4 *edge;
     int *edge_n;
     int edge_cap;
+    unsigned int *ticket;  // the last block decides the edges
 };
 
 // Range [b, e) and stencil code of the lane's cells, and the particle's
@@ -426,39 +579,20 @@ __global__ void __launch_bounds__(PSE_NBR_THREADS) k_nbr_coop(const __grid_const
                                                          const __grid_constant__ NbrArgs<T> a) {
     __shared__ int sh;
     nbr_body<T, Q>(g, a, blockIdx.x, gridDim.x, &sh);
-}
-
-// The float64 decision for the pairs k_nbr recorded within rounding of
-// r_cut (one block; a few per 10^5 particles).  Entry (s, t, code, slot):
-// slot >= 0 the float search stored the pair there, -2 it accepted it with a
-// full list, -1 it rejected it.  Clears the edge count for the next search.
-__device__ __forceinline__ void nbr_edges_body(int64_t N, const Geom<float> &g, const V4<float> *__restrict__ pos,
-                                               int *count, int *nbr, int K, int *overflow,
-                                               unsigned long long *n_pairs, const int4 *edge, int *edge_n,
-                                               int edge_cap) {
-    const int n = min(*edge_n, edge_cap);
-    for (int i = threadIdx.x; i < n; i += blockDim.x) {
-        const int4 e = edge[i];
-        const int64_t s = e.x;
-        const bool in32 = e.w != -1, in64 = pair_inside_f64(pos[s], pos[e.y], g);
-        if (in32 && !in64) {
-            if (e.w >= 0) {
-                nbr[(int64_t)e.w * N + s] = -1;
-                atomicAdd(n_pairs, ~0ull);  // - 1
-            }
-        } else if (!in32 && in64) {
-            const int k = atomicAdd(count + s, 1);
-            if (k < K) {
-                nbr[(int64_t)k * N + s] = (e.y << 6) | e.z;
-                atomicAdd(n_pairs, 1ull);
-            } else {
-                atomicSub(count + s, 1);
-                atomicExch(overflow, 1);
-            }
+    if constexpr (sizeof(T) == 4) {
+        // the float64 decisions at r_cut by the last block to finish (no
+        // launch of their own: 3 us and its gap)
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            unsigned int t;
+            asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], 1;" : "=r"(t) : "l"(a.ticket) : "memory");
+            sh = t == gridDim.x - 1;
+            if (sh) *a.ticket = 0u;
         }
+        __syncthreads();
+        if (sh)
+            nbr_edges_body(a.N, g, a.pos, a.count, a.nbr, a.K, a.overflow, a.n_pairs, a.edge, a.edge_n, a.edge_cap);
     }
-    __syncthreads();
-    if (threadIdx.x == 0) *edge_n = 0;
 }
 
 __global__ void __launch_bounds__(256) k_nbr_edges(int64_t N, Geom<float> g, const V4<float> *__restrict__ pos,
@@ -675,14 +809,32 @@ template <typename T, int Q> static void nbr_coop(const Geom<T> &g, const NbrArg
     const int64_t blocks = (groups + warps - 1) / warps, most = (int64_t)num_sms() * 32;
     k_nbr_coop<T, Q><<<(unsigned)(blocks < most ? blocks : most), PSE_NBR_THREADS, 0, s>>>(g, a);
 }
+// The whole cell list, and the search's counters cleared.
+template <typename T>
+void launch_cells(int64_t N, const SampleArgs<T> *args, Geom<T> g, const Dev<T> &d, cudaStream_t s) {
+    const int64_t nc3 = cell_slots(g.nc);
+    if (N <= PSE_CELLS_FEW && nc3 <= PSE_CELLS_SLOTS) {
+        k_cells_few<T><<<PSE_CELLS_BLOCKS, PSE_CELLS_THREADS, 0, s>>>(
+            (int)N, args, g, (int)nc3, d.cell_count, d.cell_start, d.perm, d.scan_sums, d.pos_sorted, d.loc_sorted,
+            d.rec, &d.lz->overflow, &d.lz->n_pairs);
+        return;
+    }
+    launch_bin<T>(N, args, g, d, s);
+    launch_scatter<T>(N, args, g, d, s);
+    launch_place<T>(N, args, g, d, s);
+    cudaMemsetAsync(&d.lz->overflow, 0, sizeof(int), s);
+    cudaMemsetAsync(&d.lz->n_pairs, 0, sizeof(unsigned long long), s);
+}
+
 template <typename T> void launch_nbr(int64_t N, Geom<T> g, const Dev<T> &d, cudaStream_t s) {
     if (N < PSE_NBR_COOP) {
         const NbrArgs<T> a{N, d.loc_sorted, d.pos_sorted, d.cell_start, d.nbr_count, d.nbr, nbr_k(N, d.nbr_cap),
-                           &d.lz->overflow, &d.lz->n_pairs, d.edge, d.edge_n, d.edge_cap};
+                           &d.lz->overflow, &d.lz->n_pairs, d.edge, d.edge_n, d.edge_cap, &d.lz->counter_nbr};
         if (N < PSE_NBR_COOP27) nbr_coop<T, 27>(g, a, s);
         else nbr_coop<T, 9>(g, a, s);
-    } else
-        k_nbr<T><<<nblk(N, 256), 256, 0, s>>>(N, g, d.loc_sorted, d.cell_start, d.nbr_count, d.nbr,
+        return;
+    }
+    k_nbr<T><<<nblk(N, 256), 256, 0, s>>>(N, g, d.loc_sorted, d.cell_start, d.nbr_count, d.nbr,
                                           nbr_k(N, d.nbr_cap), &d.lz->overflow, &d.lz->n_pairs, d.edge, d.edge_n,
                                           d.edge_cap);
     if constexpr (sizeof(T) == 4)
@@ -694,6 +846,7 @@ template <typename T> void launch_nbr(int64_t N, Geom<T> g, const Dev<T> &d, cud
     template void launch_bin<T>(int64_t, const SampleArgs<T> *, Geom<T>, const Dev<T> &, cudaStream_t);     \
     template void launch_scatter<T>(int64_t, const SampleArgs<T> *, Geom<T>, const Dev<T> &, cudaStream_t); \
     template void launch_place<T>(int64_t, const SampleArgs<T> *, Geom<T>, const Dev<T> &, cudaStream_t);   \
+    template void launch_cells<T>(int64_t, const SampleArgs<T> *, Geom<T>, const Dev<T> &, cudaStream_t);   \
     template void launch_nbr<T>(int64_t, Geom<T>, const Dev<T> &, cudaStream_t);
 PSE_INST(float)
 PSE_INST(double)

@@ -615,11 +615,7 @@ template <typename T> pse_status ensure(pse_ctx *c, int64_t N) {
 // Kernels before the fork: bin, scan, scatter, per-cell sort, q_1 = z1.
 template <typename T> void pre(pse_ctx *c, int64_t N, cudaStream_t s) {
     Dev<T> &d = dev<T>(c);
-    launch_bin<T>(N, d.args, geom<T>(c), d, s);
-    launch_scatter<T>(N, d.args, geom<T>(c), d, s);
-    launch_place<T>(N, d.args, geom<T>(c), d, s);
-    cudaMemsetAsync(&d.lz->overflow, 0, sizeof(int), s);
-    cudaMemsetAsync(&d.lz->n_pairs, 0, sizeof(unsigned long long), s);
+    launch_cells<T>(N, d.args, geom<T>(c), d, s);
 }
 
 // After the neighbour list: preconditioner blocks (if installed), then q_1 = z1.

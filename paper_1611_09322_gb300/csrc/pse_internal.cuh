@@ -170,7 +170,7 @@ struct LzState {
     int cont;                       // loop continues (host-loop mode reads this)
     int active;                     // matvec/update still run; changes only between loop bodies
     double num, den;                // last ||y_j - y_{j-1}||^2 and ||y_j||^2 (den = 0: no y_{j-1})
-    unsigned int counter_mv, counter_up, counter_init;
+    unsigned int counter_mv, counter_up, counter_init, counter_nbr;
     int overflow;                   // neighbour list capacity exceeded
     int pad_;
     unsigned long long n_pairs;     // directed pairs found by the neighbour search
@@ -432,6 +432,7 @@ template <typename T> void launch_scatter(int64_t N, const SampleArgs<T> *args, 
                                           cudaStream_t s);
 template <typename T>
 void launch_place(int64_t N, const SampleArgs<T> *args, Geom<T> g, const Dev<T> &d, cudaStream_t s);
+template <typename T> void launch_cells(int64_t N, const SampleArgs<T> *args, Geom<T> g, const Dev<T> &d, cudaStream_t s);
 template <typename T> void launch_nbr(int64_t N, Geom<T> g, const Dev<T> &d, cudaStream_t s);
 
 inline int nbr_k(int64_t N, int64_t cap) {
