@@ -113,17 +113,15 @@ typedef struct {
                             support node, one warp per particle (P in 3..10);
                             1: reads the planar grids directly, 16 lanes per
                             particle                                           */
-    int wave_fft;        /* FP32 sample path with k-space noise: 0 (default)
-                            cuFFT C2R; 1: on grids M = 64 and 256, the noise
-                            and the inverse FFT as three kernels of this
-                            library (noise generated inside the first pass,
-                            the last pass writing the node-major grid of the
-                            interpolation; needs interp_form = 0), cuFFT on
-                            other grids.  Alone the three passes take about
-                            as long as noise + cuFFT + grid copy (417 vs 434 us
-                            at M = 256); beside the near-field kernels of a
-                            sample their shared memory costs those kernels
-                            L1, so the default is cuFFT                        */
+    int wave_fft;        /* FP32 with k-space noise and interp_form 0: 0
+                            (default) the transforms of the wave part are this
+                            library's (the noise drawn inside the first pass,
+                            the last one writing the node-major grid of the
+                            interpolation) on grids of 145 <= M < 490 that are
+                            no power of two, above M = 245 only where M^3 is
+                            at least 10 times the particles (30 above 375),
+                            and cuFFT's elsewhere: the faster ones of the two
+                            beside the near field.  1: also on M = 64 and 256 */
 } pse_params;
 
 /* Parameters derived from (L, a, xi, tol) by Sec. II C of the paper:
@@ -484,12 +482,15 @@ enum {
     PSE_STAGE_EIGEN,          /* 0: the FP64 T_j^{1/2} e_1 and the stop test are
                                  a block of the update's launch               */
     PSE_STAGE_FINAL,          /* x = V y, + wave part, caller order           */
-    PSE_STAGE_WAVE_NOISE,     /* k-space noise and B^{1/2} scaling (fused
-                                 path: with the first FFT pass)               */
-    PSE_STAGE_FFT,            /* cuFFT C2R, three components (fused path:
-                                 the second and third passes)                 */
+    PSE_STAGE_WAVE_NOISE,     /* k-space noise and B^{1/2} scaling (own
+                                 transforms: with their passes over x and y)  */
+    PSE_STAGE_FFT,            /* cuFFT C2R, three components (0 with the own
+                                 transforms; wave_fft = 1 on M = 64, 256:
+                                 their passes over y and z)                   */
     PSE_STAGE_INTERP,         /* Gaussian interpolation at the particles      */
-    PSE_STAGE_GRID_COPY,      /* node-major copy of the velocity grid (FP32)  */
+    PSE_STAGE_GRID_COPY,      /* node-major copy of the velocity grid (FP32;
+                                 own transforms: their pass over z, which
+                                 writes it)                                   */
     PSE_NSTAGES
 };
 

@@ -1,6 +1,6 @@
 // Wave-space sample M_w^{1/2} dW2 (Sec. II B 2): complex Hermitian noise,
-// B^{1/2} scaling with the Gaussian deconvolution, inverse FFT (cuFFT C2R,
-// launched by the host), and Gaussian interpolation S^dagger = h^3 S^T at the
+// B^{1/2} scaling with the Gaussian deconvolution, inverse FFT (three passes
+// of our own in FP32, else cuFFT C2R launched by the host), and Gaussian interpolation S^dagger = h^3 S^T at the
 // particles.  sm_103a.
 //
 // Per mode k = 2 pi n / L of the half spectrum (nz >= 0):
@@ -700,14 +700,14 @@ static void interp4(int64_t N, const WaveGeom<float> &w, const Dev<float> &d, cu
 }
 
 void launch_batch_noise(const BSys *sys, int *const *tab, const int *nblk, cudaStream_t s) {
-    k_wave_noise_batch<<<nblk[BK_NOISE], 256, 0, s>>>(sys, tab[BK_NOISE]);
+    if (nblk[BK_NOISE]) k_wave_noise_batch<<<nblk[BK_NOISE], 256, 0, s>>>(sys, tab[BK_NOISE]);
 }
 void launch_batch_interp(const BSys *sys, int *const *tab, const int *nblk, int P4, cudaStream_t s) {
     if (P4 == 0) {
         k_interp_batch<<<nblk[BK_INTERP], 128, 0, s>>>(sys, tab[BK_INTERP]);
         return;
     }
-    k_grid_aos_batch<<<nblk[BK_COPY], 256, 0, s>>>(sys, tab[BK_COPY]);
+    if (nblk[BK_COPY]) k_grid_aos_batch<<<nblk[BK_COPY], 256, 0, s>>>(sys, tab[BK_COPY]);
     switch (P4) {
         case 3: k_interp4_batch<3><<<nblk[BK_INTERP], 128, 0, s>>>(sys, tab[BK_INTERP]); break;
         case 4: k_interp4_batch<4><<<nblk[BK_INTERP], 128, 0, s>>>(sys, tab[BK_INTERP]); break;
@@ -804,277 +804,556 @@ cudaError_t launch_spread(WaveGeom<T> w, Geom<T> g, SpreadTile st, const int *or
     return cudaGetLastError();
 }
 
-// ------------------------------------------------------------------ fused k-space noise and inverse FFT
-// For grids M = R^2 (R = 8, 16: M = 64, 256; FP32, k-space noise): the
-// unnormalised C2R of the noise spectrum in three passes of our own, the
-// noise generated inside the first pass and the last pass writing the
-// node-major records the interpolation reads (no spectrum written by a noise
-// kernel, no planar grid, no copy).
-//   pass x: per (ky, tile of kz < M/2): noise of the modes, DFT over kx;
-//   pass y: per (ix, tile of kz): DFT over ky, in place in the spectrum buffer;
-//   pass z: per (ix, tile of iy): the real inverse DFT over kz, two real rows
-//           per complex transform (z = IDFT(Ya + i Yb): x_a = Re z, x_b = Im z,
-//           Y extended by Y_{M-k} = conj(Y_k), the Nyquist term Y_{M/2} = 0).
-// Each line of M = R^2 points is transformed by R threads in two register
-// passes (the four-step split n = t + R m, k = k1 + R k2):
-//   A_t[k1] = w_M^{t k1} sum_m x[t + R m] w_R^{m k1},
-//   X[k1 + R k2] = sum_t A_t[k1] w_R^{t k2},  w_L = e^{2 pi i / L},
-// with one padded shared-memory transpose between them.
-constexpr int PSE_FFT_TZ = 8;   // kz values per block in the x and y passes
-constexpr int PSE_FFT_TY = 8;   // iy rows per block in the z pass
+// ------------------------------------------------------------------ the sampler's own 3-D transforms
+// FP32 grids of 16 <= M <= 512 without prime factors above 7, with the
+// node-major interpolation (P = 3..10): the inverse transform of a sample in
+// three passes of our own, the noise drawn inside the first and the last one
+// writing the node-major records that the interpolation reads, and the forward
+// transform of the forces path with the mode factor between the two passes
+// over x.  The transforms are bound by memory traffic; against noise kernel +
+// cuFFT C2R + node-major copy they save the noise's write and read and the
+// planar grids' (noise, x, y / z: M = 200 157 -> 139 / 138 -> 110 us, 189 158
+// -> 115 / 135 -> 92, 378 973 -> 1000 / 795 -> 511; fft_wins has the rule).
+//   x pass: tile of (y, kz) modes, three components: noise (or forward
+//           transform over x, mode factor, noise), inverse over x;
+//   y pass: per x, tile of kz, one component, in place;
+//   z pass: per x, tile of y rows: real transform over kz, two real rows per
+//           complex line (z = IDFT(Ya + i Yb): x_a = Re z, x_b = Im z).
+// Spectrum layout: ((c M + x) M + y) KP + kz, kz < nkz: rows padded to whole
+// sectors, the Nyquist plane of even M (zero: it carries no noise) left out.
+// Lines lie in shared memory as [point][line], so that consecutive threads
+// touch consecutive words in every pass whatever its stride; each pass is one
+// radix of a Stockham transform (natural order in and out), from one buffer
+// to the other.  A thread transforms two neighbouring lines at a time (one
+// 16-byte access, one set of indices and twiddles for both): the passes are
+// bound by instruction issue, and with one line per thread a point cost 39
+// instructions a pass (y pass at M = 200 67 us, of 30 at the memory's rate).
+constexpr int PSE_FFT_MAXM = 512;
+constexpr int PSE_FFT_TQ = 8;    // (y, kz) modes per block of the x pass
+constexpr int PSE_FFT_TX = 256;  // its threads
+constexpr int PSE_FFT_TZ = 16;   // kz per block of the y pass
+constexpr int PSE_FFT_TY = 256;  // its threads
+constexpr int PSE_FFT_TR = 8;    // y rows per block of the z passes
+constexpr int PSE_FFT_NL = 3 * PSE_FFT_TR / 2;  // their complex lines
+constexpr int PSE_FFT_LS = PSE_FFT_NL + 2;      // room per point: the fill along kz meets 2-way bank conflicts
+constexpr int PSE_FFT_TT = 384;  // threads of the z passes
 
-template <int R> __device__ __forceinline__ constexpr int bitrev_c(int v) {
-    int r = 0;
-    for (int b = 1; b < R; b <<= 1) {
-        r = (r << 1) | (v & 1);
-        v >>= 1;
-    }
-    return r;
-}
 __device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
+__device__ __forceinline__ float2 caddf(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ float2 csubf(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// i^S a (S = +1 inverse, -1 forward)
+template <int S> __device__ __forceinline__ float2 rotf(float2 a) {
+    return S > 0 ? make_float2(-a.y, a.x) : make_float2(a.y, -a.x);
+}
+// times e^{S i phi} given (cos phi, sin phi)
+template <int S> __device__ __forceinline__ float2 twf(float2 a, float c, float s) {
+    return cmulf(a, make_float2(c, S > 0 ? s : -s));
+}
 
-// In-register radix-2 DIT of R points: v in bit-reversed order, output in
-// natural order, w[k] = w_R^k for k < R/2.
-template <int R> __device__ __forceinline__ void fft_reg(float2 (&v)[R], const float2 (&w)[R / 2]) {
+// DFT of R points in registers, natural order in and out.
+template <int R, int S> struct Dft;
+template <int S> struct Dft<2, S> {
+    static __device__ __forceinline__ void run(float2 *v) {
+        const float2 a = v[0], b = v[1];
+        v[0] = caddf(a, b);
+        v[1] = csubf(a, b);
+    }
+};
+template <int S> struct Dft<3, S> {
+    static __device__ __forceinline__ void run(float2 *v) {
+        const float2 a = caddf(v[1], v[2]), b = rotf<S>(csubf(v[1], v[2]));
+        const float2 m = make_float2(v[0].x - 0.5f * a.x, v[0].y - 0.5f * a.y);
+        constexpr float h = 0.86602540378443864676f;
+        v[0] = caddf(v[0], a);
+        v[1] = make_float2(m.x + h * b.x, m.y + h * b.y);
+        v[2] = make_float2(m.x - h * b.x, m.y - h * b.y);
+    }
+};
+template <int S> struct Dft<4, S> {
+    static __device__ __forceinline__ void run(float2 *v) {
+        const float2 a = caddf(v[0], v[2]), b = csubf(v[0], v[2]), c = caddf(v[1], v[3]),
+                     d = rotf<S>(csubf(v[1], v[3]));
+        v[0] = caddf(a, c);
+        v[1] = caddf(b, d);
+        v[2] = csubf(a, c);
+        v[3] = csubf(b, d);
+    }
+};
+// prime R: pairs v[k] +- v[R - k] against the cosines and sines of 2 pi / R
+template <int R, int S> __device__ __forceinline__ void dft_prime(float2 *v, const float (&c)[R / 2], const float (&s)[R / 2]) {
+    constexpr int H = R / 2;
+    float2 a[H], b[H], out[R];
 #pragma unroll
-    for (int half = 1; half < R; half <<= 1) {
+    for (int k = 0; k < H; ++k) {
+        a[k] = caddf(v[k + 1], v[R - 1 - k]);
+        b[k] = rotf<S>(csubf(v[k + 1], v[R - 1 - k]));
+    }
+    out[0] = v[0];
 #pragma unroll
-        for (int j = 0; j < R / 2; ++j) {
-            const int pos = j & (half - 1);
-            const int i0 = ((j - pos) << 1) + pos, i1 = i0 + half;
-            const float2 t = cmulf(w[pos * (R / (2 * half))], v[i1]);
-            const float2 a = v[i0];
-            v[i0] = make_float2(a.x + t.x, a.y + t.y);
-            v[i1] = make_float2(a.x - t.x, a.y - t.y);
+    for (int k = 0; k < H; ++k) out[0] = caddf(out[0], a[k]);
+#pragma unroll
+    for (int j = 1; j <= H; ++j) {
+        float2 e = v[0], o = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int k = 1; k <= H; ++k) {
+            const int r = (j * k) % R;
+            const float cc = c[(r <= H ? r : R - r) - 1], ss = r <= H ? s[r - 1] : -s[R - r - 1];
+            e.x = fmaf(cc, a[k - 1].x, e.x);
+            e.y = fmaf(cc, a[k - 1].y, e.y);
+            o.x = fmaf(ss, b[k - 1].x, o.x);
+            o.y = fmaf(ss, b[k - 1].y, o.y);
+        }
+        out[j] = caddf(e, o);
+        out[R - j] = csubf(e, o);
+    }
+#pragma unroll
+    for (int k = 0; k < R; ++k) v[k] = out[k];
+}
+template <int S> struct Dft<5, S> {
+    static __device__ __forceinline__ void run(float2 *v) {
+        const float c[2] = {0.30901699437494742410f, -0.80901699437494742410f};
+        const float s[2] = {0.95105651629515357212f, 0.58778525229247312917f};
+        dft_prime<5, S>(v, c, s);
+    }
+};
+template <int S> struct Dft<7, S> {
+    static __device__ __forceinline__ void run(float2 *v) {
+        const float c[3] = {0.62348980185873353053f, -0.22252093395631440429f, -0.90096886790241912624f};
+        const float s[3] = {0.78183148246802980871f, 0.97492791218182360702f, 0.43388373911755812048f};
+        dft_prime<7, S>(v, c, s);
+    }
+};
+// R = A B: A-point DFTs over the stride-B subsequences, twiddles w_R^{b j},
+// B-point DFTs; TW(b, j, value) applies a twiddle.
+template <int A, int B, int S, class TW> __device__ __forceinline__ void dft_split(float2 *v, TW tw) {
+    float2 t[A * B];
+#pragma unroll
+    for (int b = 0; b < B; ++b) {
+        float2 u[A];
+#pragma unroll
+        for (int a = 0; a < A; ++a) u[a] = v[a * B + b];
+        Dft<A, S>::run(u);
+#pragma unroll
+        for (int j = 0; j < A; ++j) t[j * B + b] = b * j ? tw(b * j, u[j]) : u[j];
+    }
+#pragma unroll
+    for (int j = 0; j < A; ++j) {
+        Dft<B, S>::run(t + j * B);
+#pragma unroll
+        for (int b = 0; b < B; ++b) v[j + A * b] = t[j * B + b];
+    }
+}
+template <int S> struct Dft<6, S> {
+    static __device__ __forceinline__ void run(float2 *v) {
+        dft_split<3, 2, S>(v, [](int e, float2 a) {
+            return e == 1 ? twf<S>(a, 0.5f, 0.86602540378443864676f) : twf<S>(a, -0.5f, 0.86602540378443864676f);
+        });
+    }
+};
+template <int S> struct Dft<8, S> {
+    static __device__ __forceinline__ void run(float2 *v) {
+        dft_split<4, 2, S>(v, [](int e, float2 a) {
+            constexpr float h = 0.70710678118654752440f;
+            return e == 1 ? twf<S>(a, h, h) : (e == 2 ? rotf<S>(a) : twf<S>(a, -h, h));
+        });
+    }
+};
+template <int S> struct Dft<9, S> {
+    static __device__ __forceinline__ void run(float2 *v) {
+        dft_split<3, 3, S>(v, [](int e, float2 a) {
+            return e == 1   ? twf<S>(a, 0.76604444311897803520f, 0.64278760968653932632f)
+                   : e == 2 ? twf<S>(a, 0.17364817766693034885f, 0.98480775301220805937f)
+                            : twf<S>(a, -0.93969262078590838405f, 0.34202014332566873304f);
+        });
+    }
+};
+// One Stockham pass of radix R over this thread's butterflies j = j0, j0 + dj, ...
+// of its two lines.  ld(n): point n of both (x, y the first line's, z, w the
+// second's); st(n, value).
+template <int R, int S, class Ld, class St>
+__device__ __forceinline__ void fft_pass(int M, int ns, uint32_t mg, int j0, int dj, const float2 *tw, Ld ld, St st) {
+    const int MR = M / R, step = MR / ns;
+    for (int j = j0; j < MR; j += dj) {
+        float2 a[R], b[R];
+#pragma unroll
+        for (int m = 0; m < R; ++m) {
+            const float4 v = ld(j + m * MR);
+            a[m] = make_float2(v.x, v.y);
+            b[m] = make_float2(v.z, v.w);
+        }
+        int q = j, k = 0;
+        if (ns > 1) {
+            q = __umulhi((uint32_t)j, mg);
+            k = j - q * ns;
+            const float2 *t = tw + k * step;
+            const float2 *e = t;
+#pragma unroll
+            for (int m = 1; m < R; ++m, e += k * step) {
+                float2 w = *e;
+                if (S < 0) w.y = -w.y;
+                a[m] = cmulf(a[m], w);
+                b[m] = cmulf(b[m], w);
+            }
+        }
+        Dft<R, S>::run(a);
+        Dft<R, S>::run(b);
+        const int o = q * ns * R + k;
+#pragma unroll
+        for (int m = 0; m < R; ++m) st(o + m * ns, make_float4(a[m].x, a[m].y, b[m].x, b[m].y));
+    }
+}
+template <int S, class Ld, class St>
+__device__ __forceinline__ void fft_pass_any(const FftPlan &p, int i, int j0, int dj, const float2 *tw, Ld ld, St st) {
+    switch (p.rad[i]) {  // uniform
+        case 2: fft_pass<2, S>(p.M, p.ns[i], p.mg[i], j0, dj, tw, ld, st); break;
+        case 3: fft_pass<3, S>(p.M, p.ns[i], p.mg[i], j0, dj, tw, ld, st); break;
+        case 4: fft_pass<4, S>(p.M, p.ns[i], p.mg[i], j0, dj, tw, ld, st); break;
+        case 5: fft_pass<5, S>(p.M, p.ns[i], p.mg[i], j0, dj, tw, ld, st); break;
+        case 6: fft_pass<6, S>(p.M, p.ns[i], p.mg[i], j0, dj, tw, ld, st); break;
+        case 7: fft_pass<7, S>(p.M, p.ns[i], p.mg[i], j0, dj, tw, ld, st); break;
+        case 8: fft_pass<8, S>(p.M, p.ns[i], p.mg[i], j0, dj, tw, ld, st); break;
+        default: fft_pass<9, S>(p.M, p.ns[i], p.mg[i], j0, dj, tw, ld, st); break;
+    }
+}
+
+// Passes [i0, i1) from one shared buffer to the other (L lines of room per
+// point, this thread on lines `line` and line + 1, line even; `on`: it has
+// lines); returns the buffer that holds the result.  The caller has
+// synchronised; so has this on return.
+template <int S, int L>
+__device__ __forceinline__ float2 *fft_smem(const FftPlan &p, int i0, int i1, int line, bool on, int j0, int dj,
+                                            const float2 *tw, float2 *cur, float2 *oth) {
+    for (int i = i0; i < i1; ++i) {
+        const float2 *in = cur + line;
+        float2 *out = oth + line;
+        if (on)
+            fft_pass_any<S>(p, i, j0, dj, tw, [&](int n) { return *reinterpret_cast<const float4 *>(in + n * L); },
+                            [&](int n, float4 v) { *reinterpret_cast<float4 *>(out + n * L) = v; });
+        __syncthreads();
+        float2 *t = cur;
+        cur = oth;
+        oth = t;
+    }
+    return cur;
+}
+
+// x pass, blockIdx = (tile of the M KP modes (y, kz), species).
+// FORCES false: modes filled with the scaled projected noise; true: the
+// forward transform over x of the spread forces' spectrum, the mode factor of
+// WAVE_MODE_DET (see k_wave_apply), with noise when with_noise.
+// The three components share one second buffer (they are transformed one
+// after the other): two blocks fit an SM up to M = 430.
+template <bool FORCES>
+__global__ void __launch_bounds__(PSE_FFT_TX, 3) k_fft_x(const __grid_constant__ FftPlan p,
+                                                         const __grid_constant__ FftJob job, int with_noise) {
+    constexpr int TQ = PSE_FFT_TQ, TF = PSE_FFT_TX / TQ, TJ = 2 * TF;
+    extern __shared__ __align__(16) float2 fsm[];
+    const WaveGeom<float> &w = job.w;
+    const int M = p.M, sp = blockIdx.y;
+    float2 *A = fsm, *B = A + 3 * M * TQ, *tw = B + M * TQ;
+    for (int k = threadIdx.x; k < M; k += PSE_FFT_TX) tw[k] = p.tw[k];
+    const int plane = M * p.KP, q0 = blockIdx.x * TQ;
+    // transforms: lines (modes) q0 + line, + 1 (plane is a multiple of 4)
+    const int line = 2 * (threadIdx.x % (TQ / 2)), jj = threadIdx.x / (TQ / 2);
+    const bool on = q0 + line < plane;
+    float2 *g = job.spec + (int64_t)sp * 3 * M * plane + q0 + line;  // point n of component c: g[(c M + n) plane]
+    __syncthreads();
+    if constexpr (FORCES) {
+        for (int c = 0; c < 3; ++c) {
+            // an even number of shared passes after the first one ends in A
+            float2 *Ac = A + c * M * TQ, *cur = (p.nf & 1) ? Ac : B, *oth = (p.nf & 1) ? B : Ac;
+            const float2 *gc = g + (int64_t)c * M * plane;
+            float2 *a = cur + line;
+            if (on)
+                fft_pass_any<-1>(p, 0, jj, TJ, tw,
+                                 [&](int n) { return *reinterpret_cast<const float4 *>(gc + (int64_t)n * plane); },
+                                 [&](int n, float4 v) { *reinterpret_cast<float4 *>(a + n * TQ) = v; });
+            __syncthreads();
+            fft_smem<-1, TQ>(p, 1, p.nf, line, on, jj, TJ, tw, cur, oth);
         }
     }
-}
-
-// w_M^j for any j >= 0 from the half-circle table tw[k] = w_M^k, k < M/2.
-template <int M> __device__ __forceinline__ float2 tw_full(const float2 *tw, int j) {
-    j &= M - 1;
-    const float2 e = tw[j & (M / 2 - 1)];
-    return j < M / 2 ? e : make_float2(-e.x, -e.y);
-}
-
-// One line of M = R^2 points, natural order in `line` (stride 1, R (R + 1)
-// entries of room), transformed by the R threads t = 0..R-1 of a group;
-// returns X[t + R k2] in out[k2].  The group's threads must lie in one warp.
-template <int R>
-__device__ __forceinline__ void fft_line_sq(float2 *line, int t, const float2 *tw, const float2 (&wR)[R / 2],
-                                            float2 (&out)[R]) {
-    constexpr int M = R * R;
-    float2 v[R];
-#pragma unroll
-    for (int m = 0; m < R; ++m) v[m] = line[t + R * bitrev_c<R>(m)];
-    fft_reg<R>(v, wR);
-#pragma unroll
-    for (int k1 = 1; k1 < R; ++k1) v[k1] = cmulf(v[k1], tw_full<M>(tw, t * k1));
-    __syncwarp();
-#pragma unroll
-    for (int k1 = 0; k1 < R; ++k1) line[k1 * (R + 1) + t] = v[k1];
-    __syncwarp();
-#pragma unroll
-    for (int m = 0; m < R; ++m) out[m] = line[t * (R + 1) + bitrev_c<R>(m)];
-    fft_reg<R>(out, wR);
-    __syncwarp();
-}
-
-// Shared-memory line stride: room for the R (R + 1) transpose, padded to
-// 4 mod 16 float2 so that the TZ lines touched by one row of a tile load or
-// store start on different banks.
-template <int R> constexpr int fft_lsz() { return R * (R + 1) + ((4 - R * (R + 1)) % 16 + 16) % 16; }
-
-template <int R> __device__ __forceinline__ void load_wR(const float2 *tw, float2 (&wR)[R / 2]) {
-#pragma unroll
-    for (int k = 0; k < R / 2; ++k) wR[k] = tw[k * R];  // w_R^k = w_M^{k R}
-}
-
-// pass x: block = (tile of TZ kz values, ky); threads: 3 TZ lines x R.
-template <int R>
-__global__ void __launch_bounds__(3 * PSE_FFT_TZ * R, 3) k_fftx_noise(WaveGeom<float> w, const SampleArgs<float> *args,
-                                                                   int system, const float2 *__restrict__ tw_g,
-                                                                   float2 *spec) {
-    constexpr int M = R * R, TZ = PSE_FFT_TZ, LSZ = fft_lsz<R>(), Mh1 = M / 2 + 1;
-    extern __shared__ float2 sm[];
-    float2 *tw = sm;           // M/2
-    float2 *buf = sm + M / 2;  // [3 TZ lines][LSZ], line = c * TZ + kzl
-    for (int k = threadIdx.x; k < M / 2; k += blockDim.x) tw[k] = tw_g[k];
-    const int kz0 = blockIdx.x * TZ, ky = blockIdx.y;
-    const uint32_t strm = 2u * system + 1u;
-    const uint64_t seed = args->seed, sample = args->sample;
-    for (int i = threadIdx.x; i < M * TZ; i += blockDim.x) {
-        const int kzl = i % TZ, kx = i / TZ;
-        ModeIdx m;
-        m.ix = kx; m.iy = ky; m.iz = kz0 + kzl;
-        m.nx = kx <= M / 2 ? kx : kx - M;
-        m.ny = ky <= M / 2 ? ky : ky - M;
-        m.nz = m.iz;
-        m.live = kx != M / 2 && ky != M / 2 && (m.nx | m.ny | m.nz) != 0;
-        float2 o0 = make_float2(0.f, 0.f), o1 = o0, o2 = o0;
-        if (m.live) {
-            float wr[3], wi[3];
-            mode_noise<float>(m, M, Mh1, strm, seed, sample, wr, wi);
-            float hx, hy, hz;
-            const float sc = mode_scale<float>(m, w, hx, hy, hz);
-            const float dr = hx * wr[0] + hy * wr[1] + hz * wr[2];
-            const float di = hx * wi[0] + hy * wi[1] + hz * wi[2];
-            o0 = make_float2(sc * (wr[0] - hx * dr), sc * (wi[0] - hx * di));
-            o1 = make_float2(sc * (wr[1] - hy * dr), sc * (wi[1] - hy * di));
-            o2 = make_float2(sc * (wr[2] - hz * dr), sc * (wi[2] - hz * di));
-        }
-        buf[(0 * TZ + kzl) * LSZ + kx] = o0;
-        buf[(1 * TZ + kzl) * LSZ + kx] = o1;
-        buf[(2 * TZ + kzl) * LSZ + kx] = o2;
-    }
-    __syncthreads();
-    float2 wR[R / 2];
-    load_wR<R>(tw, wR);
-    const int line = threadIdx.x / R, t = threadIdx.x % R;
-    float2 out[R];
-    fft_line_sq<R>(buf + line * LSZ, t, tw, wR, out);
-#pragma unroll
-    for (int k2 = 0; k2 < R; ++k2) buf[line * LSZ + t + R * k2] = out[k2];
-    __syncthreads();
-    for (int i = threadIdx.x; i < 3 * M * TZ; i += blockDim.x) {
-        const int kzl = i % TZ, rest = i / TZ, ix = rest % M, c = rest / M;
-        spec[(((int64_t)c * M + ix) * M + ky) * Mh1 + kz0 + kzl] = buf[(c * TZ + kzl) * LSZ + ix];
-    }
-}
-
-// pass y: block = (tile of TZ kz values, ix); in place.
-template <int R>
-__global__ void __launch_bounds__(3 * PSE_FFT_TZ * R, 3) k_ffty(const float2 *__restrict__ tw_g, float2 *spec) {
-    constexpr int M = R * R, TZ = PSE_FFT_TZ, LSZ = fft_lsz<R>(), Mh1 = M / 2 + 1;
-    extern __shared__ float2 sm[];
-    float2 *tw = sm;
-    float2 *buf = sm + M / 2;
-    for (int k = threadIdx.x; k < M / 2; k += blockDim.x) tw[k] = tw_g[k];
-    const int kz0 = blockIdx.x * TZ, ix = blockIdx.y;
-    for (int i = threadIdx.x; i < 3 * M * TZ; i += blockDim.x) {
-        const int kzl = i % TZ, rest = i / TZ, ky = rest % M, c = rest / M;
-        buf[(c * TZ + kzl) * LSZ + ky] = spec[(((int64_t)c * M + ix) * M + ky) * Mh1 + kz0 + kzl];
-    }
-    __syncthreads();
-    float2 wR[R / 2];
-    load_wR<R>(tw, wR);
-    const int line = threadIdx.x / R, t = threadIdx.x % R;
-    float2 out[R];
-    fft_line_sq<R>(buf + line * LSZ, t, tw, wR, out);
-#pragma unroll
-    for (int k2 = 0; k2 < R; ++k2) buf[line * LSZ + t + R * k2] = out[k2];
-    __syncthreads();
-    for (int i = threadIdx.x; i < 3 * M * TZ; i += blockDim.x) {
-        const int kzl = i % TZ, rest = i / TZ, ky = rest % M, c = rest / M;
-        spec[(((int64_t)c * M + ix) * M + ky) * Mh1 + kz0 + kzl] = buf[(c * TZ + kzl) * LSZ + ky];
-    }
-}
-
-// pass z: block = (tile of TY iy rows, ix); the 3 TY real rows (c, iyl) are
-// transformed in pairs (c, iyl) + i (c, iyl + TY/2).
-template <int R>
-__global__ void __launch_bounds__(3 * PSE_FFT_TY / 2 * R) k_fftz_c2r(const float2 *__restrict__ tw_g,
-                                                                   const float2 *__restrict__ spec, V4<float> *grid4) {
-    constexpr int M = R * R, H = M / 2, TY = PSE_FFT_TY, LSZ = fft_lsz<R>(), Mh1 = M / 2 + 1, NP = 3 * TY / 2;
-    extern __shared__ float2 sm[];
-    float2 *tw = sm;                      // M/2
-    float2 *raw = tw + M / 2;             // [3][TY][H]
-    float2 *buf = raw + 3 * TY * H;       // [NP][LSZ]
-    float *xo = reinterpret_cast<float *>(raw);  // [3][TY][M], over raw once Z is built
-    for (int k = threadIdx.x; k < M / 2; k += blockDim.x) tw[k] = tw_g[k];
-    const int iy0 = blockIdx.x * TY, ix = blockIdx.y;
-    for (int i = threadIdx.x; i < 3 * TY * H; i += blockDim.x) {
-        const int k = i % H, rest = i / H, iyl = rest % TY, c = rest / TY;
-        raw[i] = spec[(((int64_t)c * M + ix) * M + iy0 + iyl) * Mh1 + k];
-    }
-    __syncthreads();
-    // pair p = c * (TY/2) + j holds rows (c, j) and (c, j + TY/2)
-    for (int i = threadIdx.x; i < NP * M; i += blockDim.x) {
-        const int k = i % M, p = i / M, c = p / (TY / 2), j = p % (TY / 2);
-        const float2 *ra = raw + (c * TY + j) * H, *rb = raw + (c * TY + j + TY / 2) * H;
-        float2 ya, yb;
-        if (k < H) {
-            ya = ra[k];
-            yb = rb[k];
-        } else if (k == H) {
-            ya = yb = make_float2(0.f, 0.f);
-        } else {
-            const float2 a = ra[M - k], b = rb[M - k];
-            ya = make_float2(a.x, -a.y);
-            yb = make_float2(b.x, -b.y);
-        }
-        buf[p * LSZ + k] = make_float2(ya.x - yb.y, ya.y + yb.x);  // Ya + i Yb
-    }
-    __syncthreads();
-    float2 wR[R / 2];
-    load_wR<R>(tw, wR);
-    const int p = threadIdx.x / R, t = threadIdx.x % R;
-    float2 out[R];
-    fft_line_sq<R>(buf + p * LSZ, t, tw, wR, out);
     {
-        const int c = p / (TY / 2), j = p % (TY / 2);
-        float *xa = xo + (c * TY + j) * M, *xb = xo + (c * TY + j + TY / 2) * M;
+        // one mode (of each kx) per thread
+        const int fl = threadIdx.x % TQ, q = q0 + fl;
+        ModeIdx m;
+        m.iy = q / p.KP;
+        m.iz = q - m.iy * p.KP;
+        m.nz = m.iz;
+        m.ny = m.iy <= M / 2 ? m.iy : m.iy - M;
+        const bool col = q < plane && m.iz < p.nkz && !((M & 1) == 0 && m.iy == M / 2);
+        const uint32_t strm = 2u * job.system + 1u;
+        const uint64_t seed = job.args->seed, sample = job.args->sample;
+        const float cd = FORCES ? (float)job.args->c_det * w.norm : 0.f, cn = FORCES ? (float)job.args->c_noise : 1.f;
+        for (int kx = threadIdx.x / TQ; kx < M; kx += TF) {
+            m.ix = kx;
+            m.nx = kx <= M / 2 ? kx : kx - M;
+            m.live = col && !((M & 1) == 0 && kx == M / 2) && (m.nx | m.ny | m.nz) != 0;
+            float2 o[3] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+            float2 *at = A + kx * TQ + fl;
+            if (m.live) {
+                float hx, hy, hz;
+                float sc = mode_scale<float>(m, w, hx, hy, hz);
+                if (!FORCES && sp) sc = w.sc_tab[sp * w.sc_stride + 2 * (m.nx * m.nx + m.ny * m.ny + m.nz * m.nz)];
+                const float hh[3] = {hx, hy, hz};
+                if constexpr (FORCES) {
+                    const float f = cd * sc * sc;
+                    const float2 v[3] = {at[0], at[M * TQ], at[2 * M * TQ]};
+                    const float dr = hx * v[0].x + hy * v[1].x + hz * v[2].x;
+                    const float di = hx * v[0].y + hy * v[1].y + hz * v[2].y;
 #pragma unroll
-        for (int k2 = 0; k2 < R; ++k2) {
-            xa[t + R * k2] = out[k2].x;
-            xb[t + R * k2] = out[k2].y;
+                    for (int d = 0; d < 3; ++d) o[d] = make_float2(f * (v[d].x - hh[d] * dr), f * (v[d].y - hh[d] * di));
+                }
+                if (!FORCES || with_noise) {
+                    float wr[3], wi[3];
+                    mode_noise<float>(m, M, w.Mh1, strm, seed, sample, wr, wi);
+                    const float f = cn * sc;
+                    const float dr = hx * wr[0] + hy * wr[1] + hz * wr[2];
+                    const float di = hx * wi[0] + hy * wi[1] + hz * wi[2];
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) {
+                        o[d].x += f * (wr[d] - hh[d] * dr);
+                        o[d].y += f * (wi[d] - hh[d] * di);
+                    }
+                }
+            }
+            at[0] = o[0];
+            at[M * TQ] = o[1];
+            at[2 * M * TQ] = o[2];
         }
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < TY * M; i += blockDim.x) {
-        const int iz = i % M, iyl = i / M;
-        V4<float> v;
-        v.x = xo[(0 * TY + iyl) * M + iz];
-        v.y = xo[(1 * TY + iyl) * M + iz];
-        v.z = xo[(2 * TY + iyl) * M + iz];
-        v.w = 0.f;
-        grid4[((int64_t)ix * M + iy0 + iyl) * M + iz] = v;
+    for (int c = 0; c < 3; ++c) {
+        const float2 *in = fft_smem<1, TQ>(p, 0, p.nf - 1, line, on, jj, TJ, tw, A + c * M * TQ, B) + line;
+        float2 *gc = g + (int64_t)c * M * plane;
+        if (on)
+            fft_pass_any<1>(p, p.nf - 1, jj, TJ, tw,
+                            [&](int n) { return *reinterpret_cast<const float4 *>(in + n * TQ); },
+                            [&](int n, float4 v) { *reinterpret_cast<float4 *>(gc + (int64_t)n * plane) = v; });
+        __syncthreads();  // B is the next component's
     }
 }
 
-template <int R> static size_t fft_smem_xy() {
-    return sizeof(float2) * (R * R / 2 + 3 * PSE_FFT_TZ * fft_lsz<R>());
-}
-template <int R> static size_t fft_smem_z() {
-    constexpr int M = R * R;  // raw (3 TY rows of M/2 float2) is reused for the 3 TY rows of M real outputs
-    return sizeof(float2) * (M / 2 + 3 * PSE_FFT_TY * (M / 2) + 3 * PSE_FFT_TY / 2 * fft_lsz<R>());
+// y pass in place, blockIdx = (tile of kz, x, component + 3 species).
+template <int S>
+__global__ void __launch_bounds__(PSE_FFT_TY, 3) k_fft_y(const __grid_constant__ FftPlan p,
+                                                         float2 *__restrict__ spec) {
+    constexpr int TZ = PSE_FFT_TZ, TJ = 2 * PSE_FFT_TY / TZ;
+    extern __shared__ __align__(16) float2 fsm[];
+    const int M = p.M;
+    float2 *A = fsm, *B = A + M * TZ, *tw = B + M * TZ;
+    for (int k = threadIdx.x; k < M; k += PSE_FFT_TY) tw[k] = p.tw[k];
+    const int line = 2 * (threadIdx.x % (TZ / 2)), jj = threadIdx.x / (TZ / 2), kz = blockIdx.x * TZ + line;
+    const bool on = kz < p.KP;  // even KP: both lines have room
+    float2 *g = spec + ((int64_t)blockIdx.z * M + blockIdx.y) * M * p.KP + kz;
+    __syncthreads();
+    float2 *a = A + line;
+    if (on)
+        fft_pass_any<S>(p, 0, jj, TJ, tw, [&](int n) { return *reinterpret_cast<const float4 *>(g + n * p.KP); },
+                        [&](int n, float4 v) { *reinterpret_cast<float4 *>(a + n * TZ) = v; });
+    __syncthreads();
+    const float2 *in = fft_smem<S, TZ>(p, 1, p.nf - 1, line, on, jj, TJ, tw, A, B) + line;
+    if (on)
+        fft_pass_any<S>(p, p.nf - 1, jj, TJ, tw, [&](int n) { return *reinterpret_cast<const float4 *>(in + n * TZ); },
+                        [&](int n, float4 v) { *reinterpret_cast<float4 *>(g + n * p.KP) = v; });
 }
 
-template <int R> static void fused_fft_launch(const WaveGeom<float> &w, const SampleArgs<float> *args, int system,
-                                              const Dev<float> &d, int parts, cudaStream_t s) {
-    constexpr int M = R * R;
-    const float2 *tw = reinterpret_cast<const float2 *>(w.fft_tw);
-    float2 *spec = reinterpret_cast<float2 *>(d.spec);
-    const dim3 gxy(M / 2 / PSE_FFT_TZ, M), gz(M / PSE_FFT_TY, M);
-    if (parts & 1) k_fftx_noise<R><<<gxy, 3 * PSE_FFT_TZ * R, fft_smem_xy<R>(), s>>>(w, args, system, tw, spec);
-    if (parts & 2) k_ffty<R><<<gxy, 3 * PSE_FFT_TZ * R, fft_smem_xy<R>(), s>>>(tw, spec);
-    if (parts & 4) k_fftz_c2r<R><<<gz, 3 * PSE_FFT_TY / 2 * R, fft_smem_z<R>(), s>>>(tw, spec, d.grid4);
+// Inverse z pass, blockIdx = (tile of y rows, x, species): spectrum rows -> node-major records.
+__global__ void __launch_bounds__(PSE_FFT_TT, 2) k_fft_z_inv(const __grid_constant__ FftPlan p,
+                                                          const float2 *__restrict__ spec,
+                                                          V4<float> *__restrict__ grid4) {
+    constexpr int TR = PSE_FFT_TR, NL = PSE_FFT_NL, LS = PSE_FFT_LS, T = PSE_FFT_TT;
+    extern __shared__ __align__(16) float2 fsm[];
+    const int M = p.M, sp = blockIdx.z, H = M / 2, nkz = p.nkz;
+    float2 *A = fsm, *B = A + M * LS, *tw = B + M * LS;
+    for (int k = threadIdx.x; k < M; k += T) tw[k] = p.tw[k];
+    const int y0 = blockIdx.x * TR, x = blockIdx.y;
+    const float2 *src = spec + ((int64_t)sp * 3 * M + x) * M * p.KP;
+    // line l = 3 pair + component holds rows y0 + 2 pair, + 1
+    for (int l = threadIdx.x / 32; l < NL; l += T / 32) {
+        const int pr = l / 3, c = l - 3 * pr, ya = y0 + 2 * pr;
+        const float2 *ra = src + ((int64_t)c * M * M + ya) * p.KP;
+        const bool oa = ya < M, ob = ya + 1 < M;
+        float2 *d = A + l;
+        for (int k0 = threadIdx.x & 31; k0 < nkz; k0 += 128) {  // four loads of each row in flight
+            float2 a[4], b[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int k = k0 + 32 * u;
+                a[u] = oa && k < nkz ? ra[k] : make_float2(0.f, 0.f);
+                b[u] = ob && k < nkz ? ra[p.KP + k] : make_float2(0.f, 0.f);
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const int k = k0 + 32 * u;
+                if (k >= nkz) break;
+                if (k == 0) {
+                    d[0] = make_float2(a[u].x, b[u].x);  // the mean of a real row is real
+                } else {
+                    d[k * LS] = make_float2(a[u].x - b[u].y, a[u].y + b[u].x);
+                    d[(M - k) * LS] = make_float2(a[u].x + b[u].y, b[u].x - a[u].y);
+                }
+            }
+        }
+        if ((M & 1) == 0 && (threadIdx.x & 31) == 0) d[H * LS] = make_float2(0.f, 0.f);  // Nyquist
+    }
+    __syncthreads();
+    const int line = 2 * (threadIdx.x % (NL / 2)), jj = threadIdx.x / (NL / 2);
+    const float2 *z = fft_smem<1, LS>(p, 0, p.nf, line, true, jj, 2 * T / NL, tw, A, B);
+    V4<float> *out = grid4 + (((int64_t)sp * M + x) * M + y0) * M;
+    // a warp writes 32 consecutive records of a pair's two rows
+    const int chunks = (M + 31) >> 5;
+    for (int t = threadIdx.x >> 5; t < TR / 2 * chunks; t += T / 32) {
+        const int pr = t & (TR / 2 - 1), n = (t / (TR / 2)) * 32 + (threadIdx.x & 31), ya = y0 + 2 * pr;
+        if (n >= M) continue;
+        const float2 *e = z + n * LS + 3 * pr;
+        const float2 v0 = e[0], v1 = e[1], v2 = e[2];
+        V4<float> r;
+        r.w = 0.f;
+        if (ya < M) {
+            r.x = v0.x; r.y = v1.x; r.z = v2.x;
+            out[2 * pr * M + n] = r;
+        }
+        if (ya + 1 < M) {
+            r.x = v0.y; r.y = v1.y; r.z = v2.y;
+            out[(2 * pr + 1) * M + n] = r;
+        }
+    }
 }
 
-bool fused_fft_supported(int M) { return M == 64 || M == 256; }
+// Forward z pass: planar real grids -> spectrum rows (kz < nkz).
+__global__ void __launch_bounds__(PSE_FFT_TT, 2) k_fft_z_fwd(const __grid_constant__ FftPlan p, const float *__restrict__ grid,
+                                                          float2 *__restrict__ spec) {
+    constexpr int TR = PSE_FFT_TR, NL = PSE_FFT_NL, LS = PSE_FFT_LS, T = PSE_FFT_TT;
+    extern __shared__ __align__(16) float2 fsm[];
+    const int M = p.M;
+    float2 *A = fsm, *B = A + M * LS, *tw = B + M * LS;
+    for (int k = threadIdx.x; k < M; k += T) tw[k] = p.tw[k];
+    const int y0 = blockIdx.x * TR, x = blockIdx.y;
+    for (int l = threadIdx.x / 32; l < NL; l += T / 32) {
+        const int pr = l / 3, c = l - 3 * pr, ya = y0 + 2 * pr;
+        const float *ra = grid + (((int64_t)c * M + x) * M + ya) * M;
+        const bool oa = ya < M, ob = ya + 1 < M;
+        for (int n = threadIdx.x & 31; n < M; n += 32)
+            A[n * LS + l] = make_float2(oa ? ra[n] : 0.f, ob ? ra[M + n] : 0.f);
+    }
+    __syncthreads();
+    const int line = 2 * (threadIdx.x % (NL / 2)), jj = threadIdx.x / (NL / 2);
+    const float2 *z = fft_smem<-1, LS>(p, 0, p.nf, line, true, jj, 2 * T / NL, tw, A, B);
+    for (int l = threadIdx.x / 32; l < NL; l += T / 32) {
+        const int pr = l / 3, c = l - 3 * pr, ya = y0 + 2 * pr;
+        float2 *ra = spec + (((int64_t)c * M + x) * M + ya) * p.KP;
+        for (int k = threadIdx.x & 31; k < p.nkz; k += 32) {
+            const float2 a = z[k * LS + l], b = z[(k ? M - k : 0) * LS + l];
+            // Ya = (Z_k + conj Z_{M-k}) / 2, Yb = (Z_k - conj Z_{M-k}) / 2i
+            if (ya < M) ra[k] = make_float2(0.5f * (a.x + b.x), 0.5f * (a.y - b.y));
+            if (ya + 1 < M) ra[p.KP + k] = make_float2(0.5f * (a.y + b.y), 0.5f * (b.x - a.x));
+        }
+    }
+}
 
-template <int R> static cudaError_t fused_fft_attrs() {
-    cudaError_t e = cudaFuncSetAttribute(k_fftx_noise<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)fft_smem_xy<R>());
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_ffty<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fft_smem_xy<R>());
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_fftz_c2r<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)fft_smem_z<R>());
+static size_t fft_smem_x(int M) { return sizeof(float2) * M * (1 + 4 * PSE_FFT_TQ); }
+static size_t fft_smem_y(int M) { return sizeof(float2) * M * (1 + 2 * PSE_FFT_TZ); }
+static size_t fft_smem_z(int M) { return sizeof(float2) * M * (1 + 2 * PSE_FFT_LS); }
+
+// Factors of M (2..4 of them, as few as possible, then the smallest largest
+// one) among the radices above; false where there are none.
+bool fft_plan(int M, FftPlan *p) {
+    static const int R[] = {9, 8, 7, 6, 5, 4, 3, 2};
+    if (M < 16 || M > PSE_FFT_MAXM) return false;
+    int best[4] = {}, nbest = 5, bmax = 99, cur[4] = {};
+    auto rec = [&](auto &&self, int m, int n, int i0) -> void {
+        if (m == 1) {
+            if (n < 2) return;
+            if (n < nbest || (n == nbest && cur[0] < bmax)) {
+                nbest = n;
+                bmax = cur[0];
+                for (int i = 0; i < n; ++i) best[i] = cur[i];
+            }
+            return;
+        }
+        if (n == 4) return;
+        for (int i = i0; i < (int)(sizeof(R) / sizeof(R[0])); ++i)
+            if (m % R[i] == 0) {
+                cur[n] = R[i];
+                self(self, m / R[i], n + 1, i);
+            }
+    };
+    rec(rec, M, 0, 0);
+    if (nbest > 4) return false;
+    p->M = M;
+    p->nkz = (M + 1) / 2;
+    p->KP = (p->nkz + 3) & ~3;
+    p->nf = nbest;
+    int ns = 1;
+    for (int i = 0; i < nbest; ++i) {
+        p->rad[i] = best[i];
+        p->ns[i] = ns;
+        p->mg[i] = ns > 1 ? (uint32_t)((0x100000000ull + ns - 1) / ns) : 0u;  // j / ns for j < 2^16
+        ns *= best[i];
+    }
+    return true;
+}
+
+// Shared memory of the passes for every grid size; once per device, outside
+// any capture.
+cudaError_t fft_prepare() {
+    const int zx = (int)fft_smem_x(PSE_FFT_MAXM), zy = (int)fft_smem_y(PSE_FFT_MAXM), zz = (int)fft_smem_z(PSE_FFT_MAXM);
+    constexpr auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    cudaError_t e = cudaFuncSetAttribute(k_fft_x<false>, attr, zx);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_x<true>, attr, zx);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_y<1>, attr, zy);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_y<-1>, attr, zy);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_z_inv, attr, zz);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_z_fwd, attr, zz);
     return e;
 }
 
-cudaError_t fused_fft_prepare(int M) {
-    if (M == 64) return fused_fft_attrs<8>();
-    if (M == 256) return fused_fft_attrs<16>();
-    return cudaErrorInvalidValue;
+// Where these transforms are faster than noise kernel + cuFFT + node-major
+// copy, from whole samples and forces calls both ways (random spheres, xi a =
+// 0.52, us, cuFFT -> ours): M = 147 355 -> 319, 189 637 -> 529, 200 at phi
+// 0.05 451 -> 374, 294 2609 -> 1935, 375 5020 -> 4160; forces 147 752 -> 662,
+// 245 3169 -> 2640.  Below 145 a sample waits for the near field either way
+// and forces lose (M = 100 250 -> 291, 128 429 -> 464).  cuFFT's transforms
+// of powers of two are as fast (256: 249 us against 255 for noise, x and y)
+// and its shorter blocks yield sooner to the near field's one-wave kernels
+// (256: 1212 -> 1293, 512: 9970 -> 11160).  The same delay outweighs the gain
+// above 245 in dense systems (M = 288: phi 0.25, M^3 / N = 6.7, 4788 -> 5143;
+// phi 0.15, 11, 2514 -> 2555; phi 0.05, 34, 1194 -> 1041), above 375 sooner
+// (378: 17, 4258 -> 4392; 34, 2562 -> 2395), and from 490 everywhere (34: 490
+// 5943 -> 6182, 486 7315 -> 5389): one block of the x pass per SM.
+bool fft_wins(int M, int nspec, int64_t N) {
+    if (M < 145 || M >= 490 || (M & (M - 1)) == 0) return false;
+    return M <= 245 || (double)M * M * M * nspec >= (M > 375 ? 30.0 : 10.0) * N;
 }
 
-void launch_fused_fft(const WaveGeom<float> &w, const SampleArgs<float> *args, int system, const Dev<float> &d,
-                      int parts, cudaStream_t s) {
-    if (w.M == 64) fused_fft_launch<8>(w, args, system, d, parts, s);
-    else fused_fft_launch<16>(w, args, system, d, parts, s);
+template <int S> static void fft_y(const FftPlan &p, const FftJob &job, int nspec, cudaStream_t s) {
+    const dim3 grid((p.nkz + PSE_FFT_TZ - 1) / PSE_FFT_TZ, p.M, 3 * nspec);
+    k_fft_y<S><<<grid, PSE_FFT_TY, fft_smem_y(p.M), s>>>(p, job.spec);
+}
+static void fft_z_inv(const FftPlan &p, const FftJob &job, int nspec, cudaStream_t s) {
+    const dim3 grid((p.M + PSE_FFT_TR - 1) / PSE_FFT_TR, p.M, nspec);
+    k_fft_z_inv<<<grid, PSE_FFT_TT, fft_smem_z(p.M), s>>>(p, job.spec, job.grid4);
+}
+// parts: bit 0 the x pass (with the noise), bit 1 the y pass, bit 2 the z pass
+void launch_fft_sample(const FftPlan &p, const FftJob &job, int parts, cudaStream_t s) {
+    const int nspec = job.w.nspec > 1 ? job.w.nspec : 1;
+    const dim3 gx((p.M * p.KP + PSE_FFT_TQ - 1) / PSE_FFT_TQ, nspec);
+    if (parts & 1) k_fft_x<false><<<gx, PSE_FFT_TX, fft_smem_x(p.M), s>>>(p, job, 0);
+    if (parts & 2) fft_y<1>(p, job, nspec, s);
+    if (parts & 4) fft_z_inv(p, job, nspec, s);
+}
+// The wave product of the spread grid (planar, `grid`): forward transform,
+// mode factor (and noise), inverse transform into the node-major grid.
+void launch_fft_forces(const FftPlan &p, const FftJob &job, const float *grid, int with_noise, cudaStream_t s) {
+    const dim3 gz((p.M + PSE_FFT_TR - 1) / PSE_FFT_TR, p.M);
+    k_fft_z_fwd<<<gz, PSE_FFT_TT, fft_smem_z(p.M), s>>>(p, grid, job.spec);
+    fft_y<-1>(p, job, 1, s);
+    const dim3 gx((p.M * p.KP + PSE_FFT_TQ - 1) / PSE_FFT_TQ);
+    k_fft_x<true><<<gx, PSE_FFT_TX, fft_smem_x(p.M), s>>>(p, job, with_noise);
+    fft_y<1>(p, job, 1, s);
+    fft_z_inv(p, job, 1, s);
 }
 
 #define PSE_INST(T)                                                                                      \

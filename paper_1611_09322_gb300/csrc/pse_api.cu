@@ -47,7 +47,9 @@ struct pse_ctx {
     cudaGraphConditionalHandle cond[6] = {};
     cufftHandle fft_r2c = 0;                            // forward FFT (spreading / grid noise)
     bool r2c_made = false;
-    bool fused_fft = false;                             // sample path: our noise + C2R kernels (FP32, M = 2^k)
+    bool may_own_fft = false;                           // our transforms can stand in for cuFFT's (FP32)
+    bool own_fft = false;                               // and do, at this N
+    FftPlan fplan{};
     SpreadTile spread{};                                // spreading tile shape
     bool spread_ready = false, spread_tuned = false;
     size_t spread_smem_max = 0;                         // dynamic shared memory the spreading may use
@@ -284,6 +286,41 @@ template <typename T> void fill_geom(pse_ctx *c) {
     wgeom<T>(c) = w;
 }
 
+// Modes of one component that a spectrum buffer has room for: cuFFT's rows of
+// M/2 + 1 or our padded ones.
+static int64_t spec_plane(int64_t M) {
+    const int64_t h1 = M / 2 + 1, kp = ((M + 1) / 2 + 3) & ~3ll;
+    return M * M * (h1 > kp ? h1 : kp);
+}
+
+// The table e^{2 pi i k / M} of our transforms.
+static pse_status fft_twiddles(std::vector<void *> &list, FftPlan *p) {
+    std::vector<float2> tw(p->M);
+    for (int k = 0; k < p->M; ++k)
+        tw[k] = make_float2((float)cos(2 * M_PI * k / p->M), (float)sin(2 * M_PI * k / p->M));
+    float2 *d = nullptr;
+    const pse_status st = alloc(list, (void **)&d, sizeof(float2) * tw.size());
+    if (st != PSE_OK) return st;
+    p->tw = d;
+    CK(cudaMemcpy(d, tw.data(), sizeof(float2) * tw.size(), cudaMemcpyHostToDevice));
+    return PSE_OK;
+}
+
+static FftJob fft_job(const pse_ctx *c) {
+    return FftJob{c->wf, c->df.args, c->params.system, (float2 *)c->df.spec, c->df.grid4};
+}
+
+// Inverse (C2R, batch 3) plan: spectrum -> planar grids.
+template <typename T> pse_status ensure_c2r(pse_ctx *c) {
+    if (c->fft_made) return PSE_OK;
+    const int M = c->plan.M, S = c->nspec > 1 ? c->nspec : 1;
+    int n[3] = {M, M, M};
+    CKF(cufftPlanMany(&c->fft, 3, n, nullptr, 1, M * M * (M / 2 + 1), nullptr, 1, M * M * M,
+                      sizeof(T) == 4 ? CUFFT_C2R : CUFFT_Z2D, 3 * S));
+    c->fft_made = true;
+    return PSE_OK;
+}
+
 // Per-context buffers: table, spectrum, grid, FFT plan, streams, events.
 template <typename T> pse_status init_ctx(pse_ctx *c) {
     fill_geom<T>(c);
@@ -343,25 +380,16 @@ template <typename T> pse_status init_ctx(pse_ctx *c) {
         if ((st = alloc(c->per_ctx, (void **)&d.table_c, sizeof(V4<T>) * PSE_TABLEC_N)) != PSE_OK) return st;
         CK(cudaMemcpy(d.table_c, tc.data(), sizeof(V4<T>) * PSE_TABLEC_N, cudaMemcpyHostToDevice));
     }
-    const int64_t M = p.M, plane = M * M * (M / 2 + 1);
+    const int64_t M = p.M;
     const size_t csize = sizeof(T) * 2;
-    if ((st = alloc(c->per_ctx, &d.spec, csize * 3 * plane * S)) != PSE_OK) return st;
+    if ((st = alloc(c->per_ctx, &d.spec, csize * 3 * spec_plane(M) * S)) != PSE_OK) return st;
     if ((st = alloc(c->per_ctx, (void **)&d.grid, sizeof(T) * 3 * M * M * M * S)) != PSE_OK) return st;
     if constexpr (sizeof(T) == 4) {
-        // power-of-two grids: the sample path's own inverse FFT (needs the
-        // node-major grid of the interpolation)
-        if (c->params.wave_fft == 1 && c->params.wave_noise == 0 && wgeom<T>(c).interp_lanes == 0 &&
-            fused_fft_supported((int)M) && fused_fft_prepare((int)M) == cudaSuccess) {
-            std::vector<float> tw(M);
-            for (int64_t k = 0; k < M / 2; ++k) {
-                tw[2 * k] = (float)cos(2 * M_PI * k / M);
-                tw[2 * k + 1] = (float)sin(2 * M_PI * k / M);
-            }
-            float *d_tw = nullptr;
-            if ((st = alloc(c->per_ctx, (void **)&d_tw, sizeof(float) * tw.size())) != PSE_OK) return st;
-            CK(cudaMemcpy(d_tw, tw.data(), sizeof(float) * tw.size(), cudaMemcpyHostToDevice));
-            wgeom<T>(c).fft_tw = d_tw;
-            c->fused_fft = true;
+        // our transforms end in the node-major grid of the interpolation
+        if (c->params.wave_noise == 0 && wgeom<T>(c).interp_lanes == 0 && fft_plan((int)M, &c->fplan) &&
+            fft_prepare() == cudaSuccess) {
+            if ((st = fft_twiddles(c->per_ctx, &c->fplan)) != PSE_OK) return st;
+            c->may_own_fft = true;
         }
         cudaGetLastError();
     }
@@ -386,10 +414,8 @@ template <typename T> pse_status init_ctx(pse_ctx *c) {
     if ((st = alloc(c->per_ctx, (void **)&d.scan_sums, sizeof(int) * PSE_SCAN_ITEMS)) != PSE_OK) return st;
     if ((st = alloc(c->per_ctx, (void **)&d.pc_theta, sizeof(float) * PSE_PRECOND_NPARAM)) != PSE_OK) return st;
     c->pc_s0 = (float)(1.0 / sqrt(p.self_mobility));
-    int n[3] = {(int)M, (int)M, (int)M};
-    CKF(cufftPlanMany(&c->fft, 3, n, nullptr, 1, (int)plane, nullptr, 1, (int)(M * M * M),
-                      sizeof(T) == 4 ? CUFFT_C2R : CUFFT_Z2D, 3 * S));
-    c->fft_made = true;
+    // a grid whose transforms are ours at every N needs no cuFFT plan
+    if (!(c->may_own_fft && fft_wins((int)M, S, 1ll << 40)) && (st = ensure_c2r<T>(c)) != PSE_OK) return st;
     // The real-space chain (cell list, neighbour list, Lanczos loop) is the
     // sample's critical path and its persistent kernels size their grids to
     // the whole GPU: its streams get the highest priority and the wave
@@ -419,7 +445,7 @@ template <typename T> pse_status init_ctx(pse_ctx *c) {
 
 // Forward (R2C, batch 3) plan: grid -> spectrum, same layouts as the C2R plan.
 template <typename T> pse_status ensure_r2c(pse_ctx *c) {
-    if (c->r2c_made) return PSE_OK;
+    if (c->r2c_made || c->own_fft) return PSE_OK;
     const int M = c->plan.M;
     const int64_t plane = (int64_t)M * M * (M / 2 + 1);
     int n[3] = {M, M, M};
@@ -540,6 +566,12 @@ template <typename T> pse_status ensure(pse_ctx *c, int64_t N) {
     drop_graph(c);
     free_list(c->per_n);
     if (c->params.matvec_shape == 0 && !c->mv_tuned) geom<T>(c).mv = default_matvec_shape<T>(c->plan, N);
+    const bool asked = c->params.wave_fft == 1 && (c->plan.M == 64 || c->plan.M == 256);
+    c->own_fft = c->may_own_fft && (asked || fft_wins(c->plan.M, c->nspec > 1 ? c->nspec : 1, N));
+    if (!c->own_fft) {
+        const pse_status st = ensure_c2r<T>(c);
+        if (st != PSE_OK) return st;
+    }
     c->N = 0;
     Dev<T> &d = dev<T>(c);
     const pse_plan_info &p = c->plan;
@@ -640,8 +672,14 @@ pse_status wave_branch(pse_ctx *c, int64_t N, cudaStream_t s, int mode, cudaEven
     Dev<T> &d = dev<T>(c);
     const WaveGeom<T> &w = wgeom<T>(c);
     if constexpr (sizeof(T) == 4) {
-        if (mode == GM_SAMPLE && c->fused_fft) {
-            launch_fused_fft(w, d.args, c->params.system, d, 7, s);
+        if (c->own_fft) {
+            if (mode == GM_SAMPLE) {
+                launch_fft_sample(c->fplan, fft_job(c), 7, s);
+            } else {
+                CK(cudaMemsetAsync(d.grid, 0, sizeof(float) * 3 * w.M * w.M * (size_t)w.M, s));
+                CK(run_spread<T>(c, c->spread, s));
+                launch_fft_forces(c->fplan, fft_job(c), d.grid, gm_noise(mode), s);
+            }
             if (sorted) cudaStreamWaitEvent(s, sorted, 0);
             launch_interp<T>(N, w, geom<T>(c), d, s);
             return PSE_OK;
@@ -812,20 +850,30 @@ template <typename T> pse_status full_step(pse_ctx *c, cudaStream_t s, cudaGraph
     const int64_t M3 = (int64_t)w.M * w.M * w.M;
     CK(cudaMemsetAsync(d.grid, 0, sizeof(T) * 3 * M3, s));
     CK(run_spread<T>(c, c->spread, s, d.rec));
-    CKF(cufftSetStream(c->fft_r2c, s));
+    bool own = false;
     if constexpr (sizeof(T) == 4) {
-        CKF(cufftExecR2C(c->fft_r2c, (cufftReal *)d.grid, (cufftComplex *)d.spec));
-    } else {
-        CKF(cufftExecD2Z(c->fft_r2c, (cufftDoubleReal *)d.grid, (cufftDoubleComplex *)d.spec));
+        own = c->own_fft;
+        if (own) {
+            launch_fft_forces(c->fplan, fft_job(c), d.grid, 0, s);
+            launch_interp<T>(N, w, geom<T>(c), d, s);
+        }
     }
-    launch_wave_apply<T>(w, d.args, c->params.system, d.spec, WAVE_MODE_DET, 0, s);
-    CKF(cufftSetStream(c->fft, s));
-    if constexpr (sizeof(T) == 4) {
-        CKF(cufftExecC2R(c->fft, (cufftComplex *)d.spec, (cufftReal *)d.grid));
-    } else {
-        CKF(cufftExecZ2D(c->fft, (cufftDoubleComplex *)d.spec, (cufftDoubleReal *)d.grid));
+    if (!own) {
+        CKF(cufftSetStream(c->fft_r2c, s));
+        if constexpr (sizeof(T) == 4) {
+            CKF(cufftExecR2C(c->fft_r2c, (cufftReal *)d.grid, (cufftComplex *)d.spec));
+        } else {
+            CKF(cufftExecD2Z(c->fft_r2c, (cufftDoubleReal *)d.grid, (cufftDoubleComplex *)d.spec));
+        }
+        launch_wave_apply<T>(w, d.args, c->params.system, d.spec, WAVE_MODE_DET, 0, s);
+        CKF(cufftSetStream(c->fft, s));
+        if constexpr (sizeof(T) == 4) {
+            CKF(cufftExecC2R(c->fft, (cufftComplex *)d.spec, (cufftReal *)d.grid));
+        } else {
+            CKF(cufftExecZ2D(c->fft, (cufftDoubleComplex *)d.spec, (cufftDoubleReal *)d.grid));
+        }
+        interp<T>(c, N, s);
     }
-    interp<T>(c, N, s);
     Dev<T> da = d;
     da.mv_add = d.uwave;
     da.want_rec = true;  // the next step spreads q_{j+1} from the records
@@ -1612,10 +1660,14 @@ pse_status pse_profile_stages(pse_ctx *c, int64_t N, const float *d_pos, uint64_
         cudaMemsetAsync(&d.lz->overflow, 0, sizeof(int), s);
         cudaMemsetAsync(&d.lz->n_pairs, 0, sizeof(unsigned long long), s);
         return PSE_OK; });
-    const bool fused = c->fused_fft;
-    if (r == PSE_OK) r = timed(PSE_STAGE_WAVE_NOISE, c->params.wave_noise ? 2 : 1, [&] {
-        if (fused) {  // noise generated inside the first FFT pass (x)
-            launch_fused_fft(c->wf, d.args, c->params.system, d, 1, s);
+    // our transforms: noise with the passes over x and y, then the one over z
+    // that writes the node-major grid; with wave_fft = 1 (M = 64, 256) the
+    // last two passes are the FFT stage
+    const bool own = c->own_fft, split = own && c->params.wave_fft == 1 && (c->plan.M == 64 || c->plan.M == 256);
+    const FftJob job = fft_job(c);
+    if (r == PSE_OK) r = timed(PSE_STAGE_WAVE_NOISE, split ? 1 : (own || c->params.wave_noise ? 2 : 1), [&] {
+        if (own) {
+            launch_fft_sample(c->fplan, job, split ? 1 : 3, s);
             return PSE_OK;
         }
         if (c->params.wave_noise == 0) {
@@ -1627,17 +1679,16 @@ pse_status pse_profile_stages(pse_ctx *c, int64_t N, const float *d_pos, uint64_
         CKF(cufftExecR2C(c->fft_r2c, (cufftReal *)d.grid, (cufftComplex *)d.spec));
         launch_wave_apply<float>(c->wf, d.args, c->params.system, d.spec, WAVE_MODE_GRIDNOISE, 0, s);
         return PSE_OK; });
-    if (r == PSE_OK) r = timed(PSE_STAGE_FFT, fused ? 2 : 0, [&] {
-        if (fused) {  // y and z passes, the last one writing the node-major grid
-            launch_fused_fft(c->wf, d.args, c->params.system, d, 6, s);
-            return PSE_OK;
-        }
+    if (r == PSE_OK && split)
+        r = timed(PSE_STAGE_FFT, 2, [&] { launch_fft_sample(c->fplan, job, 6, s); return PSE_OK; });
+    if (r == PSE_OK && !own) r = timed(PSE_STAGE_FFT, 0, [&] {
         CKF(cufftSetStream(c->fft, s));
         CKF(cufftExecC2R(c->fft, (cufftComplex *)d.spec, (cufftReal *)d.grid));
         return PSE_OK; });
-    if (r == PSE_OK)
-        r = timed(PSE_STAGE_GRID_COPY, (c->wf.interp_lanes == 0 && !fused) ? 1 : 0, [&] {
-            if (!fused) launch_grid_copy<float>(c->wf, c->df, s);
+    if (r == PSE_OK && !split && c->wf.interp_lanes == 0)
+        r = timed(PSE_STAGE_GRID_COPY, 1, [&] {
+            if (own) launch_fft_sample(c->fplan, job, 4, s);
+            else launch_grid_copy<float>(c->wf, c->df, s);
             return PSE_OK; });
     if (r == PSE_OK)
         r = timed(PSE_STAGE_INTERP, 1, [&] { launch_interp<float>(N, c->wf, c->gf, c->df, s); return PSE_OK; });
@@ -1698,7 +1749,7 @@ static pse_status xi_trial(double L, double a, const pse_params &p, int64_t N, c
         st = pse_profile_stages(c, N, d_pos, 1, 900001, d_out, sm, nl, s);
         stage[0] = sm[PSE_STAGE_NEIGHBOURS] + sm[PSE_STAGE_MATVEC];
         stage[1] = sm[PSE_STAGE_WAVE_NOISE];
-        stage[2] = sm[PSE_STAGE_FFT];
+        stage[2] = sm[PSE_STAGE_FFT] + sm[PSE_STAGE_GRID_COPY];
     }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);

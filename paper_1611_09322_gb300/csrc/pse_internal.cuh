@@ -124,7 +124,6 @@ template <typename T> struct WaveGeom {
     uint32_t dv_h1_m, dv_M_m;  // division of 32-bit mode ids by Mh1 and M: multipliers
     int dv_h1_l, dv_M_l;       // and shifts (Granlund-Montgomery, round-up form)
     int big;             // M^2 Mh1 >= 2^32: 64-bit mode ids
-    const void *fft_tw;  // M/2 float2 e^{2 pi i k / M} (power-of-two grids, fused FFT path)
     int interp_lanes;    // lanes per particle in the interpolation (8, 16, 32; 0 = pick)
     int nspec;           // spectra / grids, one per species (1: monodisperse)
     int64_t sc_stride;   // entries of one species' block of sc_tab
@@ -519,13 +518,29 @@ template <typename T> void launch_matvec_caller(int64_t N, const SampleArgs<T> *
 template <typename T> void launch_wave_noise(WaveGeom<T> w, const SampleArgs<T> *args, int system, void *spec,
                                              cudaStream_t s);
 template <typename T> void launch_interp(int64_t N, WaveGeom<T> w, Geom<T> g, const Dev<T> &d, cudaStream_t s);
-// fused k-space noise + three-pass C2R into the node-major grid (FP32,
-// power-of-two M in 16..512); prepare once per M outside any capture
-bool fused_fft_supported(int M);
-cudaError_t fused_fft_prepare(int M);
-// parts: bit 0 the noise + x pass, bit 1 the y pass, bit 2 the z pass
-void launch_fused_fft(const WaveGeom<float> &w, const SampleArgs<float> *args, int system, const Dev<float> &d,
-                      int parts, cudaStream_t s);
+// The sampler's own transforms (FP32; kernels_wave.cu): grid side, its factors
+// with their strides (products of the earlier ones) and division multipliers,
+// kz kept (no Nyquist plane) and padded row length of the spectrum, and the
+// table e^{2 pi i k / M}.
+struct FftPlan {
+    int M, KP, nkz, nf;
+    int rad[4], ns[4];
+    uint32_t mg[4];
+    const float2 *tw;
+};
+struct FftJob {
+    WaveGeom<float> w;
+    const SampleArgs<float> *args;
+    int system;
+    float2 *spec;
+    V4<float> *grid4;
+};
+bool fft_plan(int M, FftPlan *p);
+cudaError_t fft_prepare();
+// whether they are the faster ones beside the near field of N particles
+bool fft_wins(int M, int nspec, int64_t N);
+void launch_fft_sample(const FftPlan &p, const FftJob &job, int parts, cudaStream_t s);
+void launch_fft_forces(const FftPlan &p, const FftJob &job, const float *grid, int with_noise, cudaStream_t s);
 // resident blocks per SM of the FP32 4x4 matvec (its persistent grid is one wave of them)
 int matvec_blocks_per_sm();
 int update_blocks_per_sm();

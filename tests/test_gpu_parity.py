@@ -479,3 +479,40 @@ def test_neighbour_search_lane_groups(torch, N, L, kind):
     plan = ewald.plan(L, 1.0, 0.5, 1e-3)
     ref = pse.RealOperator(pos.astype(np.float64), plan)(v.astype(np.float64))
     assert _rel(got, ref) < 1e-5, _rel(got, ref)
+
+
+@pytest.mark.parametrize("M", [147, 150, 162, 175, 192, 245, 360, 486])
+def test_own_transforms(torch, M):
+    """Grids with the library's own transforms (odd, even, radices 2..9, two
+    to four passes, M = 147 and 150 with ragged tiles in every pass): wave
+    part of a sample, deterministic product and sample with forces against the
+    planar form, which keeps cuFFT; two species of one radius (one grid each)
+    against the one-species wave part; the oracle at the two smallest.  1e-5
+    is float rounding through transform and interpolation, as above."""
+    from oracle import ewald, pse
+    from paper_1611_09322_gb300 import PolySampler
+    N = 2000
+    pos, L, _ = _hs(N, 0.1 * (147 / M) ** 3, 33)  # the same spacing at every M
+    d = torch.from_numpy(pos).cuda()
+    F = torch.from_numpy(np.random.default_rng(M).standard_normal((N, 3)).astype(np.float32)).cuda()
+    outs = []
+    for form in (0, 1):
+        s = _sampler(L, xi=0.5, tol=1e-3, grid_M=M, fixed_iter=3, interp_form=form)
+        w = s.sample(d, SEED, 11, parts=True)[2]
+        det = s.mobility_apply(d, F) - s.real_matvec(d, F)
+        outs.append([t.cpu().numpy() for t in (w, det, s.sample_with_forces(d, F, SEED, 5, 0.7, 1.3))])
+        launches = s.profile_stages(d, SEED, 11)
+        # noise with x and y, then z; the planar form has no node-major grid
+        assert (launches["wave_noise"][1], launches["grid_copy"][1]) == ((2, 1) if form == 0 else (1, 0))
+        s.close()
+    for a, b in zip(*outs):
+        assert _maxrel(a, b) < 1e-5, _maxrel(a, b)
+    s = PolySampler(L, (1.0, 1.0), xi=0.5, tol=1e-3, grid_M=M, fixed_iter=3)
+    sp = (torch.arange(N, device="cuda") % 2).int()
+    assert _maxrel(s.sample(d, sp, SEED, 11, parts=True)[2].cpu().numpy(), outs[0][0]) < 1e-5
+    s.close()
+    if M <= 150:
+        plan = ewald.plan(L, 1.0, 0.5, 1e-3, M=M)
+        p64 = pos.astype(np.float64)
+        assert _maxrel(outs[0][0], pse.wave_sample_grid(p64, plan, SEED, 11)) < 1e-4
+        assert _maxrel(outs[0][1], pse.wave_apply_grid(F.cpu().numpy().astype(np.float64), p64, plan)) < 1e-4
