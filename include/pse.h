@@ -69,8 +69,9 @@ typedef struct {
                             size in [M, 1.12 M] at creation and keep the fastest
                             (a finer grid only lowers the NUFFT error); needs
                             the GPU at pse_create_ex.  0: the Sec. II C grid.
-                            bit 1: time every spreading tile shape at the first
-                            forces call and keep the fastest.
+                            bit 1: time every form of the spreading (vector
+                            reductions, tile shapes) at the first forces call
+                            and keep the fastest.
                             bit 2: time every near-field matvec launch shape
                             at the first sample and keep the fastest.
                             bit 3: once the grid is fixed (planned, tuned or
@@ -85,10 +86,11 @@ typedef struct {
                             1: white noise drawn on the M^3 grid and taken to
                             k-space by a forward FFT -- same covariance, other
                             samples (the fluctuating-hydrodynamics form)       */
-    int spread_tile;     /* 0 (default): spreading tile chosen automatically
-                            (largest that fits shared memory, or timed with
-                            autotune bit 1); 1, 2 or 4: tiles of that many
-                            cells per side (PSE_ENOTSUPPORTED at the first
+    int spread_tile;     /* 0 (default): FP32 with interp_form 0 spreads by
+                            vector reductions into the node-major grid, else
+                            by tiles, the largest that fits shared memory (or
+                            the fastest form, timed with autotune bit 1); 1, 2
+                            or 4: tiles of that many cells per side (PSE_ENOTSUPPORTED at the first
                             forces call if it does not fit shared memory)      */
     int matvec_shape;    /* 0 (default): a launch shape chosen by the number of
                             particles and neighbours (FP32; pse_get_stats

@@ -271,7 +271,8 @@ __device__ __forceinline__ int wrap_grid(int i, int M) {  // valid for i in [-M,
 // each particle's P^3 support, w = exp(-ch2 (u - p)^2) per axis as in the
 // interpolation (the Gaussian's constant is applied in the mode factor).
 //
-// One CTA per tile of G^3 cells.  The tile's particles (cell-sorted, so each
+// FP64, the planar interpolation and a tile asked for: one CTA per tile of
+// G^3 cells (FP32 with the node-major grid: k_spread4).  The tile's particles (cell-sorted, so each
 // cell is a contiguous run) are spread into a padded E^3 node block in shared
 // memory with shared-memory atomics, CP components per pass.  The block
 // starts at the node orig[t] of each axis (host-computed: the support start of
@@ -690,6 +691,77 @@ template <int P> __global__ void __launch_bounds__(128) k_interp4_batch(const BS
         if (base + wofs < S.N) interp4_warp<P>(base + wofs, S.N, S.w, S.d.pos_sorted, S.d.grid4, S.d.uwave);
 }
 
+// Spreading into the node-major grid, the interpolation's mirror image: a
+// group of P lanes per particle, lane c on the z-node c, one 16-byte vector
+// reduction (all three components) per node.  Bound by the reductions that L2
+// takes (2e5 particles, P = 5: 2.5e7 of them in 73 us, 5.5 TB/s); the tiles of
+// k_spread serialise on shared-memory atomics and their blocks pass through
+// memory twice more (146 us and 78 us for the gather).  Forces calls, tiles ->
+// reductions, us: 1e3 particles 117 -> 114, 1e5 369 -> 305, 2e5 664 -> 493,
+// 1e6 2657 -> 1999; P = 9, 1e5 dense 1393 -> 1115, 3e4 dilute 1912 -> 736; no
+// density, support or N was found where tiles win.
+template <int P>
+__global__ void __launch_bounds__(128) k_spread4(int64_t N, WaveGeom<float> w, const V4<float> *__restrict__ pos_sorted,
+                                                 const SampleArgs<float> *args, const Rec<float> *__restrict__ src,
+                                                 V4<float> *grid4) {
+    constexpr int R = 32 / P;
+    const int lane = threadIdx.x & 31, g = lane / P, c = lane - g * P;
+    const int64_t s = ((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5) * R + g;
+    const bool act = g < R && s < N;
+    const int base = (g < R ? g : 0) * P;
+    const V4<float> p = pos_sorted[act ? s : 0];
+    const int M = w.M;
+    int i0x, i0y, i0z;
+    float ux, uy, uz;
+    support(p.x, w, i0x, ux);
+    support(p.y, w, i0y, uy);
+    support(p.z, w, i0z, uz);
+    const float fc = float(c), ex = ux - fc, ey = uy - fc, ez = uz - fc;
+    const float wxc = expf(-w.ch2 * ex * ex), wyc = expf(-w.ch2 * ey * ey), wzc = expf(-w.ch2 * ez * ez);
+    const int izc = wrap_grid(i0z + c, M);
+    float fx = 0.f, fy = 0.f, fz = 0.f;
+    if (act) {
+        if (src) {  // a sorted-order vector (the Lanczos vector of the full-mobility iteration)
+            const V4<float> q = src[s].q;
+            fx = q.x; fy = q.y; fz = q.z;
+        } else {
+            const float *F = args->vin + 3 * caller_of(p.w);
+            fx = F[0]; fy = F[1]; fz = F[2];
+        }
+    }
+    float wyz[P];
+    int row[P];
+#pragma unroll
+    for (int b = 0; b < P; ++b) {
+        wyz[b] = __shfl_sync(0xffffffffu, wyc, base + b) * wzc;
+        row[b] = wrap_grid(i0y + b, M) * M + izc;
+    }
+    const int64_t MM = (int64_t)M * M;
+#pragma unroll 1
+    for (int a = 0; a < P; ++a) {
+        const float wxa = __shfl_sync(0xffffffffu, wxc, base + a);
+        V4<float> *plane = grid4 + wrap_grid(i0x + a, M) * MM;
+        if (act) {
+#pragma unroll
+            for (int b = 0; b < P; ++b) {
+                const float wt = wxa * wyz[b];
+                asm volatile("red.relaxed.gpu.global.add.v4.f32 [%0], {%1, %2, %3, %4};" ::"l"(plane + row[b]),
+                             "f"(wt * fx), "f"(wt * fy), "f"(wt * fz), "f"(0.f)
+                             : "memory");
+            }
+        }
+    }
+}
+// Node-major force grid to the planar grids that cuFFT reads.
+__global__ void k_grid_planar(int64_t M3, const V4<float> *__restrict__ g4, float *__restrict__ g) {
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= M3) return;
+    const V4<float> v = g4[i];
+    g[i] = v.x;
+    g[M3 + i] = v.y;
+    g[2 * M3 + i] = v.z;
+}
+
 static inline unsigned nbw(int64_t n, int b) { return (unsigned)((n + b - 1) / b); }
 
 template <int P>
@@ -720,6 +792,31 @@ void launch_batch_interp(const BSys *sys, int *const *tab, const int *nblk, int 
     }
 }
 
+// Spread into d.grid4 (cleared here); P in 3..10.
+cudaError_t launch_spread4(int64_t N, const WaveGeom<float> &w, const Dev<float> &d, const Rec<float> *src,
+                           cudaStream_t s) {
+    const cudaError_t e = cudaMemsetAsync(d.grid4, 0, sizeof(V4<float>) * w.M * w.M * (size_t)w.M, s);
+    if (e != cudaSuccess) return e;
+    auto go = [&](auto kernel) {
+        const int64_t per = 32 / w.P, warps = (N + per - 1) / per;
+        kernel<<<nbw(warps * 32, 128), 128, 0, s>>>(N, w, d.pos_sorted, d.args, src, d.grid4);
+    };
+    switch (w.P) {
+        case 3: go(k_spread4<3>); break;
+        case 4: go(k_spread4<4>); break;
+        case 5: go(k_spread4<5>); break;
+        case 6: go(k_spread4<6>); break;
+        case 7: go(k_spread4<7>); break;
+        case 8: go(k_spread4<8>); break;
+        case 9: go(k_spread4<9>); break;
+        default: go(k_spread4<10>); break;
+    }
+    return cudaGetLastError();
+}
+void launch_grid_planar(const WaveGeom<float> &w, const Dev<float> &d, cudaStream_t s) {
+    const int64_t M3 = (int64_t)w.M * w.M * w.M;
+    k_grid_planar<<<nbw(M3, 256), 256, 0, s>>>(M3, d.grid4, d.grid);
+}
 template <typename T>
 void launch_wave_noise(WaveGeom<T> w, const SampleArgs<T> *args, int system, void *spec, cudaStream_t s) {
     const int64_t plane = (int64_t)w.M * w.M * w.Mh1;
@@ -1222,16 +1319,33 @@ __global__ void __launch_bounds__(PSE_FFT_TT, 2) k_fft_z_inv(const __grid_consta
     }
 }
 
-// Forward z pass: planar real grids -> spectrum rows (kz < nkz).
+// Forward z pass: real grids, planar or (grid4) node-major, -> spectrum rows
+// (kz < nkz).
 __global__ void __launch_bounds__(PSE_FFT_TT, 2) k_fft_z_fwd(const __grid_constant__ FftPlan p, const float *__restrict__ grid,
-                                                          float2 *__restrict__ spec) {
+                                                          const V4<float> *__restrict__ grid4, float2 *__restrict__ spec) {
     constexpr int TR = PSE_FFT_TR, NL = PSE_FFT_NL, LS = PSE_FFT_LS, T = PSE_FFT_TT;
     extern __shared__ __align__(16) float2 fsm[];
     const int M = p.M;
     float2 *A = fsm, *B = A + M * LS, *tw = B + M * LS;
     for (int k = threadIdx.x; k < M; k += T) tw[k] = p.tw[k];
     const int y0 = blockIdx.x * TR, x = blockIdx.y;
-    for (int l = threadIdx.x / 32; l < NL; l += T / 32) {
+    if (grid4) {
+        // a warp reads 32 consecutive records of a pair's two rows
+        const V4<float> *in = grid4 + ((int64_t)x * M + y0) * M;
+        const int chunks = (M + 31) >> 5;
+        for (int t = threadIdx.x >> 5; t < TR / 2 * chunks; t += T / 32) {
+            const int pr = t & (TR / 2 - 1), n = (t / (TR / 2)) * 32 + (threadIdx.x & 31), ya = y0 + 2 * pr;
+            if (n >= M) continue;
+            V4<float> a{}, b{};
+            if (ya < M) a = in[2 * pr * M + n];
+            if (ya + 1 < M) b = in[(2 * pr + 1) * M + n];
+            float2 *e = A + n * LS + 3 * pr;
+            e[0] = make_float2(a.x, b.x);
+            e[1] = make_float2(a.y, b.y);
+            e[2] = make_float2(a.z, b.z);
+        }
+    }
+    for (int l = grid4 ? NL : threadIdx.x / 32; l < NL; l += T / 32) {
         const int pr = l / 3, c = l - 3 * pr, ya = y0 + 2 * pr;
         const float *ra = grid + (((int64_t)c * M + x) * M + ya) * M;
         const bool oa = ya < M, ob = ya + 1 < M;
@@ -1344,11 +1458,12 @@ void launch_fft_sample(const FftPlan &p, const FftJob &job, int parts, cudaStrea
     if (parts & 2) fft_y<1>(p, job, nspec, s);
     if (parts & 4) fft_z_inv(p, job, nspec, s);
 }
-// The wave product of the spread grid (planar, `grid`): forward transform,
-// mode factor (and noise), inverse transform into the node-major grid.
+// The wave product of the spread grid (planar, or with grid null the node-major
+// one): forward transform, mode factor (and noise), inverse transform into the
+// node-major grid.
 void launch_fft_forces(const FftPlan &p, const FftJob &job, const float *grid, int with_noise, cudaStream_t s) {
     const dim3 gz((p.M + PSE_FFT_TR - 1) / PSE_FFT_TR, p.M);
-    k_fft_z_fwd<<<gz, PSE_FFT_TT, fft_smem_z(p.M), s>>>(p, grid, job.spec);
+    k_fft_z_fwd<<<gz, PSE_FFT_TT, fft_smem_z(p.M), s>>>(p, grid, grid ? nullptr : job.grid4, job.spec);
     fft_y<-1>(p, job, 1, s);
     const dim3 gx((p.M * p.KP + PSE_FFT_TQ - 1) / PSE_FFT_TQ);
     k_fft_x<true><<<gx, PSE_FFT_TX, fft_smem_x(p.M), s>>>(p, job, with_noise);

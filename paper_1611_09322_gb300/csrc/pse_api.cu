@@ -52,6 +52,7 @@ struct pse_ctx {
     FftPlan fplan{};
     SpreadTile spread{};                                // spreading tile shape
     bool spread_ready = false, spread_tuned = false;
+    bool spread4 = false;                               // spreading by vector reductions instead of tiles (FP32)
     size_t spread_smem_max = 0;                         // dynamic shared memory the spreading may use
     int *sp_orig = nullptr;                             // block origin of each tile index (ncell + 1)
     int2 *sp_cover = nullptr;                           // M * PSE_COVER (tile, offset) pairs
@@ -527,11 +528,22 @@ template <typename T> pse_status set_spread_tile(pse_ctx *c, const SpreadTile &t
     return PSE_OK;
 }
 
-template <typename T>
-cudaError_t run_spread(pse_ctx *c, const SpreadTile &t, cudaStream_t s, const Rec<T> *src = nullptr) {
+// Spread the caller's forces (src null) or a sorted-order vector: by vector
+// reductions into the node-major grid, or by tiles into the planar grids.
+template <typename T> cudaError_t run_spread(pse_ctx *c, cudaStream_t s, const Rec<T> *src = nullptr) {
     Dev<T> &d = dev<T>(c);
+    if constexpr (sizeof(T) == 4) {
+        if (c->spread4) {
+            const cudaError_t e = launch_spread4(c->N, c->wf, d, src, s);
+            if (e == cudaSuccess && !c->own_fft) launch_grid_planar(c->wf, d, s);
+            return e;
+        }
+    }
+    const int64_t M = c->plan.M;
+    const cudaError_t e = cudaMemsetAsync(d.grid, 0, sizeof(T) * 3 * M * M * M, s);
+    if (e != cudaSuccess) return e;
     const bool tp = c->sp_two_phase;
-    return launch_spread<T>(wgeom<T>(c), geom<T>(c), t, c->sp_orig, tp ? c->sp_cover : nullptr,
+    return launch_spread<T>(wgeom<T>(c), geom<T>(c), c->spread, c->sp_orig, tp ? c->sp_cover : nullptr,
                             tp ? c->sp_cnt : nullptr, tp ? (T *)c->sp_scratch : nullptr, d, s, src);
 }
 
@@ -552,8 +564,11 @@ template <typename T> pse_status choose_spread(pse_ctx *c) {
         if (ok) break;
     }
     if (!ok) return PSE_ENOTSUPPORTED;
-    pse_status st = set_spread_tile<T>(c, c->spread);
-    if (st != PSE_OK) return st;
+    c->spread4 = want == 0 && sizeof(T) == 4 && dev<T>(c).grid4;
+    if (!c->spread4) {
+        const pse_status st = set_spread_tile<T>(c, c->spread);
+        if (st != PSE_OK) return st;
+    }
     c->spread_ready = true;
     return PSE_OK;
 }
@@ -676,9 +691,8 @@ pse_status wave_branch(pse_ctx *c, int64_t N, cudaStream_t s, int mode, cudaEven
             if (mode == GM_SAMPLE) {
                 launch_fft_sample(c->fplan, fft_job(c), 7, s);
             } else {
-                CK(cudaMemsetAsync(d.grid, 0, sizeof(float) * 3 * w.M * w.M * (size_t)w.M, s));
-                CK(run_spread<T>(c, c->spread, s));
-                launch_fft_forces(c->fplan, fft_job(c), d.grid, gm_noise(mode), s);
+                CK(run_spread<T>(c, s));
+                launch_fft_forces(c->fplan, fft_job(c), c->spread4 ? nullptr : d.grid, gm_noise(mode), s);
             }
             if (sorted) cudaStreamWaitEvent(s, sorted, 0);
             launch_interp<T>(N, w, geom<T>(c), d, s);
@@ -688,13 +702,10 @@ pse_status wave_branch(pse_ctx *c, int64_t N, cudaStream_t s, int mode, cudaEven
     if (mode == GM_SAMPLE && c->params.wave_noise == 0) {
         launch_wave_noise<T>(w, d.args, c->params.system, d.spec, s);
     } else {
-        const int64_t M3 = (int64_t)w.M * w.M * w.M;
-        if (mode == GM_SAMPLE) {
+        if (mode == GM_SAMPLE)
             launch_grid_noise<T>(w, d.args, c->params.system, d.grid, s);
-        } else {
-            CK(cudaMemsetAsync(d.grid, 0, sizeof(T) * 3 * M3, s));
-            CK(run_spread<T>(c, c->spread, s));
-        }
+        else
+            CK(run_spread<T>(c, s));
         CKF(cufftSetStream(c->fft_r2c, s));
         if constexpr (sizeof(T) == 4) {
             CKF(cufftExecR2C(c->fft_r2c, (cufftReal *)d.grid, (cufftComplex *)d.spec));
@@ -847,14 +858,12 @@ template <typename T> pse_status full_step(pse_ctx *c, cudaStream_t s, cudaGraph
     const int64_t N = c->N;
     Dev<T> &d = dev<T>(c);
     const WaveGeom<T> &w = wgeom<T>(c);
-    const int64_t M3 = (int64_t)w.M * w.M * w.M;
-    CK(cudaMemsetAsync(d.grid, 0, sizeof(T) * 3 * M3, s));
-    CK(run_spread<T>(c, c->spread, s, d.rec));
+    CK(run_spread<T>(c, s, d.rec));
     bool own = false;
     if constexpr (sizeof(T) == 4) {
         own = c->own_fft;
         if (own) {
-            launch_fft_forces(c->fplan, fft_job(c), d.grid, 0, s);
+            launch_fft_forces(c->fplan, fft_job(c), c->spread4 ? nullptr : d.grid, 0, s);
             launch_interp<T>(N, w, geom<T>(c), d, s);
         }
     }
@@ -1128,40 +1137,50 @@ pse_status full_impl(pse_ctx *c, int64_t N, const T *pos, uint64_t seed, uint64_
     return PSE_OK;
 }
 
-// Time every tile shape that fits (3 spreads each after one warm-up) on the
-// cell list of the current call and keep the fastest.
+// Time the vector reductions and every tile shape that fits (3 spreads each
+// after one warm-up) on the cell list of the current call and keep the fastest.
 template <typename T> pse_status tune_spread(pse_ctx *c, cudaStream_t s) {
-    Dev<T> &d = dev<T>(c);
-    const int64_t M3 = (int64_t)c->plan.M * c->plan.M * c->plan.M;
     cudaEvent_t e0, e1;
     CK(cudaEventCreate(&e0));
     CK(cudaEventCreate(&e1));
     float best = 1e30f;
     SpreadTile keep = c->spread;
+    bool keep4 = c->spread4;
+    auto time = [&] {  // the current form; true if it is the fastest so far
+        float ms = 0.f;
+        bool ok = true;
+        for (int rep = 0; rep < 4 && ok; ++rep) {
+            if (rep == 1) cudaEventRecord(e0, s);
+            ok = run_spread<T>(c, s) == cudaSuccess;
+        }
+        cudaEventRecord(e1, s);
+        if (!ok || cudaEventSynchronize(e1) != cudaSuccess) return false;
+        cudaEventElapsedTime(&ms, e0, e1);
+        if (ms >= best) return false;
+        best = ms;
+        return true;
+    };
+    if (c->spread4) time();
+    c->spread4 = false;
     for (int CP : {3, 1})
         for (int G : {4, 2, 1}) {
             SpreadTile t;
             if (!spread_tile(c->plan, G, CP, sizeof(T), c->spread_smem_max, &t)) continue;
             if (set_spread_tile<T>(c, t) != PSE_OK) continue;
-            float ms = 0.f;
-            bool ok = true;
-            for (int rep = 0; rep < 4 && ok; ++rep) {
-                if (rep == 1) cudaEventRecord(e0, s);
-                ok = cudaMemsetAsync(d.grid, 0, sizeof(T) * 3 * M3, s) == cudaSuccess &&
-                     run_spread<T>(c, t, s) == cudaSuccess;
-            }
-            cudaEventRecord(e1, s);
-            if (!ok || cudaEventSynchronize(e1) != cudaSuccess) continue;
-            cudaEventElapsedTime(&ms, e0, e1);
-            if (ms < best) {
-                best = ms;
+            if (time()) {
                 keep = t;
+                keep4 = false;
             }
         }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     cudaGetLastError();
     c->spread_tuned = true;
+    c->spread4 = keep4;
+    if (keep4) {
+        drop_graph(c);
+        return PSE_OK;
+    }
     return set_spread_tile<T>(c, keep);
 }
 

@@ -518,6 +518,11 @@ template <typename T> void launch_matvec_caller(int64_t N, const SampleArgs<T> *
 template <typename T> void launch_wave_noise(WaveGeom<T> w, const SampleArgs<T> *args, int system, void *spec,
                                              cudaStream_t s);
 template <typename T> void launch_interp(int64_t N, WaveGeom<T> w, Geom<T> g, const Dev<T> &d, cudaStream_t s);
+// FP32 spreading by vector reductions into the node-major grid (P in 3..10),
+// and its planar copy
+cudaError_t launch_spread4(int64_t N, const WaveGeom<float> &w, const Dev<float> &d, const Rec<float> *src,
+                           cudaStream_t s);
+void launch_grid_planar(const WaveGeom<float> &w, const Dev<float> &d, cudaStream_t s);
 // The sampler's own transforms (FP32; kernels_wave.cu): grid side, its factors
 // with their strides (products of the earlier ones) and division multipliers,
 // kz kept (no Nyquist plane) and padded row length of the spectrum, and the

@@ -212,3 +212,30 @@ def test_mobility_apply_symmetric_positive_at_full_size(torch):
     assert abs(a - b) < 1e-4 * abs(float((F.double() * MF).sum()))
     assert float((F.double() * MF).sum()) > 0 and float((Gv.double() * MG).sum()) > 0
     s.close()
+
+
+@pytest.mark.parametrize("P,M,N", [(3, 30, 1), (4, 32, 7), (5, 48, 33), (6, 48, 700), (7, 50, 2000), (8, 147, 2000),
+                                   (9, 50, 2001), (10, 150, 999)])
+def test_spread_by_reductions(torch, P, M, N):
+    """Spreading by vector reductions (the default) against the tile form
+    (spread_tile = 1) for every support, with cuFFT's and our transforms (M =
+    147, 150), partly filled warps, particles on the faces of the box and two
+    in one place.  Both add the same FP32 products in another order: 1e-5 is
+    over 10 times the rounding of a few hundred terms per node."""
+    rng = np.random.default_rng(P)
+    L = 30.0 if M < 100 else 60.0
+    pos = rng.uniform(0, L, (N, 3)).astype(np.float32)
+    pos[: N // 3, 0] = 0.0
+    if N > 5:
+        pos[5] = pos[4]
+        pos[6] = np.nextafter(np.float32(L), np.float32(0))
+    d, F = torch.from_numpy(pos).cuda(), torch.from_numpy(_forces(N, 2)).cuda()
+    outs = []
+    for tile in (0, 1):
+        s = _sampler(L, xi=0.5, tol=1e-2, grid_M=M, support_P=P, fixed_iter=2, spread_tile=tile)
+        outs.append([t.cpu().numpy() for t in (s.mobility_apply(d, F) - s.real_matvec(d, F),
+                                               s.sample_with_forces(d, F, SEED, 3, 0.5, 1.0),
+                                               s.sample_full_lanczos(d, SEED, 1))])
+        s.close()
+    for a, b in zip(*outs):
+        assert _maxrel(a, b) < 1e-5, _maxrel(a, b)
