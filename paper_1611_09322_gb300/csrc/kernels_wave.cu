@@ -909,8 +909,8 @@ cudaError_t launch_spread(WaveGeom<T> w, Geom<T> g, SpreadTile st, const int *or
 // transform of the forces path with the mode factor between the two passes
 // over x.  The transforms are bound by memory traffic; against noise kernel +
 // cuFFT C2R + node-major copy they save the noise's write and read and the
-// planar grids' (noise, x, y / z: M = 200 157 -> 139 / 138 -> 110 us, 189 158
-// -> 115 / 135 -> 92, 378 973 -> 1000 / 795 -> 511; fft_wins has the rule).
+// planar grids' (noise, x, y / z: M = 200 157 -> 139 / 138 -> 77 us, 189 158
+// -> 115 / 135 -> 66, 378 973 -> 1000 / 795 -> 511; fft_wins has the rule).
 //   x pass: tile of (y, kz) modes, three components: noise (or forward
 //           transform over x, mode factor, noise), inverse over x;
 //   y pass: per x, tile of kz, one component, in place;
@@ -933,7 +933,12 @@ constexpr int PSE_FFT_TY = 256;  // its threads
 constexpr int PSE_FFT_TR = 8;    // y rows per block of the z passes
 constexpr int PSE_FFT_NL = 3 * PSE_FFT_TR / 2;  // their complex lines
 constexpr int PSE_FFT_LS = PSE_FFT_NL + 2;      // room per point: the fill along kz meets 2-way bank conflicts
-constexpr int PSE_FFT_TT = 384;  // threads of the z passes
+// Threads of the z passes: a radix-8 pass has M / 8 butterflies on 6 pairs of
+// lines, so 384 threads are half idle on small grids while three or more
+// blocks of 192 fit an SM (us, 384 -> 192: M = 147 42 -> 33, 200 84 -> 77, 245
+// 145 -> 125, 294 260 -> 252); where two blocks fit, 192 are too few (375 554
+// -> 648).
+constexpr int PSE_FFT_TT_MANY = 384, PSE_FFT_TT_FEW = 192, PSE_FFT_FEW_MAXM = 300;
 
 __device__ __forceinline__ float2 cmulf(float2 a, float2 b) {
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
@@ -1257,10 +1262,11 @@ __global__ void __launch_bounds__(PSE_FFT_TY, 3) k_fft_y(const __grid_constant__
 }
 
 // Inverse z pass, blockIdx = (tile of y rows, x, species): spectrum rows -> node-major records.
-__global__ void __launch_bounds__(PSE_FFT_TT, 2) k_fft_z_inv(const __grid_constant__ FftPlan p,
+template <int T>
+__global__ void __launch_bounds__(T, 768 / T) k_fft_z_inv(const __grid_constant__ FftPlan p,
                                                           const float2 *__restrict__ spec,
                                                           V4<float> *__restrict__ grid4) {
-    constexpr int TR = PSE_FFT_TR, NL = PSE_FFT_NL, LS = PSE_FFT_LS, T = PSE_FFT_TT;
+    constexpr int TR = PSE_FFT_TR, NL = PSE_FFT_NL, LS = PSE_FFT_LS;
     extern __shared__ __align__(16) float2 fsm[];
     const int M = p.M, sp = blockIdx.z, H = M / 2, nkz = p.nkz;
     float2 *A = fsm, *B = A + M * LS, *tw = B + M * LS;
@@ -1321,9 +1327,10 @@ __global__ void __launch_bounds__(PSE_FFT_TT, 2) k_fft_z_inv(const __grid_consta
 
 // Forward z pass: real grids, planar or (grid4) node-major, -> spectrum rows
 // (kz < nkz).
-__global__ void __launch_bounds__(PSE_FFT_TT, 2) k_fft_z_fwd(const __grid_constant__ FftPlan p, const float *__restrict__ grid,
+template <int T>
+__global__ void __launch_bounds__(T, 768 / T) k_fft_z_fwd(const __grid_constant__ FftPlan p, const float *__restrict__ grid,
                                                           const V4<float> *__restrict__ grid4, float2 *__restrict__ spec) {
-    constexpr int TR = PSE_FFT_TR, NL = PSE_FFT_NL, LS = PSE_FFT_LS, T = PSE_FFT_TT;
+    constexpr int TR = PSE_FFT_TR, NL = PSE_FFT_NL, LS = PSE_FFT_LS;
     extern __shared__ __align__(16) float2 fsm[];
     const int M = p.M;
     float2 *A = fsm, *B = A + M * LS, *tw = B + M * LS;
@@ -1419,8 +1426,10 @@ cudaError_t fft_prepare() {
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_x<true>, attr, zx);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_y<1>, attr, zy);
     if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_y<-1>, attr, zy);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_z_inv, attr, zz);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_z_fwd, attr, zz);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_z_inv<PSE_FFT_TT_MANY>, attr, zz);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_z_inv<PSE_FFT_TT_FEW>, attr, zz);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_z_fwd<PSE_FFT_TT_MANY>, attr, zz);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_fft_z_fwd<PSE_FFT_TT_FEW>, attr, zz);
     return e;
 }
 
@@ -1448,7 +1457,10 @@ template <int S> static void fft_y(const FftPlan &p, const FftJob &job, int nspe
 }
 static void fft_z_inv(const FftPlan &p, const FftJob &job, int nspec, cudaStream_t s) {
     const dim3 grid((p.M + PSE_FFT_TR - 1) / PSE_FFT_TR, p.M, nspec);
-    k_fft_z_inv<<<grid, PSE_FFT_TT, fft_smem_z(p.M), s>>>(p, job.spec, job.grid4);
+    if (p.M <= PSE_FFT_FEW_MAXM)
+        k_fft_z_inv<PSE_FFT_TT_FEW><<<grid, PSE_FFT_TT_FEW, fft_smem_z(p.M), s>>>(p, job.spec, job.grid4);
+    else
+        k_fft_z_inv<PSE_FFT_TT_MANY><<<grid, PSE_FFT_TT_MANY, fft_smem_z(p.M), s>>>(p, job.spec, job.grid4);
 }
 // parts: bit 0 the x pass (with the noise), bit 1 the y pass, bit 2 the z pass
 void launch_fft_sample(const FftPlan &p, const FftJob &job, int parts, cudaStream_t s) {
@@ -1463,7 +1475,11 @@ void launch_fft_sample(const FftPlan &p, const FftJob &job, int parts, cudaStrea
 // node-major grid.
 void launch_fft_forces(const FftPlan &p, const FftJob &job, const float *grid, int with_noise, cudaStream_t s) {
     const dim3 gz((p.M + PSE_FFT_TR - 1) / PSE_FFT_TR, p.M);
-    k_fft_z_fwd<<<gz, PSE_FFT_TT, fft_smem_z(p.M), s>>>(p, grid, grid ? nullptr : job.grid4, job.spec);
+    const V4<float> *grid4 = grid ? nullptr : job.grid4;
+    if (p.M <= PSE_FFT_FEW_MAXM)
+        k_fft_z_fwd<PSE_FFT_TT_FEW><<<gz, PSE_FFT_TT_FEW, fft_smem_z(p.M), s>>>(p, grid, grid4, job.spec);
+    else
+        k_fft_z_fwd<PSE_FFT_TT_MANY><<<gz, PSE_FFT_TT_MANY, fft_smem_z(p.M), s>>>(p, grid, grid4, job.spec);
     fft_y<-1>(p, job, 1, s);
     const dim3 gx((p.M * p.KP + PSE_FFT_TQ - 1) / PSE_FFT_TQ);
     k_fft_x<true><<<gx, PSE_FFT_TX, fft_smem_x(p.M), s>>>(p, job, with_noise);
