@@ -706,6 +706,8 @@ void launch_batch_nbr(const BSys *sys, int nsys, int *const *tab, const int *nbl
 }
 
 // ------------------------------------------------------------------ exclusive scan
+#define PSE_SCAN_NT 8  // tiles of PSE_SCAN_ITEMS per block of the one-launch form
+#define PSE_SCAN_CLUSTER (PSE_CELLS_BLOCKS * PSE_SCAN_NT * PSE_SCAN_ITEMS)
 // Three passes: per-block scan of PSE_SCAN_ITEMS ints (1024 threads x 4),
 // a one-block scan of the block totals, then the carry-in add.
 __global__ void k_scan_block(const int *in, int *out, int64_t n, int *sums) {
@@ -762,6 +764,77 @@ __global__ void k_scan_add(int *out, int64_t n, const int *sums) {
     if (i < n) out[i] += sums[i / PSE_SCAN_ITEMS];
 }
 
+// The same scan by one cluster of 8 blocks with everything in registers, the
+// tiles of PSE_SCAN_ITEMS dealt to the blocks in consecutive runs of nt <= NT;
+// clears the search's counters too.  The work is a few microseconds of
+// latency either way, so a launch and its gap are what counts: three scan
+// launches and two clears -> one launch, samples of 1.6e4 particles 137 -> 124
+// us, 1e5 of two sizes 405 -> 383, Brownian step of 3e4 208 -> 198, forces of
+// 2e5 482 -> 473.  Up to the cell slots that the registers of a cluster hold.
+template <int NT>
+__global__ void __cluster_dims__(PSE_CELLS_BLOCKS, 1, 1) __launch_bounds__(1024)
+    k_scan_cluster(const int4 *__restrict__ in, int4 *__restrict__ out, int n, int nt, int *sums, int *overflow,
+                   unsigned long long *n_pairs) {
+    __shared__ int wsum[NT][32];
+    const int blk = blockIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int4 v[NT];
+    int tot[NT], inc[NT];
+    const int i0 = blk * nt * PSE_SCAN_ITEMS + 4 * threadIdx.x;
+#pragma unroll
+    for (int k = 0; k < NT; ++k) {
+        const int i = i0 + k * PSE_SCAN_ITEMS;
+        v[k] = k < nt && i < n ? __ldg(in + i / 4) : make_int4(0, 0, 0, 0);
+    }
+    if (blk == 0 && threadIdx.x == 0) {
+        *overflow = 0;
+        *n_pairs = 0ull;
+    }
+#pragma unroll
+    for (int k = 0; k < NT; ++k) inc[k] = tot[k] = v[k].x + v[k].y + v[k].z + v[k].w;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1)
+#pragma unroll
+        for (int k = 0; k < NT; ++k) {
+            const int u = __shfl_up_sync(0xffffffffu, inc[k], o);
+            if (lane >= o) inc[k] += u;
+        }
+    if (lane == 31)
+#pragma unroll
+        for (int k = 0; k < NT; ++k) wsum[k][wid] = inc[k];
+    __syncthreads();
+    if (wid < NT) {
+        int w = wsum[wid][lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, w, o);
+            if (lane >= o) w += u;
+        }
+        wsum[wid][lane] = w;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int t = 0;
+#pragma unroll
+        for (int k = 0; k < NT; ++k) t += wsum[k][31];
+        sums[blk] = t;
+    }
+    cluster_sync();
+    int base = 0;
+    for (int b = 0; b < blk; ++b) base += __ldcg(sums + b);
+#pragma unroll
+    for (int k = 0; k < NT; ++k) {
+        const int i = i0 + k * PSE_SCAN_ITEMS;
+        int4 r;
+        r.x = base + inc[k] - tot[k] + (wid ? wsum[k][wid - 1] : 0);
+        r.y = r.x + v[k].x;
+        r.z = r.y + v[k].y;
+        r.w = r.z + v[k].z;
+        if (k < nt && i < n) out[i / 4] = r;
+        base += wsum[k][31];
+    }
+    if (blk == PSE_CELLS_BLOCKS - 1 && threadIdx.x == 0) reinterpret_cast<int *>(out)[n] = base;
+}
+
 int num_sms() {
     static int n = 0;
     if (n == 0) {
@@ -775,11 +848,24 @@ int num_sms() {
     return n;
 }
 
-void launch_scan(const int *in, int *out, int64_t n, int *sums, cudaStream_t s) {
+int scan_launches(int64_t n) { return n <= PSE_SCAN_CLUSTER && n % 4 == 0 ? 1 : 3; }
+static void launch_scan(const int *in, int *out, int64_t n, int *sums, LzState *lz, cudaStream_t s) {
     const int nb = (int)((n + PSE_SCAN_ITEMS - 1) / PSE_SCAN_ITEMS);
+    if (scan_launches(n) == 1) {
+        const int nt = (nb + PSE_CELLS_BLOCKS - 1) / PSE_CELLS_BLOCKS;
+        auto go = [&](auto kernel) {
+            kernel<<<PSE_CELLS_BLOCKS, 1024, 0, s>>>((const int4 *)in, (int4 *)out, (int)n, nt, sums, &lz->overflow,
+                                                     &lz->n_pairs);
+        };
+        if (nt <= 1) go(k_scan_cluster<1>);
+        else go(k_scan_cluster<PSE_SCAN_NT>);
+        return;
+    }
     if (nb > 0) k_scan_block<<<nb, 1024, 0, s>>>(in, out, n, sums);
     k_scan_sums<<<1, 1024, 0, s>>>(sums, nb, out + n);
     if (n > 0) k_scan_add<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(out, n, sums);
+    cudaMemsetAsync(&lz->overflow, 0, sizeof(int), s);
+    cudaMemsetAsync(&lz->n_pairs, 0, sizeof(unsigned long long), s);
 }
 
 // ------------------------------------------------------------------ launchers
@@ -790,7 +876,7 @@ void launch_bin(int64_t N, const SampleArgs<T> *args, Geom<T> g, const Dev<T> &d
     const int64_t nc3 = cell_slots(g.nc);
     cudaMemsetAsync(d.cell_count, 0, sizeof(int) * nc3, s);
     k_bin<T><<<nblk(N, 256), 256, 0, s>>>(N, args, g, d.cell_of, d.slot, d.cell_count);
-    launch_scan(d.cell_count, d.cell_start, nc3, d.scan_sums, s);
+    launch_scan(d.cell_count, d.cell_start, nc3, d.scan_sums, d.lz, s);
 }
 
 template <typename T>
@@ -822,8 +908,6 @@ void launch_cells(int64_t N, const SampleArgs<T> *args, Geom<T> g, const Dev<T> 
     launch_bin<T>(N, args, g, d, s);
     launch_scatter<T>(N, args, g, d, s);
     launch_place<T>(N, args, g, d, s);
-    cudaMemsetAsync(&d.lz->overflow, 0, sizeof(int), s);
-    cudaMemsetAsync(&d.lz->n_pairs, 0, sizeof(unsigned long long), s);
 }
 
 template <typename T> void launch_nbr(int64_t N, Geom<T> g, const Dev<T> &d, cudaStream_t s) {

@@ -40,6 +40,8 @@ struct NoAllocScratch {
     SampleArgs<float> args;
     LzState lz;
 };
+// the scan moves four at a time
+static_assert(offsetof(NoAllocScratch, cell_count) % 16 == 0 && offsetof(NoAllocScratch, cell_start) % 16 == 0);
 
 }  // namespace
 }  // namespace pse

@@ -1670,14 +1670,12 @@ pse_status pse_profile_stages(pse_ctx *c, int64_t N, const float *d_pos, uint64_
         launches[stage] += nl;
         return PSE_OK;
     };
-    const int nscan = 3;
+    const int nscan = scan_launches(c->ncell3);
     pse_status r = PSE_OK;
     if (r == PSE_OK) r = timed(PSE_STAGE_CELLS, 1 + nscan, [&] { launch_bin<float>(N, d.args, c->gf, d, s); return PSE_OK; });
     if (r == PSE_OK) r = timed(PSE_STAGE_SORT, 2, [&] {
         launch_scatter<float>(N, d.args, c->gf, d, s);
         launch_place<float>(N, d.args, c->gf, d, s);
-        cudaMemsetAsync(&d.lz->overflow, 0, sizeof(int), s);
-        cudaMemsetAsync(&d.lz->n_pairs, 0, sizeof(unsigned long long), s);
         return PSE_OK; });
     // our transforms: noise with the passes over x and y, then the one over z
     // that writes the node-major grid; with wave_fft = 1 (M = 64, 256) the

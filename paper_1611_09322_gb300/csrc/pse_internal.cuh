@@ -426,7 +426,7 @@ int num_sms();
 // cells / scan / neighbour list
 template <typename T> void launch_bin(int64_t N, const SampleArgs<T> *args, Geom<T> g, const Dev<T> &d,
                                       cudaStream_t s);
-void launch_scan(const int *in, int *out, int64_t n, int *sums, cudaStream_t s);
+int scan_launches(int64_t n);
 template <typename T> void launch_scatter(int64_t N, const SampleArgs<T> *args, Geom<T> g, const Dev<T> &d,
                                           cudaStream_t s);
 template <typename T>

@@ -459,9 +459,10 @@ def test_fp64_stored_pair_blocks(torch, N):
 
 @pytest.mark.parametrize("N,L,kind", [(1, 20.0, "u"), (3, 20.0, "u"), (700, 14.0, "u"), (9999, 60.0, "clump"),
                                       (10000, 60.0, "clump"), (10001, 45.0, "u"), (8192, 50.0, "clump"),
-                                      (8193, 40.0, "u"), (2000, 300.0, "u"), (69999, 90.0, "u")])
+                                      (8193, 40.0, "u"), (2000, 300.0, "u"), (69999, 90.0, "u"), (2000, 340.0, "u"), (2000, 350.0, "u")])
 def test_neighbour_search_lane_groups(torch, N, L, kind):
-    """The one-launch cell list (up to 8192 particles and 65536 cell slots)
+    """The one-launch cell list (up to 8192 particles and 65536 cell slots),
+    the one-launch scan (up to 262144 slots, L = 340; three launches at 350)
     and the searches with 27 and 9 lanes per particle, at the sizes where one
     takes over from the other, in boxes of 2 and more cells per side and with
     a clump that puts over 32 particles in one cell: the near-field product is
