@@ -1282,33 +1282,58 @@ __global__ void k_det_final(int64_t N, const SampleArgs<T> *args, const V4<T> *p
 // Overlap repulsion F_s = k_rep sum_t (2a - r) rhat over the list entries of
 // s closer than 2a (pair vectors from cell-local offsets, as in the matvec),
 // plus the external force, written in caller order.
-template <typename T>
+// TPP lanes per particle take every TPP-th entry, four of them in flight.
+// Bound by the latency of entry -> offsets: one entry at a time took 25 us at
+// 3e4 particles, on a step's critical path.  Steps in us (one lane and one
+// entry; 1, 4 and 16 lanes with four): 3e4 particles 198; 184, 179, 183, FP64
+// 1e3 -; 257, 235, 233, 1e5 -; 314, 312, 323, 3e5 -; 835, 836, 868, 1e6 -;
+// 2233, 2259, 2396: four lanes up to PSE_REP_LANES, one above.
+#define PSE_REP_LANES 200000
+template <typename T, int TPP>
 __global__ void k_repulsion(int64_t N, Geom<T> g, const SampleArgs<T> *args, const V4<T> *__restrict__ loc,
                             const int *__restrict__ count, const int *__restrict__ nbr,
                             const V4<T> *__restrict__ pos_sorted, T *F) {
-    const int64_t s = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (s >= N) return;
+    constexpr int U = 4;
+    const int64_t t = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int sub = (int)(t & (TPP - 1));
+    const int64_t s = t / TPP < N ? t / TPP : N - 1;  // the last groups past the end repeat particle N - 1
     const V4<T> li = loc[s];
     const T two_a = T(2) * g.a, k = (T)args->k_rep;
     T fx = 0, fy = 0, fz = 0;
     const int cnt = count[s];
-    for (int q = 0; q < cnt; ++q) {
-        const int e = nbr[(int64_t)q * N + s];
-        if (e < 0) continue;  // a pair removed by the float64 decision at r_cut
-        const V4<T> lt = loc[e >> 6];
-        const int ox = ((e >> 4) & 3) - 1, oy = ((e >> 2) & 3) - 1, oz = (e & 3) - 1;
-        const T dx = (li.x - lt.x) - (T(ox) * g.cs + T(ox) * g.cs_lo);
-        const T dy = (li.y - lt.y) - (T(oy) * g.cs + T(oy) * g.cs_lo);
-        const T dz = (li.z - lt.z) - (T(oz) * g.cs + T(oz) * g.cs_lo);
-        const T r2 = dx * dx + dy * dy + dz * dz;
-        if (r2 < two_a * two_a && r2 > T(0)) {
-            const T r = sqrt_hd(r2);
-            const T f = k * (two_a - r) / r;
-            fx += f * dx;
-            fy += f * dy;
-            fz += f * dz;
+    for (int q0 = sub; q0 < cnt; q0 += U * TPP) {
+        int e[U];
+        V4<T> l[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int q = q0 + u * TPP;
+            e[u] = q < cnt ? nbr[(int64_t)q * N + s] : -1;  // -1: removed by the float64 decision at r_cut
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) l[u] = loc[e[u] < 0 ? s : e[u] >> 6];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int ox = ((e[u] >> 4) & 3) - 1, oy = ((e[u] >> 2) & 3) - 1, oz = (e[u] & 3) - 1;
+            const T dx = (li.x - l[u].x) - (T(ox) * g.cs + T(ox) * g.cs_lo);
+            const T dy = (li.y - l[u].y) - (T(oy) * g.cs + T(oy) * g.cs_lo);
+            const T dz = (li.z - l[u].z) - (T(oz) * g.cs + T(oz) * g.cs_lo);
+            const T r2 = dx * dx + dy * dy + dz * dz;
+            if (e[u] >= 0 && r2 < two_a * two_a && r2 > T(0)) {
+                const T r = sqrt_hd(r2);
+                const T f = k * (two_a - r) / r;
+                fx += f * dx;
+                fy += f * dy;
+                fz += f * dz;
+            }
         }
     }
+#pragma unroll
+    for (int o = TPP / 2; o; o >>= 1) {
+        fx += __shfl_xor_sync(0xffffffffu, fx, o);
+        fy += __shfl_xor_sync(0xffffffffu, fy, o);
+        fz += __shfl_xor_sync(0xffffffffu, fz, o);
+    }
+    if (sub || t / TPP >= N) return;
     const int64_t o = 3 * w_bits_r(pos_sorted[s].w);
     if (args->fext) {
         fx += args->fext[o];
@@ -1655,7 +1680,11 @@ void launch_lz_final_forces(int64_t N, const SampleArgs<T> *args, const Dev<T> &
                                              sizeof(T) == 4 ? d.pc_on : nullptr, d.udet);
 }
 template <typename T> void launch_repulsion(int64_t N, Geom<T> g, const Dev<T> &d, cudaStream_t s) {
-    k_repulsion<T><<<nb(N, 128), 128, 0, s>>>(N, g, d.args, d.loc_sorted, d.nbr_count, d.nbr, d.pos_sorted, d.bd_force);
+    auto go = [&](auto kernel, int tpp) {
+        kernel<<<nb(N * tpp, 128), 128, 0, s>>>(N, g, d.args, d.loc_sorted, d.nbr_count, d.nbr, d.pos_sorted, d.bd_force);
+    };
+    if (N < PSE_REP_LANES) go(k_repulsion<T, 4>, 4);
+    else go(k_repulsion<T, 1>, 1);
 }
 template <typename T> void launch_advance(int64_t N, Geom<T> g, const Dev<T> &d, cudaStream_t s) {
     k_advance<T><<<nb(3 * N, 256), 256, 0, s>>>(N, g, d.args);

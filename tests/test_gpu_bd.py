@@ -103,3 +103,26 @@ def test_bd_trajectory_diffuses(torch):
     free = 6 * (1.0 / (6 * math.pi)) * dt * steps
     assert free / 3 < msd < 1.05 * free, (msd, free)
     s.close()
+
+
+@pytest.mark.parametrize("N", [1, 2, 33, 1000, 199999, 200000])
+def test_repulsion_lane_groups(torch, N):
+    """The deterministic step (kT = 0) is dt times the product of the oracle's
+    repulsion, with four lanes and one per particle, odd and full last groups:
+    a jittered lattice with every neighbour overlapping (r > 1.3 a), so the
+    FP32 pair vectors are good to 1e-6 and the product to 1e-4, as above."""
+    from oracle import pse
+    from paper_1611_09322_gb300 import Sampler
+    n = max(8, math.ceil(N ** (1 / 3)))
+    L = 1.9 * n
+    rng = np.random.default_rng(N)
+    idx = np.arange(N)
+    pos = (np.stack([idx // (n * n), idx // n % n, idx % n], 1) + 0.5) * 1.9 + rng.uniform(-0.2, 0.2, (N, 3))
+    pos = pos.astype(np.float32)
+    F = pse.repulsion_forces(pos, L, 1.0, 3.0)
+    s = Sampler(L, 1.0, xi=0.7, tol=1e-3)
+    d = torch.from_numpy(pos).cuda()
+    ref = 1e-2 * s.mobility_apply(d, torch.from_numpy(F.astype(np.float32)).cuda()).cpu().numpy()
+    s.bd_step(d, SEED, 1, 1e-2, 0.0, 3.0)
+    _close(_wrapdiff(d.cpu().numpy().astype(np.float64), pos.astype(np.float64), L), ref, 1e-4, L, np.float32)
+    s.close()
