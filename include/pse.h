@@ -541,8 +541,8 @@ pse_status pse_real_matvec_noalloc(double L, double a, double xi, double tol, in
  * xi, cut-offs and grid); one pse_batch_sample is ONE CUDA graph launch whose
  * kernels each work for all systems at once (a block -> system table): cell
  * lists, neighbour lists, q_1, the wave noise and interpolation, and in the
- * device-side loop the near-field matvec, the Lanczos update and the FP64
- * eigen-solves; systems that converge drop out of the loop.  The inverse
+ * device-side loop the near-field matvec and the Lanczos update with the
+ * FP64 T_j^{1/2} e_1; systems that converge drop out of the loop.  The inverse
  * FFTs run as one batched cuFFT call per grid size: each system's grid is
  * raised to the next size of a fixed list (16, 20, 24, 28, 32, 40, 48, ...,
  * a finer grid only lowers the NUFFT error), so systems share sizes.

@@ -2,8 +2,8 @@
 // search the paper's real-space sum uses, Sec. III), sm_103a.
 //
 // Particles are binned into ncell^3 cells of side >= r_cut (ids in 4x4x4
-// brick-major order), counting-sorted into cell order (deterministic: ties in a cell are ordered by caller
-// index), and every sorted particle gets an ELL list of the particles within
+// brick-major order), counting-sorted into cell order (deterministic: ties in
+// a cell are ordered by caller index), and every sorted particle gets an ELL list of the particles within
 // r_cut.  Each entry packs the neighbour's sorted index with the 3x3x3
 // stencil offset of its cell, so pair vectors are formed from cell-local
 // offsets: d = (l_i - l_t) - dc * cs, accurate to a few float ulps of the

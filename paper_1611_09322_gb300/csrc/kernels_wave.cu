@@ -1,7 +1,8 @@
 // Wave-space sample M_w^{1/2} dW2 (Sec. II B 2): complex Hermitian noise,
 // B^{1/2} scaling with the Gaussian deconvolution, inverse FFT (three passes
-// of our own in FP32, else cuFFT C2R launched by the host), and Gaussian interpolation S^dagger = h^3 S^T at the
-// particles.  sm_103a.
+// of our own where fft_wins says so, else cuFFT C2R launched by the host), and
+// Gaussian interpolation S^dagger = h^3 S^T at the particles; the forces
+// path's spreading and forward transform.  sm_103a.
 //
 // Per mode k = 2 pi n / L of the half spectrum (nz >= 0):
 //   vhat(k) = V^{-1/2} sinc(ka)/k sqrt(1 + k^2/4xi^2) exp(-(1 - eta) k^2 / 8xi^2)
@@ -272,8 +273,8 @@ __device__ __forceinline__ int wrap_grid(int i, int M) {  // valid for i in [-M,
 // interpolation (the Gaussian's constant is applied in the mode factor).
 //
 // FP64, the planar interpolation and a tile asked for: one CTA per tile of
-// G^3 cells (FP32 with the node-major grid: k_spread4).  The tile's particles (cell-sorted, so each
-// cell is a contiguous run) are spread into a padded E^3 node block in shared
+// G^3 cells (FP32 with the node-major grid: k_spread4).  The tile's particles
+// (cell-sorted, so each cell is a contiguous run) are spread into a padded E^3 node block in shared
 // memory with shared-memory atomics, CP components per pass.  The block
 // starts at the node orig[t] of each axis (host-computed: the support start of
 // the tile's lower corner less one node) and E bounds the support of every

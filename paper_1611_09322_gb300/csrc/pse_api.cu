@@ -2,17 +2,18 @@
 // graph and the entry points.
 //
 // One sample is one graph launch.  The graph forks after the cell sort:
-//   real branch:  neighbour list -> WHILE { matvec -> update -> eig(T_j) }
-//   wave branch:  k-space noise -> cuFFT C2R (x3) -> interpolation
+//   real branch:  neighbour list -> WHILE { matvec -> update and T_j^{1/2} e_1 }
+//   wave branch:  k-space noise -> inverse FFT (x3) -> interpolation
 // and joins in the final combination kernel.  The Lanczos loop runs on the
-// device: after the matvec and update of step j, the eigen kernel (FP64, one
-// warp) solves T_j, runs the stop test and sets the WHILE node's condition,
-// so the host never waits inside a sample.  Per-call arguments (pointers,
+// device: a block of step j's update computes T_j^{1/2} e_1 in FP64, runs the
+// stop test and sets the WHILE node's condition, so the host never waits
+// inside a sample.  Per-call arguments (pointers,
 // seed, sample index) live in a small device struct refreshed by one copy
 // before launch.  The forces path (c_det M F + c_noise M^{1/2} z) adds M_r F
-// on the real branch before the loop, and its wave branch spreads F, runs
-// cuFFT R2C, applies the deterministic mode factor with the k-space noise
-// fused in, then C2R and interpolation.
+// on the real branch before the loop, and its wave branch spreads F,
+// transforms forward, applies the deterministic mode factor with the k-space
+// noise fused in, then transforms back and interpolates.  The transforms are
+// ours (kernels_wave.cu) or cuFFT's.
 #include <math.h>
 #include <stdlib.h>
 #include <string.h>
@@ -730,8 +731,7 @@ pse_status wave_branch(pse_ctx *c, int64_t N, cudaStream_t s, int mode, cudaEven
 // Capture pieces of one sample.  The prologue runs on c->s_main (which must
 // be capturing): cell list, wave branch forked onto c->s_wave, neighbour
 // list, preconditioner blocks and q_1.  The loop body is one Lanczos step
-// (matvec -> update -> eigen-solve of T_j, all on `sa`).  The
-// epilogue joins the wave branch and writes the output.
+// (matvec -> update with T_j^{1/2} e_1, both on `sa`).  The epilogue joins the wave branch and writes the output.
 // The list-free matvec (FP32 monodisperse sampling without preconditioner)
 // needs no neighbour list: the sample then builds none.
 template <typename T> bool nolist_sample(pse_ctx *c, int mode) {
@@ -825,8 +825,7 @@ static cudaError_t add_while(cudaStream_t s, cudaGraphConditionalHandle *h, cuda
 }
 
 // One whole sample on c->s_main (capturing): prologue, a WHILE node whose
-// body is one Lanczos step with the eigen kernel setting the condition, and
-// the epilogue.
+// body is one Lanczos step whose update sets the condition, and the epilogue.
 template <typename T> pse_status capture_sample(pse_ctx *c, int mode) {
     const pse_status wst = capture_pre<T>(c, mode);
     if (!gm_noise(mode)) {
@@ -853,7 +852,7 @@ template <typename T> pse_status capture_sample(pse_ctx *c, int mode) {
 // (spread from the matvec records, forward FFT, the deterministic mode
 // factor of Sec. III, inverse FFT, interpolation into uwave), then the
 // near-field matvec with uwave added to its rows (so alpha_j = q_j . M q_j),
-// the three-term update and the eigen-solve with the stop test.
+// the three-term update with T_j^{1/2} e_1 and the stop test.
 template <typename T> pse_status full_step(pse_ctx *c, cudaStream_t s, cudaGraphConditionalHandle h) {
     const int64_t N = c->N;
     Dev<T> &d = dev<T>(c);
