@@ -119,11 +119,12 @@ typedef struct {
                             (default) the transforms of the wave part are this
                             library's (the noise drawn inside the first pass,
                             the last one writing the node-major grid of the
-                            interpolation) on grids of 145 <= M < 490 that are
-                            no power of two, above M = 245 only where M^3 is
-                            at least 10 times the particles (30 above 375),
-                            and cuFFT's elsewhere: the faster ones of the two
-                            beside the near field.  1: also on M = 64 and 256 */
+                            interpolation) on grids of 126 <= M < 490 other
+                            than 144 and powers of two, above M = 245 only
+                            where M^3 is at least 10 times the particles (30
+                            above 375), and cuFFT's elsewhere: the faster ones
+                            of the two beside the near field.  1: also on M =
+                            64 and 256                                       */
 } pse_params;
 
 /* Parameters derived from (L, a, xi, tol) by Sec. II C of the paper:

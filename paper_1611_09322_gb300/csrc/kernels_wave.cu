@@ -1438,17 +1438,19 @@ cudaError_t fft_prepare() {
 // copy, from whole samples and forces calls both ways (random spheres, xi a =
 // 0.52, us, cuFFT -> ours): M = 147 355 -> 319, 189 637 -> 529, 200 at phi
 // 0.05 451 -> 374, 294 2609 -> 1935, 375 5020 -> 4160; forces 147 752 -> 662,
-// 245 3169 -> 2640.  Below 145 a sample waits for the near field either way
-// and forces lose (M = 100 250 -> 291, 128 429 -> 464).  cuFFT's transforms
-// of powers of two are as fast (256: 249 us against 255 for noise, x and y)
-// and its shorter blocks yield sooner to the near field's one-wave kernels
+// 245 3169 -> 2640; with the z passes in blocks of 192 also M = 126 363 -> 316,
+// 135 433 -> 368, 140 446 -> 406 (their samples 172 -> 152, 172 -> 160 at phi
+// 0.03), not 144 (394 -> 417, sample 275 -> 289).  Below 126 neither side wins
+// throughout (forces M = 98 230 -> 209, 100 209 -> 216, 125 298 -> 307; samples
+// wait for the near field).  cuFFT's transforms of powers of two are as fast
+// (256: 249 us against 255 for noise, x and y) and its shorter blocks yield sooner to the near field's one-wave kernels
 // (256: 1212 -> 1293, 512: 9970 -> 11160).  The same delay outweighs the gain
 // above 245 in dense systems (M = 288: phi 0.25, M^3 / N = 6.7, 4788 -> 5143;
 // phi 0.15, 11, 2514 -> 2555; phi 0.05, 34, 1194 -> 1041), above 375 sooner
 // (378: 17, 4258 -> 4392; 34, 2562 -> 2395), and from 490 everywhere (34: 490
 // 5943 -> 6182, 486 7315 -> 5389): one block of the x pass per SM.
 bool fft_wins(int M, int nspec, int64_t N) {
-    if (M < 145 || M >= 490 || (M & (M - 1)) == 0) return false;
+    if (M < 126 || M == 144 || M >= 490 || (M & (M - 1)) == 0) return false;
     return M <= 245 || (double)M * M * M * nspec >= (M > 375 ? 30.0 : 10.0) * N;
 }
 

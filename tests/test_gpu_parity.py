@@ -482,7 +482,7 @@ def test_neighbour_search_lane_groups(torch, N, L, kind):
     assert _rel(got, ref) < 1e-5, _rel(got, ref)
 
 
-@pytest.mark.parametrize("M", [147, 150, 162, 175, 192, 245, 360, 486])
+@pytest.mark.parametrize("M", [126, 140, 147, 150, 162, 175, 192, 245, 360, 486])
 def test_own_transforms(torch, M):
     """Grids with the library's own transforms (odd, even, radices 2..9, two
     to four passes, M = 147 and 150 with ragged tiles in every pass): wave
