@@ -416,7 +416,8 @@ template <typename T> pse_status init_ctx(pse_ctx *c) {
     if ((st = alloc(c->per_ctx, (void **)&d.scan_sums, sizeof(int) * PSE_SCAN_ITEMS)) != PSE_OK) return st;
     if ((st = alloc(c->per_ctx, (void **)&d.pc_theta, sizeof(float) * PSE_PRECOND_NPARAM)) != PSE_OK) return st;
     c->pc_s0 = (float)(1.0 / sqrt(p.self_mobility));
-    // a grid whose transforms are ours at every N needs no cuFFT plan
+    // a grid whose transforms are ours at every N needs no cuFFT plan; where
+    // some N takes cuFFT's, the plan is made here and not in a sample's call
     if (!(c->may_own_fft && fft_wins((int)M, S, 1ll << 40)) && (st = ensure_c2r<T>(c)) != PSE_OK) return st;
     // The real-space chain (cell list, neighbour list, Lanczos loop) is the
     // sample's critical path and its persistent kernels size their grids to
@@ -581,14 +582,10 @@ template <typename T> pse_status ensure(pse_ctx *c, int64_t N) {
     cudaDeviceSynchronize();
     drop_graph(c);
     free_list(c->per_n);
+    c->N = 0;  // until every buffer is there again
     if (c->params.matvec_shape == 0 && !c->mv_tuned) geom<T>(c).mv = default_matvec_shape<T>(c->plan, N);
     const bool asked = c->params.wave_fft == 1 && (c->plan.M == 64 || c->plan.M == 256);
     c->own_fft = c->may_own_fft && (asked || fft_wins(c->plan.M, c->nspec > 1 ? c->nspec : 1, N));
-    if (!c->own_fft) {
-        const pse_status st = ensure_c2r<T>(c);
-        if (st != PSE_OK) return st;
-    }
-    c->N = 0;
     Dev<T> &d = dev<T>(c);
     const pse_plan_info &p = c->plan;
     const int64_t nc3 = cell_slots(p.ncell);

@@ -1,0 +1,82 @@
+"""Host code of the library over a stand-in for the CUDA runtime and cuFFT
+(fake_cuda.c, preloaded in a child process): what is freed and allocated when
+a call fails half-way, and which kernels a call launches.  No GPU is used."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+PRELUDE = """
+import ctypes, sys
+sys.path.insert(0, %r)
+from paper_1611_09322_gb300 import _lib
+lib = _lib.load()
+fake = ctypes.CDLL(None)
+fake.fake_mallocs.restype = fake.fake_live.restype = fake.fake_launches.restype = ctypes.c_long
+fake.fake_cost.argtypes = [ctypes.c_char_p, ctypes.c_double]
+P = ctypes.c_void_p(64)  # kernels do not run: no position is read
+
+def params(**kw):
+    p = _lib.pse_params()
+    p.tol, p.use_graph = 1e-3, -1
+    for k, v in kw.items():
+        setattr(p, k, v)
+    return p
+
+def create(L, **kw):
+    c = ctypes.c_void_p()
+    st = lib.pse_create_ex(ctypes.byref(c), L, 1.0, ctypes.byref(params(**kw)))
+    assert st == 0, st
+    return c
+
+def launches(name):
+    return fake.fake_launches(name.encode())
+""" % ROOT
+
+
+@pytest.fixture(scope="module")
+def child(tmp_path_factory):
+    from paper_1611_09322_gb300 import build
+    build.build_cuda()
+    so = str(tmp_path_factory.mktemp("fake") / "libfake.so")
+    subprocess.run(["gcc", "-O1", "-shared", "-fPIC", os.path.join(HERE, "fake_cuda.c"), "-o", so], check=True)
+
+    def run(body):
+        script = str(tmp_path_factory.mktemp("case") / "case.py")
+        with open(script, "w") as f:
+            f.write(PRELUDE + body)
+        r = subprocess.run([sys.executable, script], env=dict(os.environ, LD_PRELOAD=so), cwd=ROOT,
+                           capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, r.stdout + r.stderr
+    return run
+
+
+def test_failed_call_at_another_n_frees_no_buffer_in_use(child):
+    """A call at a new N that fails after the old N's buffers were freed, at
+    any of its allocations, leaves nothing behind: the next call at the old N
+    allocates again.  On a 250^3 grid, where few particles take the library's
+    own transforms and many cuFFT, the plan is made with the context: no later
+    call depends on it."""
+    child("""
+c = ctypes.c_void_p()
+fake.fake_fail_plans(1)
+assert lib.pse_create_ex(ctypes.byref(c), 250.0, 1.0, ctypes.byref(params(xi=0.5, grid_M=250))) == 4
+c = create(250.0, xi=0.5, grid_M=250)
+few, many = 1000, 3_000_000
+assert lib.pse_sample(c, few, P, 1, 1, P, None) == 0 and launches("k_fft_x") == 1
+live = fake.fake_live()
+for k in (1, 2, 5, 15, 25):
+    fake.fake_fail_malloc(k)
+    assert lib.pse_sample(c, many, P, 1, 1, P, None) == 2
+    fake.fake_reset()
+    assert lib.pse_sample(c, few, P, 1, 1, P, None) == 0
+    assert fake.fake_mallocs() > 20 and fake.fake_live() == live
+fake.fake_fail_plans(1)
+fake.fake_reset()
+assert lib.pse_sample(c, many, P, 1, 1, P, None) == 0 and launches("k_fft_x") == 0
+lib.pse_destroy(c)
+""")
