@@ -62,6 +62,7 @@ struct pse_ctx {
     size_t sp_scratch_bytes = 0;
     bool sp_two_phase = false;
     bool mv_tuned = false;                              // matvec launch shape timed
+    bool mv_list = false;                               // a list shape was the faster one (FP64: no stored pair blocks)
     cudaStream_t last_stream = nullptr;
     void *stage_pos = nullptr, *stage_out = nullptr;  // device staging for the host-buffer call
     // pipelined host-buffer calls: two staging pairs, a copy stream, and per
@@ -639,7 +640,7 @@ template <typename T> pse_status ensure(pse_ctx *c, int64_t N) {
     d.pair = nullptr;
     d.pent = nullptr;
     d.pair_cols = 0;
-    d.use_pair = sizeof(T) == 8 && c->params.matvec_shape == 0;
+    d.use_pair = sizeof(T) == 8 && c->params.matvec_shape == 0 && !c->mv_list;
     d.want_rec = false;
     if (d.use_pair) {
         const double mean = (double)N * 4.18879020478639 * p.r_cut * p.r_cut * p.r_cut / (p.L * p.L * p.L);
@@ -1047,9 +1048,10 @@ template <typename T> pse_status tune_matvec(pse_ctx *c, cudaStream_t s) {
             cudaEventElapsedTime(&ms, e0, e1);
             best = ms < best ? ms : best;
         }
-        if (best >= t[keep]) d.use_pair = false;
-        else keep = geom<T>(c).mv;
+        if (best < t[keep]) keep = geom<T>(c).mv;
+        else d.use_pair = false;
     }
+    c->mv_list = !stored(d);  // the choice stands when N changes
     geom<T>(c).mv = keep;
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);

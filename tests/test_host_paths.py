@@ -80,3 +80,22 @@ fake.fake_reset()
 assert lib.pse_sample(c, many, P, 1, 1, P, None) == 0 and launches("k_fft_x") == 0
 lib.pse_destroy(c)
 """)
+
+
+@pytest.mark.parametrize("stored_ms,list_ms", [(0.5, 1.0), (1.0, 0.5)])
+def test_timed_fp64_product_is_kept_at_another_n(child, stored_ms, list_ms):
+    """autotune bit 2 in FP64 times the stored pair blocks against the list
+    shapes once per context; the choice holds at every later N."""
+    want = (1, 1, 1) if stored_ms < list_ms else (1, 0, 0)  # products, stored ones, pair evaluations
+    child(f"""
+c = create(40.0, xi=0.5, precision=1, autotune=4)
+fake.fake_cost(b"k_lz_matvec", {list_ms})
+fake.fake_cost(b"k_lz_matvec_stored", {stored_ms})
+for N in (1000, 2000, 1000):
+    assert lib.pse_sample_f64(c, N, P, 1, 1, P, None, None, None) == 0
+    fake.fake_reset()
+    assert lib.pse_sample_f64(c, N, P, 1, 2, P, None, None, None) == 0
+    n = launches("k_lz_matvec"), launches("k_lz_matvec_stored"), launches("k_pairs")
+    assert n == {want}, (N, n)
+lib.pse_destroy(c)
+""")
