@@ -476,8 +476,10 @@ pse_status pse_precond_blocks(pse_ctx *ctx, int64_t N, const float *d_pos, float
 /* Stage indices of pse_profile_stages (the paper's Fig. gel split: real-space
  * matvecs, other Lanczos work, FFT + scaling + RNG, spreading/interpolation). */
 enum {
-    PSE_STAGE_CELLS = 0,      /* binning + cell scan                         */
-    PSE_STAGE_SORT,           /* scatter into cell order + per-cell sort      */
+    PSE_STAGE_CELLS = 0,      /* binning + cell scan (up to 8192 particles
+                                 and 65536 cells: the whole cell list)       */
+    PSE_STAGE_SORT,           /* scatter into cell order + per-cell sort (0
+                                 where one launch makes the cell list)       */
     PSE_STAGE_REAL_NOISE,     /* z1 and ||z1||                                */
     PSE_STAGE_NEIGHBOURS,     /* neighbour count, scan, fill                  */
     PSE_STAGE_MATVEC,         /* M_r q_j, all iterations                      */

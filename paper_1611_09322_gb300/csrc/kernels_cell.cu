@@ -895,11 +895,13 @@ template <typename T, int Q> static void nbr_coop(const Geom<T> &g, const NbrArg
     const int64_t blocks = (groups + warps - 1) / warps, most = (int64_t)num_sms() * 32;
     k_nbr_coop<T, Q><<<(unsigned)(blocks < most ? blocks : most), PSE_NBR_THREADS, 0, s>>>(g, a);
 }
+// Whether one launch makes the whole cell list.
+bool cells_few(int64_t N, int nc) { return N <= PSE_CELLS_FEW && cell_slots(nc) <= PSE_CELLS_SLOTS; }
 // The whole cell list, and the search's counters cleared.
 template <typename T>
 void launch_cells(int64_t N, const SampleArgs<T> *args, Geom<T> g, const Dev<T> &d, cudaStream_t s) {
     const int64_t nc3 = cell_slots(g.nc);
-    if (N <= PSE_CELLS_FEW && nc3 <= PSE_CELLS_SLOTS) {
+    if (cells_few(N, g.nc)) {
         k_cells_few<T><<<PSE_CELLS_BLOCKS, PSE_CELLS_THREADS, 0, s>>>(
             (int)N, args, g, (int)nc3, d.cell_count, d.cell_start, d.perm, d.scan_sums, d.pos_sorted, d.loc_sorted,
             d.rec, &d.lz->overflow, &d.lz->n_pairs);
@@ -910,6 +912,8 @@ void launch_cells(int64_t N, const SampleArgs<T> *args, Geom<T> g, const Dev<T> 
     launch_place<T>(N, args, g, d, s);
 }
 
+// FP32 launches of launch_nbr.
+int nbr_launches(int64_t N) { return N < PSE_NBR_COOP ? 1 : 2; }
 template <typename T> void launch_nbr(int64_t N, Geom<T> g, const Dev<T> &d, cudaStream_t s) {
     if (N < PSE_NBR_COOP) {
         const NbrArgs<T> a{N, d.loc_sorted, d.pos_sorted, d.cell_start, d.nbr_count, d.nbr, nbr_k(N, d.nbr_cap),

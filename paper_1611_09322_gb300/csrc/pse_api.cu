@@ -1668,10 +1668,13 @@ pse_status pse_profile_stages(pse_ctx *c, int64_t N, const float *d_pos, uint64_
         launches[stage] += nl;
         return PSE_OK;
     };
-    const int nscan = scan_launches(c->ncell3);
+    const bool few = cells_few(N, c->gf.nc);  // cells and sort in one launch
     pse_status r = PSE_OK;
-    if (r == PSE_OK) r = timed(PSE_STAGE_CELLS, 1 + nscan, [&] { launch_bin<float>(N, d.args, c->gf, d, s); return PSE_OK; });
-    if (r == PSE_OK) r = timed(PSE_STAGE_SORT, 2, [&] {
+    if (r == PSE_OK) r = timed(PSE_STAGE_CELLS, few ? 1 : 1 + scan_launches(c->ncell3), [&] {
+        if (few) pre<float>(c, N, s);
+        else launch_bin<float>(N, d.args, c->gf, d, s);
+        return PSE_OK; });
+    if (r == PSE_OK && !few) r = timed(PSE_STAGE_SORT, 2, [&] {
         launch_scatter<float>(N, d.args, c->gf, d, s);
         launch_place<float>(N, d.args, c->gf, d, s);
         return PSE_OK; });
@@ -1707,7 +1710,7 @@ pse_status pse_profile_stages(pse_ctx *c, int64_t N, const float *d_pos, uint64_
             return PSE_OK; });
     if (r == PSE_OK)
         r = timed(PSE_STAGE_INTERP, 1, [&] { launch_interp<float>(N, c->wf, c->gf, c->df, s); return PSE_OK; });
-    if (r == PSE_OK) r = timed(PSE_STAGE_NEIGHBOURS, 1, [&] {
+    if (r == PSE_OK) r = timed(PSE_STAGE_NEIGHBOURS, nbr_launches(N), [&] {
         launch_nbr<float>(N, c->gf, d, s);
         return PSE_OK; });
     if (r == PSE_OK) r = timed(PSE_STAGE_REAL_NOISE, c->pc_enabled ? 2 : 1, [&] {

@@ -427,6 +427,8 @@ int num_sms();
 template <typename T> void launch_bin(int64_t N, const SampleArgs<T> *args, Geom<T> g, const Dev<T> &d,
                                       cudaStream_t s);
 int scan_launches(int64_t n);
+bool cells_few(int64_t N, int nc);
+int nbr_launches(int64_t N);
 template <typename T> void launch_scatter(int64_t N, const SampleArgs<T> *args, Geom<T> g, const Dev<T> &d,
                                           cudaStream_t s);
 template <typename T>

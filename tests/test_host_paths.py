@@ -99,3 +99,27 @@ for N in (1000, 2000, 1000):
     assert n == {want}, (N, n)
 lib.pse_destroy(c)
 """)
+
+
+@pytest.mark.parametrize("N,M", [(1000, 48), (8192, 147), (8193, 48), (69999, 48), (70000, 64)])
+def test_stage_timer_launches_what_a_sample_does(child, N, M):
+    """pse_profile_stages: the kernels of pse_sample, each counted in a stage,
+    with the one-launch cell list (up to 8192 particles) and without it, with
+    cuFFT and with the library's own transforms."""
+    child(f"""
+N, M = {N}, {M}
+names = ["k_cells_few", "k_bin", "k_scan", "k_scatter", "k_place", "k_fft", "k_wave_noise", "k_grid_aos", "k_interp",
+         "k_nbr", "k_lz_init", "k_lz_matvec", "k_lz_update", "k_lz_final"]
+c = create(60.0, xi=0.5, grid_M=M)
+assert lib.pse_sample(c, N, P, 1, 1, P, None) == 0
+fake.fake_reset()
+assert lib.pse_sample(c, N, P, 1, 1, P, None) == 0
+sample = [launches(n) for n in names]
+assert sum(sample) == launches("k_"), sample
+fake.fake_reset()
+ms, nl = (ctypes.c_double * len(_lib.STAGES))(), (ctypes.c_int * len(_lib.STAGES))()
+assert lib.pse_profile_stages(c, N, P, 1, 1, P, ms, nl, None) == 0
+assert [launches(n) for n in names] == sample, dict(zip(names, sample))
+assert sum(nl) == launches("k_"), dict(zip(_lib.STAGES, nl))
+lib.pse_destroy(c)
+""")
