@@ -403,7 +403,8 @@ def kernel_roofline(stages, N, M, n_pairs, peak, interp_kernel="k_interp4"):
     interp_bytes = 16 * N + (16 if interp_kernel == "k_interp4" else 12) * M ** 3 + 16 * N
     per_kernel = {
         "matvec": ("k_lz_matvec", matvec_bytes(N, n_pairs)),
-        "neighbours": ("k_nbr", 16 * N + 4 * n_pairs + 4 * N),
+        # (two launches from 7e4 particles on: the search and its float64 decisions at r_cut)
+        "neighbours": ("k_nbr", (16 * N + 4 * n_pairs + 4 * N) // max(stages["neighbours"][1], 1)),
         "lanczos_update": ("k_lz_update", 80 * N),
         "interp": (interp_kernel, interp_bytes),
         "grid_copy": ("k_grid_aos", 28 * M ** 3),
