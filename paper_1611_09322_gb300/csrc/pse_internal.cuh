@@ -284,11 +284,12 @@ __device__ __forceinline__ float warp_sum_f(float v) {
 // 1/x and x^{-1/2} in FP64 for the scalar tails of the Lanczos kernels, where
 // one thread's chain of dependent FP64 operations is what is waited for: such
 // an operation takes ~70 cycles here and a compiled division ~3500.  Seed: the
-// FP32 approximation of the significand (relative error < 2^-22); one
-// third-order step, r (1 + e + e^2) with e = 1 - x r, or r (1 + e/2 + 3 e^2/8)
-// with e = 1 - x r^2 (the binomial series), leaves e^3 ~ 2^-66, so the result
-// is rounded to 1-2 ulp.  Zero, denormals, infinities and NaN take the
-// ordinary operations.
+// FP32 value at the rounded significand, off by at most 2^-23 (a correctly
+// rounded reciprocal) or 2^-22 + 2^-25 (rsqrtf: 2 ulp); one third-order step,
+// r (1 + e + e^2) with e = 1 - x r, or r (1 + e/2 + 3 e^2/8) with e = 1 - x r^2
+// (the binomial series), leaves below 2^-64.  1/x is then off by the last
+// rounding (0.51 ulp), x^{-1/2} by that of its residual too (1.1 ulp).  Zero,
+// denormals, infinities and NaN take the ordinary operations.
 __device__ __forceinline__ bool normal_f64(int hi) { return (unsigned)((hi & 0x7fffffff) - 0x00100000) < 0x7fe00000u; }
 __device__ __forceinline__ double rcp_f64(double x) {
     const int hi = __double2hiint(x), E = ((hi >> 20) & 0x7ff) - 1023;
