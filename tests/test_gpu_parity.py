@@ -431,15 +431,16 @@ def test_pipelined_host_buffers(torch):
     s.close()
 
 
-@pytest.mark.parametrize("N", [1, 5, 700, 15500])
+@pytest.mark.parametrize("N", [1, 5, 700, 15500, 60001])
 def test_fp64_stored_pair_blocks(torch, N):
     """FP64 products over stored pair blocks (matvec_shape 0) against the list
     form (shape 1): a dilute box with a clump whose lists run past the stored
-    columns, coincident pairs included, at the sizes of the two thread layouts.
+    columns, coincident pairs included, at the sizes of the three thread
+    layouts (16 lanes per particle, 4 from 15000 and 2 from 60000 on).
     The two evaluate the same blocks in another order of summation: 1e-12 is
     over 1000 times the rounding of lists of a few hundred pairs."""
     rng = np.random.default_rng(N)
-    L = 60.0
+    L = 60.0 if N < 60000 else 110.0
     pos = rng.uniform(0, L, (N, 3))
     m = min(N, 120)
     pos[:m] = 30.0 + rng.uniform(-1.2, 1.2, (m, 3))
