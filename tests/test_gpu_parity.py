@@ -483,13 +483,24 @@ def test_neighbour_search_lane_groups(torch, N, L, kind):
     assert _rel(got, ref) < 1e-5, _rel(got, ref)
 
 
-@pytest.mark.parametrize("M", [126, 140, 147, 150, 162, 175, 192, 245, 360, 486])
+def _n_radices(M):
+    """Least number of factors 2..9 whose product is M."""
+    return 1 if M < 10 else 1 + min(_n_radices(M // r) for r in range(2, 10) if M % r == 0)
+
+
+def test_own_transform_sizes_have_two_to_four_radices():
+    assert [_n_radices(M) for M in (64, 126, 140, 147, 150, 162, 175, 192, 245, 250, 300, 360, 375, 486)] == \
+        [2] + 8 * [3] + [4, 4, 3, 4, 3]
+
+
+@pytest.mark.parametrize("M", [64, 126, 140, 147, 150, 162, 175, 192, 245, 250, 300, 360, 375, 486])
 def test_own_transforms(torch, M):
-    """Grids with the library's own transforms (odd, even, radices 2..9, two
-    to four passes, M = 147 and 150 with ragged tiles in every pass): wave
+    """Grids with the library's own transforms (odd, even, radices 2..9; two
+    passes at M = 64, where they are asked for, four at 250, 300 and 375, else
+    three; ragged tiles in every pass at M = 147 and 150): wave
     part of a sample, deterministic product and sample with forces against the
     planar form, which keeps cuFFT; two species of one radius (one grid each)
-    against the one-species wave part; the oracle at the two smallest.  1e-5
+    against the one-species wave part; the oracle up to M = 150.  1e-5
     is float rounding through transform and interpolation, as above."""
     from oracle import ewald, pse
     from paper_1611_09322_gb300 import PolySampler
@@ -498,21 +509,24 @@ def test_own_transforms(torch, M):
     d = torch.from_numpy(pos).cuda()
     F = torch.from_numpy(np.random.default_rng(M).standard_normal((N, 3)).astype(np.float32)).cuda()
     outs = []
+    asked = int(M == 64)
     for form in (0, 1):
-        s = _sampler(L, xi=0.5, tol=1e-3, grid_M=M, fixed_iter=3, interp_form=form)
+        s = _sampler(L, xi=0.5, tol=1e-3, grid_M=M, fixed_iter=3, interp_form=form, wave_fft=asked)
         w = s.sample(d, SEED, 11, parts=True)[2]
         det = s.mobility_apply(d, F) - s.real_matvec(d, F)
         outs.append([t.cpu().numpy() for t in (w, det, s.sample_with_forces(d, F, SEED, 5, 0.7, 1.3))])
         launches = s.profile_stages(d, SEED, 11)
         # noise with x and y, then z; the planar form has no node-major grid
-        assert (launches["wave_noise"][1], launches["grid_copy"][1]) == ((2, 1) if form == 0 else (1, 0))
+        # (asked for, y and z are the FFT stage)
+        assert (launches["wave_noise"][1], launches["grid_copy"][1]) == ((2 - asked, 1 - asked) if form == 0 else (1, 0))
         s.close()
     for a, b in zip(*outs):
         assert _maxrel(a, b) < 1e-5, _maxrel(a, b)
-    s = PolySampler(L, (1.0, 1.0), xi=0.5, tol=1e-3, grid_M=M, fixed_iter=3)
-    sp = (torch.arange(N, device="cuda") % 2).int()
-    assert _maxrel(s.sample(d, sp, SEED, 11, parts=True)[2].cpu().numpy(), outs[0][0]) < 1e-5
-    s.close()
+    if not asked:  # (two species refuse wave_fft = 1)
+        s = PolySampler(L, (1.0, 1.0), xi=0.5, tol=1e-3, grid_M=M, fixed_iter=3)
+        sp = (torch.arange(N, device="cuda") % 2).int()
+        assert _maxrel(s.sample(d, sp, SEED, 11, parts=True)[2].cpu().numpy(), outs[0][0]) < 1e-5
+        s.close()
     if M <= 150:
         plan = ewald.plan(L, 1.0, 0.5, 1e-3, M=M)
         p64 = pos.astype(np.float64)
