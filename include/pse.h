@@ -117,14 +117,16 @@ typedef struct {
                             particle                                           */
     int wave_fft;        /* FP32 with k-space noise and interp_form 0: 0
                             (default) the transforms of the wave part are this
-                            library's (the noise drawn inside the first pass,
-                            the last one writing the node-major grid of the
-                            interpolation) on grids of 126 <= M < 490 other
-                            than 144 and powers of two, above M = 245 only
-                            where M^3 is at least 10 times the particles (30
-                            above 375), and cuFFT's elsewhere: the faster ones
-                            of the two beside the near field.  1: also on M =
-                            64 and 256                                       */
+                            library's (the noise drawn inside one of their
+                            passes, the last one writing the node-major grid of
+                            the interpolation) where they are the faster ones,
+                            and cuFFT's elsewhere.  Forces calls: on grids of
+                            126 <= M < 490 (162 if M is a product of 2 and 3)
+                            other than powers of two.  Samples: on the same
+                            grids up to M = 200; above, where the grid has at
+                            least 6 sites per particle (12 if M is a product
+                            of 2 and 3; 10 from M = 246 and 30 from 376 on).
+                            1: also on M = 64 and 256                        */
 } pse_params;
 
 /* Parameters derived from (L, a, xi, tol) by Sec. II C of the paper:

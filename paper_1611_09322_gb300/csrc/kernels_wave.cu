@@ -1,6 +1,6 @@
 // Wave-space sample M_w^{1/2} dW2 (Sec. II B 2): complex Hermitian noise,
 // B^{1/2} scaling with the Gaussian deconvolution, inverse FFT (three passes
-// of our own where fft_wins says so, else cuFFT C2R launched by the host), and
+// of our own where fft_wins_* says so, else cuFFT C2R launched by the host), and
 // Gaussian interpolation S^dagger = h^3 S^T at the particles; the forces
 // path's spreading and forward transform.  sm_103a.
 //
@@ -911,7 +911,7 @@ cudaError_t launch_spread(WaveGeom<T> w, Geom<T> g, SpreadTile st, const int *or
 // over x.  The transforms are bound by memory traffic; against noise kernel +
 // cuFFT C2R + node-major copy they save the noise's write and read and the
 // planar grids' (noise, x, y / z: M = 200 157 -> 139 / 138 -> 77 us, 189 158
-// -> 115 / 135 -> 66, 378 973 -> 1000 / 795 -> 511; fft_wins has the rule).
+// -> 115 / 135 -> 66, 378 973 -> 1000 / 795 -> 511; fft_wins_* have the rule).
 //   x pass: tile of (y, kz) modes, three components: noise (or forward
 //           transform over x, mode factor, noise), inverse over x;
 //   y pass: per x, tile of kz, one component, in place;
@@ -1434,24 +1434,44 @@ cudaError_t fft_prepare() {
     return e;
 }
 
-// Where these transforms are faster than noise kernel + cuFFT + node-major
-// copy, from whole samples and forces calls both ways (random spheres, xi a =
-// 0.52, us, cuFFT -> ours): M = 147 355 -> 319, 189 637 -> 529, 200 at phi
-// 0.05 451 -> 374, 294 2609 -> 1935, 375 5020 -> 4160; forces 147 752 -> 662,
-// 245 3169 -> 2640; with the z passes in blocks of 192 also M = 126 363 -> 316,
-// 135 433 -> 368, 140 446 -> 406 (their samples 172 -> 152, 172 -> 160 at phi
-// 0.03), not 144 (394 -> 417, sample 275 -> 289).  Below 126 neither side wins
-// throughout (forces M = 98 230 -> 209, 100 209 -> 216, 125 298 -> 307; samples
-// wait for the near field).  cuFFT's transforms of powers of two are as fast
-// (256: 249 us against 255 for noise, x and y) and its shorter blocks yield sooner to the near field's one-wave kernels
-// (256: 1212 -> 1293, 512: 9970 -> 11160).  The same delay outweighs the gain
-// above 245 in dense systems (M = 288: phi 0.25, M^3 / N = 6.7, 4788 -> 5143;
-// phi 0.15, 11, 2514 -> 2555; phi 0.05, 34, 1194 -> 1041), above 375 sooner
-// (378: 17, 4258 -> 4392; 34, 2562 -> 2395), and from 490 everywhere (34: 490
-// 5943 -> 6182, 486 7315 -> 5389): one block of the x pass per SM.
-bool fft_wins(int M, int nspec, int64_t N) {
-    if (M < 126 || M == 144 || M >= 490 || (M & (M - 1)) == 0) return false;
-    return M <= 245 || (double)M * M * M * nspec >= (M > 375 ? 30.0 : 10.0) * N;
+// Where these transforms are faster than cuFFT's: a whole call both ways, in
+// turn, on every grid size without prime factors above 7 from 96 to 500 and at
+// M^3 / N = 57, 17, 8.5 and 4.2 (lattices of spheres, xi a = 0.52), cuFFT over
+// ours, so above 1 where ours win.
+// Sizes: from M = 126 on for sizes with a factor 5 or 7 (samples at 17, forces
+// at 17: M = 120 1.00, 1.01; 125 1.00, 0.95; 126 0.97, 1.14; 135 1.00, 1.16;
+// 147 1.15, 1.30; 200 1.14, 1.15; 245 1.27, 1.35); from 162 on without, since
+// cuFFT is at its best on small products of 2 and 3 (96 0.98, 1.01; 108 0.92,
+// 0.99; 128 1.00, 0.97; 144 0.96, 0.95; 162 1.12, 1.19; 192 1.04, 1.05); not
+// powers of two (256 0.96, 1.00); up to 486 (480 1.02, 1.04; 486 1.20, 1.26;
+// 490 0.97, 0.97; 500 0.93, 0.92: an empirical line).
+static bool fft_sizes(int M) {
+    int m = M;
+    while (m % 2 == 0) m /= 2;
+    const bool pow2 = m == 1;
+    while (m % 3 == 0) m /= 3;
+    return M >= (m == 1 ? 162 : 126) && M < 490 && !pow2;
+}
+// Forces: at every density (at 4.2: M = 147 1.04, 189 1.04, 243 1.01, 245 1.07,
+// 288 1.03, 294 1.08, 343 1.01; their transforms are the longer branch).
+bool fft_wins_forces(int M) { return fft_sizes(M); }
+// Samples: in dense systems the near field is the longer branch, and while
+// blocks of our passes are resident its one-wave kernels wait for them longer
+// than for cuFFT's shorter blocks.  Below M = 200 that is within the spread of
+// sizes at any density (at 4.2: 162 1.02, 168 0.98, 189 1.03, 196 1.00); above,
+// ours lose at 4.2 (216 0.98, 225 0.96, 240 0.98, 243 0.96, 250 0.96, 288
+// 0.92) and, on products of 2 and 3, at 8.5 (216 0.96, 243 0.96, 288 0.93, 324
+// 0.99; other sizes 210 1.06, 225 1.00, 245 1.09, 250 0.98, 270 0.96, 294
+// 1.14, 336 1.04); at 17 they win up to 375 (243 1.01, 252 1.09, 294 1.34, 324
+// 1.05, 375 1.21) and are even above (378 0.99, 384 1.02, 405 1.16, 420 0.99),
+// at 34 everywhere (378 1.09, 420 1.11, 480 1.04).
+bool fft_wins_sample(int M, int nspec, int64_t N) {
+    if (!fft_sizes(M)) return false;
+    int m = M;
+    while (m % 2 == 0) m /= 2;
+    while (m % 3 == 0) m /= 3;
+    const double per = (double)M * M * M * nspec / N, most = m == 1 ? 12.0 : 6.0;
+    return M <= 200 || per >= (M > 375 ? 30.0 : (M > 245 && most < 10.0 ? 10.0 : most));
 }
 
 template <int S> static void fft_y(const FftPlan &p, const FftJob &job, int nspec, cudaStream_t s) {

@@ -49,7 +49,7 @@ struct pse_ctx {
     cufftHandle fft_r2c = 0;                            // forward FFT (spreading / grid noise)
     bool r2c_made = false;
     bool may_own_fft = false;                           // our transforms can stand in for cuFFT's (FP32)
-    bool own_fft = false;                               // and do, at this N
+    bool own_sample = false, own_fft = false;           // and do in samples of this N, in forces calls
     FftPlan fplan{};
     SpreadTile spread{};                                // spreading tile shape
     bool spread_ready = false, spread_tuned = false;
@@ -313,6 +313,14 @@ static FftJob fft_job(const pse_ctx *c) {
     return FftJob{c->wf, c->df.args, c->params.system, (float2 *)c->df.spec, c->df.grid4};
 }
 
+// Whether the transforms of samples of N particles are ours.
+static bool asked_own(const pse_ctx *c) {
+    return c->params.wave_fft == 1 && (c->plan.M == 64 || c->plan.M == 256);
+}
+static bool own_transforms(const pse_ctx *c, int64_t N) {
+    return c->may_own_fft && (asked_own(c) || fft_wins_sample(c->plan.M, c->nspec > 1 ? c->nspec : 1, N));
+}
+
 // Inverse (C2R, batch 3) plan: spectrum -> planar grids.
 template <typename T> pse_status ensure_c2r(pse_ctx *c) {
     if (c->fft_made) return PSE_OK;
@@ -393,6 +401,7 @@ template <typename T> pse_status init_ctx(pse_ctx *c) {
             fft_prepare() == cudaSuccess) {
             if ((st = fft_twiddles(c->per_ctx, &c->fplan)) != PSE_OK) return st;
             c->may_own_fft = true;
+            c->own_fft = asked_own(c) || fft_wins_forces((int)M);
         }
         cudaGetLastError();
     }
@@ -419,7 +428,7 @@ template <typename T> pse_status init_ctx(pse_ctx *c) {
     c->pc_s0 = (float)(1.0 / sqrt(p.self_mobility));
     // a grid whose transforms are ours at every N needs no cuFFT plan; where
     // some N takes cuFFT's, the plan is made here and not in a sample's call
-    if (!(c->may_own_fft && fft_wins((int)M, S, 1ll << 40)) && (st = ensure_c2r<T>(c)) != PSE_OK) return st;
+    if (!own_transforms(c, 1ll << 40) && (st = ensure_c2r<T>(c)) != PSE_OK) return st;
     // The real-space chain (cell list, neighbour list, Lanczos loop) is the
     // sample's critical path and its persistent kernels size their grids to
     // the whole GPU: its streams get the highest priority and the wave
@@ -585,8 +594,7 @@ template <typename T> pse_status ensure(pse_ctx *c, int64_t N) {
     free_list(c->per_n);
     c->N = 0;  // until every buffer is there again
     if (c->params.matvec_shape == 0 && !c->mv_tuned) geom<T>(c).mv = default_matvec_shape<T>(c->plan, N);
-    const bool asked = c->params.wave_fft == 1 && (c->plan.M == 64 || c->plan.M == 256);
-    c->own_fft = c->may_own_fft && (asked || fft_wins(c->plan.M, c->nspec > 1 ? c->nspec : 1, N));
+    c->own_sample = own_transforms(c, N);
     Dev<T> &d = dev<T>(c);
     const pse_plan_info &p = c->plan;
     const int64_t nc3 = cell_slots(p.ncell);
@@ -686,7 +694,7 @@ pse_status wave_branch(pse_ctx *c, int64_t N, cudaStream_t s, int mode, cudaEven
     Dev<T> &d = dev<T>(c);
     const WaveGeom<T> &w = wgeom<T>(c);
     if constexpr (sizeof(T) == 4) {
-        if (c->own_fft) {
+        if (mode == GM_SAMPLE ? c->own_sample : c->own_fft) {
             if (mode == GM_SAMPLE) {
                 launch_fft_sample(c->fplan, fft_job(c), 7, s);
             } else {
@@ -1681,7 +1689,7 @@ pse_status pse_profile_stages(pse_ctx *c, int64_t N, const float *d_pos, uint64_
     // our transforms: noise with the passes over x and y, then the one over z
     // that writes the node-major grid; with wave_fft = 1 (M = 64, 256) the
     // last two passes are the FFT stage
-    const bool own = c->own_fft, split = own && c->params.wave_fft == 1 && (c->plan.M == 64 || c->plan.M == 256);
+    const bool own = c->own_sample, split = own && asked_own(c);
     const FftJob job = fft_job(c);
     if (r == PSE_OK) r = timed(PSE_STAGE_WAVE_NOISE, split ? 1 : (own || c->params.wave_noise ? 2 : 1), [&] {
         if (own) {

@@ -545,8 +545,11 @@ struct FftJob {
 };
 bool fft_plan(int M, FftPlan *p);
 cudaError_t fft_prepare();
-// whether they are the faster ones beside the near field of N particles
-bool fft_wins(int M, int nspec, int64_t N);
+// whether they are the faster ones: in forces calls and in full-mobility
+// Lanczos products; in samples, beside the near field of N particles (a
+// subset of the former's grids)
+bool fft_wins_forces(int M);
+bool fft_wins_sample(int M, int nspec, int64_t N);
 void launch_fft_sample(const FftPlan &p, const FftJob &job, int parts, cudaStream_t s);
 void launch_fft_forces(const FftPlan &p, const FftJob &job, const float *grid, int with_noise, cudaStream_t s);
 // resident blocks per SM of the FP32 4x4 matvec (its persistent grid is one wave of them)

@@ -88,7 +88,7 @@ int cudaLaunchKernel(const void *k, dim3 g, dim3 b, void **args, size_t smem, vo
     return __cudaLaunchKernel((void *)k, g, b, args, smem, s);
 }
 int cudaFuncSetAttribute(const void *f, int a, int v) { (void)f; (void)a; (void)v; return 0; }
-int cudaFuncGetAttributes(void *at, const void *f) { (void)f; memset(at, 0, 8); return 0; }
+int cudaFuncGetAttributes(void *at, const void *f) { (void)f; memset(at, 0, 64); return 0; }
 int cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const void *f, int b, size_t smem, unsigned fl) {
     (void)f; (void)b; (void)smem; (void)fl;
     *n = 2;
@@ -116,7 +116,11 @@ int cudaMemGetInfo(size_t *left, size_t *all) { *left = *all = (size_t)280 << 30
 /* ---- device, streams, events */
 int cudaGetDevice(int *d) { *d = 0; return 0; }
 int cudaSetDevice(int d) { (void)d; return 0; }
-int cudaDeviceGetAttribute(int *v, int a, int d) { (void)a; (void)d; *v = 152; return 0; }
+int cudaDeviceGetAttribute(int *v, int a, int d) { /* 97: shared memory per block (opt-in); else the SM count */
+    (void)d;
+    *v = a == 97 ? 232448 : 152;
+    return 0;
+}
 int cudaDeviceGetStreamPriorityRange(int *lo, int *hi) { *lo = 0; *hi = -5; return 0; }
 int cudaDeviceSynchronize(void) { return 0; }
 int cudaGetLastError(void) { return 0; }

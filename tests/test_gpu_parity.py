@@ -532,3 +532,27 @@ def test_own_transforms(torch, M):
         p64 = pos.astype(np.float64)
         assert _maxrel(outs[0][0], pse.wave_sample_grid(p64, plan, SEED, 11)) < 1e-4
         assert _maxrel(outs[0][1], pse.wave_apply_grid(F.cpu().numpy().astype(np.float64), p64, plan)) < 1e-4
+
+
+def test_cufft_samples_beside_own_forces(torch):
+    """A dense system on 216^3, whose samples take cuFFT and whose forces calls
+    the library's own transforms on the same buffers, calls of both kinds in
+    turn: against the planar form, which keeps cuFFT for both (1e-5 as above)."""
+    N, M = 900_000, 216
+    L = 293.0
+    g = torch.Generator(device="cuda").manual_seed(4)
+    d = torch.rand(N, 3, generator=g, device="cuda") * L
+    F = torch.randn(N, 3, generator=g, device="cuda")
+    outs = []
+    for form in (0, 1):
+        s = _sampler(L, xi=0.5, tol=1e-3, grid_M=M, fixed_iter=2, interp_form=form)
+        o = []
+        for k in range(2):
+            o += [s.sample(d, SEED, k, parts=True)[2], s.sample_with_forces(d, F, SEED, 7 + k, 0.7, 1.3),
+                  s.mobility_apply(d, F) - s.real_matvec(d, F)]
+        launches = s.profile_stages(d, SEED, 11)
+        assert (launches["wave_noise"][1], launches["grid_copy"][1]) == (1, 1 - form)
+        outs.append([t.cpu().numpy() for t in o])
+        s.close()
+    for a, b in zip(*outs):
+        assert _maxrel(a, b) < 1e-5, _maxrel(a, b)

@@ -123,3 +123,25 @@ assert [launches(n) for n in names] == sample, dict(zip(names, sample))
 assert sum(nl) == launches("k_"), dict(zip(_lib.STAGES, nl))
 lib.pse_destroy(c)
 """)
+
+
+# grid, its sites per particle, own transforms in samples, in forces calls
+@pytest.mark.parametrize("M,per,sample,forces", [
+    (64, 20, 0, 0), (125, 20, 0, 0), (126, 20, 1, 1), (126, 4, 1, 1), (128, 20, 0, 0), (140, 4, 1, 1), (144, 20, 0, 0),
+    (160, 4, 1, 1), (162, 4, 1, 1), (200, 4, 1, 1), (216, 8, 0, 1), (216, 13, 1, 1), (225, 4, 0, 1), (225, 8, 1, 1),
+    (245, 4, 0, 1), (245, 8, 1, 1), (250, 8, 0, 1), (250, 11, 1, 1), (256, 20, 0, 0), (288, 11, 0, 1), (288, 13, 1, 1),
+    (378, 20, 0, 1), (378, 31, 1, 1), (486, 31, 1, 1), (490, 40, 0, 0)])
+def test_rule_for_the_transforms(child, M, per, sample, forces):
+    """Which transforms samples and forces calls take, on both sides of every
+    line of the rule."""
+    child(f"""
+M, N = {M}, int({M} ** 3 / {per})
+c = create(1.2 * M, xi=0.4, grid_M=M, max_iter=4)
+fake.fake_reset()
+assert lib.pse_sample(c, N, P, 1, 1, P, None) == 0
+assert (launches("k_fft_"), launches("k_wave_noise")) == ((3, 0) if {sample} else (0, 1))
+fake.fake_reset()
+assert lib.pse_sample_with_forces(c, N, P, P, 1, 1, 1.0, 1.0, P, None) == 0
+assert (launches("k_fft_"), launches("k_wave_apply")) == ((5, 0) if {forces} else (0, 1))
+lib.pse_destroy(c)
+""")
