@@ -65,10 +65,14 @@ typedef struct {
     int use_graph;       /* >= 0 (default): one CUDA graph per sample with a
                             device-side Lanczos loop; -1: plain stream launches
                             with a host-side loop (one sync per iteration)      */
-    int autotune;        /* bit 0: time cuFFT C2R for every 2,3,5,7-smooth grid
-                            size in [M, 1.12 M] at creation and keep the fastest
-                            (a finer grid only lowers the NUFFT error); needs
-                            the GPU at pse_create_ex.  0: the Sec. II C grid.
+    int autotune;        /* bit 0: time the wave part (noise to grid, with the
+                            transforms that a sample of volume fraction 0.1
+                            takes; the library's own count 1.15 times, for
+                            their cost to the near field beside them) on every
+                            2,3,5,7-smooth grid size in [M, 1.12 M] at creation
+                            and keep the fastest (a finer grid only lowers the
+                            NUFFT error); needs the GPU at pse_create_ex.  0:
+                            the Sec. II C grid.
                             bit 1: time every form of the spreading (vector
                             reductions, tile shapes) at the first forces call
                             and keep the fastest.
@@ -204,8 +208,8 @@ pse_status pse_get_plan(const pse_ctx *ctx, pse_plan_info *out);
  *   t_real: time of the xi-dependent real-space work at xi0 (neighbour list
  *           and near-field matvecs; the neighbour count within r_cut ~ 1/xi
  *           grows as r_cut^d_f),
- *   t_wave: time of the xi-dependent wave-space work at xi0 (k-space noise
- *           and FFT, ~ xi^3 Fourier modes),
+ *   t_wave: time of the xi-dependent wave-space work at xi0 (k-space noise,
+ *           FFT and node-major copy, ~ xi^3 Fourier modes),
  *   d_f:    fractal dimension of the suspension in [1, 3] (3: hard spheres).
  * The minimiser of t_real (xi0/xi)^d_f + t_wave (xi/xi0)^3 is
  *   *xi_star = xi0 (d_f t_real / (3 t_wave))^(1/(d_f + 3)),
@@ -219,13 +223,14 @@ pse_status pse_xi_model(double xi0, double t_real, double t_wave, double d_f, do
 typedef struct {
     double xi_start;     /* p->xi (or 0.5 / a)                                  */
     double t_real, t_wave; /* xi-dependent stage times at xi_start, one staged
-                            sample: neighbour list + matvecs; noise + FFT      */
+                            sample: neighbour list + matvecs; noise, FFT and
+                            node-major copy                                    */
     double xi_model;     /* pse_xi_model(xi_start, t_real, t_wave, d_f)          */
     double xi_best;      /* fastest trial (xi_start on ties)                     */
     double ms_start, ms_best;
     int M_best;          /* its grid: create the sampler with xi = xi_best and
                             grid_M = M_best                                     */
-    int n_grids;         /* candidate grids whose FFT was timed                 */
+    int n_grids;         /* candidate grids whose wave part was timed           */
     int n_tried;         /* trials below; trial 0 is the start context          */
     double xi_tried[PSE_XI_TRIALS];
     double ms_tried[PSE_XI_TRIALS]; /* -1: unusable (list overflow, no
@@ -244,9 +249,10 @@ typedef struct {
  *      0.75 xi* and 1.35 xi* (at most PSE_XI_GRIDS).  On a fixed grid the wave
  *      part costs the same for every xi it admits while the real part shrinks
  *      as xi grows, so each grid is paired with the largest xi whose plan fits
- *      it (k_cut L / pi <= M, eta <= 1).  Each grid's cuFFT C2R is timed and
- *      its sample time predicted from the start context's stage times scaled
- *      by eq. work (real part ~ xi^-d_f, noise ~ M^3, FFT as timed).
+ *      it (k_cut L / pi <= M, eta <= 1).  Each grid's wave part is timed (as
+ *      for autotune bit 0, with the transforms that a sample of N takes) and
+ *      its sample time predicted: the start context's, with that wave part in
+ *      place of its own and the real part scaled by eq. work (~ xi^-d_f).
  *   3. The best predictions are timed as whole samples (up to seven), and the
  *      fastest trial, the start context included, is reported.
  * Every trial context is destroyed before the next is made; d_pos (3N

@@ -681,9 +681,43 @@ template <typename T> void real_setup(pse_ctx *c, int64_t N, cudaStream_t s) {
     launch_lz_init<T>(N, d.args, c->params.system, d, s);
 }
 
-template <typename T> void interp(pse_ctx *c, int64_t N, cudaStream_t s) {
-    launch_grid_copy<T>(wgeom<T>(c), dev<T>(c), s);
-    launch_interp<T>(N, wgeom<T>(c), geom<T>(c), dev<T>(c), s);
+// cuFFT's transforms: planar grids -> spectrum; spectrum -> planar grids and
+// their node-major copy (where the interpolation reads one).
+template <typename T> pse_status grid_to_spec(pse_ctx *c, cudaStream_t s) {
+    Dev<T> &d = dev<T>(c);
+    CKF(cufftSetStream(c->fft_r2c, s));
+    if constexpr (sizeof(T) == 4) CKF(cufftExecR2C(c->fft_r2c, (cufftReal *)d.grid, (cufftComplex *)d.spec));
+    else CKF(cufftExecD2Z(c->fft_r2c, (cufftDoubleReal *)d.grid, (cufftDoubleComplex *)d.spec));
+    return PSE_OK;
+}
+template <typename T> pse_status spec_to_grid(pse_ctx *c, cudaStream_t s) {
+    Dev<T> &d = dev<T>(c);
+    CKF(cufftSetStream(c->fft, s));
+    if constexpr (sizeof(T) == 4) CKF(cufftExecC2R(c->fft, (cufftComplex *)d.spec, (cufftReal *)d.grid));
+    else CKF(cufftExecZ2D(c->fft, (cufftDoubleComplex *)d.spec, (cufftDoubleReal *)d.grid));
+    launch_grid_copy<T>(wgeom<T>(c), d, s);
+    return PSE_OK;
+}
+
+// A sample's velocity grid in the form that its interpolation reads.
+template <typename T> pse_status sample_grid(pse_ctx *c, cudaStream_t s) {
+    Dev<T> &d = dev<T>(c);
+    const WaveGeom<T> &w = wgeom<T>(c);
+    if constexpr (sizeof(T) == 4) {
+        if (c->own_sample) {
+            launch_fft_sample(c->fplan, fft_job(c), 7, s);
+            return PSE_OK;
+        }
+    }
+    if (c->params.wave_noise == 0) {
+        launch_wave_noise<T>(w, d.args, c->params.system, d.spec, s);
+    } else {
+        launch_grid_noise<T>(w, d.args, c->params.system, d.grid, s);
+        const pse_status st = grid_to_spec<T>(c, s);
+        if (st != PSE_OK) return st;
+        launch_wave_apply<T>(w, d.args, c->params.system, d.spec, WAVE_MODE_GRIDNOISE, 1, s);
+    }
+    return spec_to_grid<T>(c, s);
 }
 
 // The wave branch on `s`.  `sorted` (may be null): an event the
@@ -693,42 +727,23 @@ template <typename T>
 pse_status wave_branch(pse_ctx *c, int64_t N, cudaStream_t s, int mode, cudaEvent_t sorted = nullptr) {
     Dev<T> &d = dev<T>(c);
     const WaveGeom<T> &w = wgeom<T>(c);
-    if constexpr (sizeof(T) == 4) {
-        if (mode == GM_SAMPLE ? c->own_sample : c->own_fft) {
-            if (mode == GM_SAMPLE) {
-                launch_fft_sample(c->fplan, fft_job(c), 7, s);
-            } else {
-                CK(run_spread<T>(c, s));
-                launch_fft_forces(c->fplan, fft_job(c), c->spread4 ? nullptr : d.grid, gm_noise(mode), s);
-            }
-            if (sorted) cudaStreamWaitEvent(s, sorted, 0);
-            launch_interp<T>(N, w, geom<T>(c), d, s);
-            return PSE_OK;
-        }
-    }
-    if (mode == GM_SAMPLE && c->params.wave_noise == 0) {
-        launch_wave_noise<T>(w, d.args, c->params.system, d.spec, s);
+    pse_status st = PSE_OK;
+    if (mode == GM_SAMPLE) {
+        st = sample_grid<T>(c, s);
     } else {
-        if (mode == GM_SAMPLE)
-            launch_grid_noise<T>(w, d.args, c->params.system, d.grid, s);
-        else
-            CK(run_spread<T>(c, s));
-        CKF(cufftSetStream(c->fft_r2c, s));
+        CK(run_spread<T>(c, s));
+        bool own = false;
         if constexpr (sizeof(T) == 4) {
-            CKF(cufftExecR2C(c->fft_r2c, (cufftReal *)d.grid, (cufftComplex *)d.spec));
-        } else {
-            CKF(cufftExecD2Z(c->fft_r2c, (cufftDoubleReal *)d.grid, (cufftDoubleComplex *)d.spec));
+            own = c->own_fft;
+            if (own) launch_fft_forces(c->fplan, fft_job(c), c->spread4 ? nullptr : d.grid, gm_noise(mode), s);
         }
-        launch_wave_apply<T>(w, d.args, c->params.system, d.spec,
-                             mode == GM_SAMPLE ? WAVE_MODE_GRIDNOISE : WAVE_MODE_DET, gm_noise(mode), s);
+        if (!own) {
+            if ((st = grid_to_spec<T>(c, s)) != PSE_OK) return st;
+            launch_wave_apply<T>(w, d.args, c->params.system, d.spec, WAVE_MODE_DET, gm_noise(mode), s);
+            st = spec_to_grid<T>(c, s);
+        }
     }
-    CKF(cufftSetStream(c->fft, s));
-    if constexpr (sizeof(T) == 4) {
-        CKF(cufftExecC2R(c->fft, (cufftComplex *)d.spec, (cufftReal *)d.grid));
-    } else {
-        CKF(cufftExecZ2D(c->fft, (cufftDoubleComplex *)d.spec, (cufftDoubleReal *)d.grid));
-    }
-    launch_grid_copy<T>(w, d, s);
+    if (st != PSE_OK) return st;
     if (sorted) cudaStreamWaitEvent(s, sorted, 0);
     launch_interp<T>(N, w, geom<T>(c), d, s);
     return PSE_OK;
@@ -867,27 +882,15 @@ template <typename T> pse_status full_step(pse_ctx *c, cudaStream_t s, cudaGraph
     bool own = false;
     if constexpr (sizeof(T) == 4) {
         own = c->own_fft;
-        if (own) {
-            launch_fft_forces(c->fplan, fft_job(c), c->spread4 ? nullptr : d.grid, 0, s);
-            launch_interp<T>(N, w, geom<T>(c), d, s);
-        }
+        if (own) launch_fft_forces(c->fplan, fft_job(c), c->spread4 ? nullptr : d.grid, 0, s);
     }
     if (!own) {
-        CKF(cufftSetStream(c->fft_r2c, s));
-        if constexpr (sizeof(T) == 4) {
-            CKF(cufftExecR2C(c->fft_r2c, (cufftReal *)d.grid, (cufftComplex *)d.spec));
-        } else {
-            CKF(cufftExecD2Z(c->fft_r2c, (cufftDoubleReal *)d.grid, (cufftDoubleComplex *)d.spec));
-        }
+        pse_status st = grid_to_spec<T>(c, s);
+        if (st != PSE_OK) return st;
         launch_wave_apply<T>(w, d.args, c->params.system, d.spec, WAVE_MODE_DET, 0, s);
-        CKF(cufftSetStream(c->fft, s));
-        if constexpr (sizeof(T) == 4) {
-            CKF(cufftExecC2R(c->fft, (cufftComplex *)d.spec, (cufftReal *)d.grid));
-        } else {
-            CKF(cufftExecZ2D(c->fft, (cufftDoubleComplex *)d.spec, (cufftDoubleReal *)d.grid));
-        }
-        interp<T>(c, N, s);
+        if ((st = spec_to_grid<T>(c, s)) != PSE_OK) return st;
     }
+    launch_interp<T>(N, w, geom<T>(c), d, s);
     Dev<T> da = d;
     da.mv_add = d.uwave;
     da.want_rec = true;  // the next step spreads q_{j+1} from the records
@@ -1280,68 +1283,81 @@ static int smooth_2357(int n) {
     return n == 1;
 }
 
-// Device time (ms) of one cuFFT C2R (batch 3) on each grid Ms[i], the mean of
-// 3 transforms after one warm-up; 1e30 where no plan or memory was had.
-template <typename T> void time_fft_sizes(const int *Ms, int n, float *ms_out) {
-    int Mmax = 0;
+pse_status create_impl(pse_ctx **out, double L, double a, const pse_params *p, int nspec = 0,
+                       const double *radii = nullptr);
+
+// Device time (ms) of a sample's wave part on c's grid, from the noise to the
+// grid that the interpolation reads, with the transforms that a sample of N
+// particles takes there: the mean of 3 passes after one warm-up.  Our passes
+// count for PSE_OWN_BESIDE times their time alone:
+// in a sample they delay the near field more than cuFFT's blocks do.  Whole
+// samples on every smooth grid in [M0, 1.12 M0], M0 = 48 .. 375 at volume
+// fractions 0.05, 0.1 and 0.3 (66 systems): the grid taken is slower than the
+// best one by 0.6% on average (at most 5.6%) at a factor of 1, 0.4% at 1.05 and
+// 1.1, 0.3% (5.1%) at 1.15 and 1.2, 0.45% (15%) at 1.3; by cuFFT's C2R alone
+// 1.8% (19%).
+#define PSE_OWN_BESIDE 1.15f
+template <typename T> pse_status time_wave(pse_ctx *c, int64_t N, float *ms) {
+    c->own_sample = own_transforms(c, N);
+    if (c->params.wave_noise == 1) {
+        const pse_status st = ensure_r2c<T>(c);
+        if (st != PSE_OK) return st;
+    }
+    SampleArgs<T> a{};
+    a.c_noise = 1.0;
+    cudaStream_t s = c->s_main;
+    CK(push_args(c, dev<T>(c).args, &a, sizeof(a), s));
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    pse_status st = cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess ? PSE_OK : PSE_ECUDA;
+    for (int rep = 0; rep < 4 && st == PSE_OK; ++rep) {
+        if (rep == 1) cudaEventRecord(e0, s);
+        st = sample_grid<T>(c, s);
+    }
+    if (st == PSE_OK) {
+        cudaEventRecord(e1, s);
+        if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(ms, e0, e1) != cudaSuccess) st = PSE_ECUDA;
+        *ms *= (c->own_sample ? PSE_OWN_BESIDE : 1.f) / 3.f;
+    }
+    if (e0) cudaEventDestroy(e0);
+    if (e1) cudaEventDestroy(e1);
+    return st;
+}
+// The same on each grid Ms[i], by a context of its own (splitting xis[i], or
+// p's if xis is null); 1e30 where none could be made.
+void time_wave_grids(double L, double a, const pse_params &p, int nspec, const double *radii, int64_t N,
+                     const int *Ms, const double *xis, int n, float *ms_out) {
     for (int i = 0; i < n; ++i) {
         ms_out[i] = 1e30f;
-        if (Ms[i] > Mmax) Mmax = Ms[i];
-    }
-    const size_t cbytes = sizeof(T) * 2 * 3 * (size_t)Mmax * Mmax * (Mmax / 2 + 1);
-    const size_t rbytes = sizeof(T) * 3 * (size_t)Mmax * Mmax * Mmax;
-    void *spec = nullptr, *grid = nullptr;
-    if (cudaMalloc(&spec, cbytes) != cudaSuccess || cudaMalloc(&grid, rbytes) != cudaSuccess) {
-        cudaGetLastError();
-        cudaFree(spec);
-        return;
-    }
-    cudaMemset(spec, 0, cbytes);
-    cudaEvent_t e0, e1;
-    cudaEventCreate(&e0);
-    cudaEventCreate(&e1);
-    for (int i = 0; i < n; ++i) {
-        const int M = Ms[i];
-        cufftHandle h;
-        int dims[3] = {M, M, M};
-        if (cufftPlanMany(&h, 3, dims, nullptr, 1, M * M * (M / 2 + 1), nullptr, 1, M * M * M,
-                          sizeof(T) == 4 ? CUFFT_C2R : CUFFT_Z2D, 3) != CUFFT_SUCCESS)
-            continue;
+        pse_params q = p;
+        q.autotune = 0;
+        q.grid_M = Ms[i];
+        if (xis) q.xi = xis[i];
+        pse_ctx *c = nullptr;
+        if (create_impl(&c, L, a, &q, nspec, radii) != PSE_OK) continue;
         float ms = 0.f;
-        for (int rep = 0; rep < 4; ++rep) {
-            if (rep == 1) cudaEventRecord(e0, 0);
-            if constexpr (sizeof(T) == 4) cufftExecC2R(h, (cufftComplex *)spec, (cufftReal *)grid);
-            else cufftExecZ2D(h, (cufftDoubleComplex *)spec, (cufftDoubleReal *)grid);
-        }
-        cudaEventRecord(e1, 0);
-        cudaEventSynchronize(e1);
-        cudaEventElapsedTime(&ms, e0, e1);
-        cufftDestroy(h);
-        ms_out[i] = ms / 3.f;
+        if ((q.precision == PSE_FP64 ? time_wave<double>(c, N, &ms) : time_wave<float>(c, N, &ms)) == PSE_OK)
+            ms_out[i] = ms;
+        pse_destroy(c);
     }
-    cudaEventDestroy(e0);
-    cudaEventDestroy(e1);
-    cudaFree(spec);
-    cudaFree(grid);
     cudaGetLastError();
 }
 
-// Fastest cuFFT C2R (batch 3) grid among the 2,3,5,7-smooth sizes in
-// [M, 1.12 M] (a finer grid only lowers the quadrature error).
-template <typename T> pse_status tune_fft_size(int M0, int *best_M) {
-    *best_M = M0;
+// The 2,3,5,7-smooth grid in [M0, 1.12 M0] whose wave part is the fastest (a
+// finer grid only lowers the quadrature error), at the particles of a
+// suspension of volume fraction 0.1: none are known when a context is made.
+int tune_fft_size(double L, double a, const pse_params &p, int nspec, const double *radii, int M0) {
     int Ms[64], n = 0;
     for (int M = M0; M <= (int)(M0 * 1.12) + 1 && n < 64; ++M)
         if (smooth_2357(M)) Ms[n++] = M;
     float ms[64];
-    time_fft_sizes<T>(Ms, n, ms);
+    time_wave_grids(L, a, p, nspec, radii, (int64_t)fmin(ceil(0.1 * 3 / (4 * M_PI) * pow(L / a, 3)), 1e15), Ms, nullptr, n, ms);
     float best = 1e30f;
     for (int i = 0; i < n; ++i)
         if (ms[i] < best) {
             best = ms[i];
-            *best_M = Ms[i];
+            M0 = Ms[i];
         }
-    return PSE_OK;
+    return M0;
 }
 
 // Largest xi whose Sec. II C plan fits a grid of M points per side
@@ -1372,8 +1388,7 @@ double xi_max_for_grid(double L, double a, const pse_params &p0, int M) {
     return lo;
 }
 
-pse_status create_impl(pse_ctx **out, double L, double a, const pse_params *p, int nspec = 0,
-                       const double *radii = nullptr) {
+pse_status create_impl(pse_ctx **out, double L, double a, const pse_params *p, int nspec, const double *radii) {
     if (!out) return PSE_EINVAL;
     *out = nullptr;
     if (!p) return PSE_EINVAL;
@@ -1385,9 +1400,8 @@ pse_status create_impl(pse_ctx **out, double L, double a, const pse_params *p, i
     pse_status st = pse_plan(L, a, p, &c->plan);
     if (st != PSE_OK) { delete c; return st; }
     if ((p->autotune & 1) && p->grid_M <= 0) {
-        int Mbest = c->plan.M;
-        st = (p->precision == PSE_FP64) ? tune_fft_size<double>(c->plan.M, &Mbest) : tune_fft_size<float>(c->plan.M, &Mbest);
-        if (st == PSE_OK && Mbest != c->plan.M) {
+        const int Mbest = tune_fft_size(L, a, *p, nspec, radii, c->plan.M);
+        if (Mbest != c->plan.M) {
             c->params.grid_M = Mbest;
             st = pse_plan(L, a, &c->params, &c->plan);
             if (st != PSE_OK) { delete c; return st; }
@@ -1701,8 +1715,8 @@ pse_status pse_profile_stages(pse_ctx *c, int64_t N, const float *d_pos, uint64_
             return PSE_OK;
         }
         launch_grid_noise<float>(c->wf, d.args, c->params.system, d.grid, s);
-        CKF(cufftSetStream(c->fft_r2c, s));
-        CKF(cufftExecR2C(c->fft_r2c, (cufftReal *)d.grid, (cufftComplex *)d.spec));
+        const pse_status ws = grid_to_spec<float>(c, s);
+        if (ws != PSE_OK) return ws;
         launch_wave_apply<float>(c->wf, d.args, c->params.system, d.spec, WAVE_MODE_GRIDNOISE, 0, s);
         return PSE_OK; });
     if (r == PSE_OK && split)
@@ -1746,7 +1760,7 @@ pse_status pse_profile_stages(pse_ctx *c, int64_t N, const float *d_pos, uint64_
 // Mean device time of `reps` samples of a fresh context with parameters p
 // (two untimed samples first: graph capture and launch-shape tuning), its
 // Lanczos count and grid; with `stage`, also the times of one staged sample's
-// neighbour list + matvecs, k-space noise and FFT.
+// neighbour list + matvecs and of its noise, FFT and node-major copy.
 static pse_status xi_trial(double L, double a, const pse_params &p, int64_t N, const float *d_pos, float *d_out,
                            int reps, cudaStream_t s, double *ms, int *iters, int *M, double *stage) {
     pse_ctx *c = nullptr;
@@ -1774,8 +1788,7 @@ static pse_status xi_trial(double L, double a, const pse_params &p, int64_t N, c
         int nl[PSE_NSTAGES];
         st = pse_profile_stages(c, N, d_pos, 1, 900001, d_out, sm, nl, s);
         stage[0] = sm[PSE_STAGE_NEIGHBOURS] + sm[PSE_STAGE_MATVEC];
-        stage[1] = sm[PSE_STAGE_WAVE_NOISE];
-        stage[2] = sm[PSE_STAGE_FFT] + sm[PSE_STAGE_GRID_COPY];
+        stage[1] = sm[PSE_STAGE_WAVE_NOISE] + sm[PSE_STAGE_FFT] + sm[PSE_STAGE_GRID_COPY];
     }
     if (e0) cudaEventDestroy(e0);
     if (e1) cudaEventDestroy(e1);
@@ -1807,12 +1820,12 @@ pse_status pse_tune_xi(double L, double a, const pse_params *p, int64_t N, const
     p0.xi = xi0;
     p0.autotune &= ~8;  // every trial keeps the xi it is given
     out->xi_start = xi0;
-    double stage[3];
+    double stage[2];
     pse_status st = xi_trial(L, a, p0, N, d_pos, d_out, reps, s, &out->ms_tried[0], &out->iters_tried[0],
                              &out->M_tried[0], stage);
     if (st == PSE_OK) {
         out->t_real = stage[0];
-        out->t_wave = stage[1] + stage[2];
+        out->t_wave = stage[1];
         st = pse_xi_model(xi0, out->t_real, out->t_wave, d_f, &out->xi_model);
     }
     if (st != PSE_OK) {
@@ -1845,14 +1858,13 @@ pse_status pse_tune_xi(double L, double a, const pse_params *p, int64_t N, const
         xis[ng++] = xi;
     }
     out->n_grids = ng;
-    float fft_ms[PSE_XI_GRIDS];
-    time_fft_sizes<float>(Ms, ng, fft_ms);
-    // predicted sample time per grid: eq. work's xi-dependent terms from the
-    // start context, the FFT as timed, the rest unchanged
+    float wave_ms[PSE_XI_GRIDS];
+    time_wave_grids(L, a, pg, 0, nullptr, N, Ms, xis, ng, wave_ms);
+    // predicted sample time per grid: eq. work's real term scaled from the
+    // start context, the wave part as timed, the rest unchanged
     double pred[PSE_XI_GRIDS];
     for (int i = 0; i < ng; ++i)
-        pred[i] = out->ms_start - out->t_real - out->t_wave + out->t_real * pow(xi0 / xis[i], d_f) +
-                  stage[1] * pow((double)Ms[i] / M0, 3) + fft_ms[i];
+        pred[i] = out->ms_start - out->t_real - out->t_wave + out->t_real * pow(xi0 / xis[i], d_f) + wave_ms[i];
     int k = 1;
     for (; k < PSE_XI_TRIALS; ++k) {  // time the best predictions in order
         int b = -1;

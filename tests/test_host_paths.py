@@ -33,6 +33,11 @@ def create(L, **kw):
     assert st == 0, st
     return c
 
+# grid points per unit length at xi a = 0.5, tol 1e-3 (k_cut / pi)
+_info = _lib.pse_plan_info()
+assert lib.pse_plan(60.0, 1.0, ctypes.byref(params(xi=0.5)), ctypes.byref(_info)) == 0
+per_length = _info.k_cut / 3.141592653589793
+
 def launches(name):
     return fake.fake_launches(name.encode())
 """ % ROOT
@@ -144,4 +149,56 @@ fake.fake_reset()
 assert lib.pse_sample_with_forces(c, N, P, P, 1, 1, 1.0, 1.0, P, None) == 0
 assert (launches("k_fft_"), launches("k_wave_apply")) == ((5, 0) if {forces} else (0, 1))
 lib.pse_destroy(c)
+""")
+
+
+COSTS = """
+def costs(own, c2r):  # ms: each own pass; the C2R; noise and copy take 0.2 each
+    for name, ms in ((b"k_fft_", own), (b"C2R", c2r), (b"k_wave_noise", 0.2), (b"k_grid_aos", 0.2)):
+        fake.fake_cost(name, ms)
+"""
+
+
+@pytest.mark.parametrize("own,c2r,M", [(0.1, 1.0, 126), (1.0, 1.0, 120), (0.37, 0.9, 126), (0.38, 0.9, 120)])
+def test_grid_tuning_times_the_transforms_that_run(child, own, c2r, M):
+    """autotune bit 0: of the grids 120, 125, 128 (noise kernel, cuFFT, copy)
+    and 126 and 135 (three passes of the library's own, counted 1.15 times) the
+    first of the faster kind is taken; two species too."""
+    child(COSTS + f"""
+costs({own}, {c2r})
+L = 120 / per_length  # the planned grid is 120
+info = _lib.pse_plan_info()
+c = create(L, xi=0.5, autotune=1)
+assert lib.pse_get_plan(c, ctypes.byref(info)) == 0
+assert info.M == {M}, info.M
+lib.pse_destroy(c)
+c = ctypes.c_void_p()
+radii = (ctypes.c_double * 2)(1.0, 1.5)
+costs({own}, {c2r} - 0.2)  # the noise is a launch per species
+assert lib.pse_create_poly(ctypes.byref(c), L, 2, radii, ctypes.byref(params(xi=0.5, autotune=1))) == 0
+assert lib.pse_get_plan(c, ctypes.byref(info)) == 0 and info.M == {M}, info.M
+lib.pse_destroy(c)
+""")
+
+
+def test_xi_tuning_predicts_with_the_transforms_that_run(child):
+    """pse_tune_xi: a candidate's predicted time is the start's, less its
+    xi-dependent stages, plus the scaled real part and the wave part as it
+    would run on the candidate's grid: 1.15 times three passes of 0.1 ms, or
+    0.2 + 0.9 + 0.2 ms.  The reported t_wave is the start grid's."""
+    child(COSTS + """
+costs(0.1, 0.9)
+fake.fake_cost(b"k_nbr", 0.3)
+fake.fake_cost(b"k_lz_matvec", 0.5)
+out = _lib.pse_xi_tuning()
+assert lib.pse_tune_xi(119.9 / per_length, 1.0, ctypes.byref(params(xi=0.5)), 50000, P, 3.0, 2, ctypes.byref(out), None) == 0
+assert out.M_tried[0] == 120 and abs(out.t_wave - 1.3) < 1e-5 and abs(out.t_real - 0.8) < 1e-5
+seen = set()
+for k in range(1, out.n_tried):
+    M = out.M_tried[k]
+    wave = out.ms_pred[k] - (out.ms_start - out.t_real - out.t_wave + out.t_real * (0.5 / out.xi_tried[k]) ** 3)
+    own = M >= 126 and M not in (128, 144)
+    seen.add(own)
+    assert abs(wave - (0.345 if own else 1.3)) < 1e-5, (M, wave)
+assert out.n_tried == 8 and True in seen
 """)
