@@ -242,9 +242,10 @@ typedef struct {
 
 /* Choice of the splitting parameter for a configuration (Sec. II C: the work
  * of eq. work is minimised at xi*).
- *   1. Times `reps` FP32 samples (0 selects 5) of a context created with *p
- *      at xi_start and one staged sample, giving t_real and t_wave; predicts
- *      xi* with pse_xi_model.
+ *   1. Times three rounds of `reps` FP32 samples (0 selects 5), of which the
+ *      fastest counts, of a context created with *p at xi_start and one
+ *      staged sample, giving t_real and t_wave; predicts xi* with
+ *      pse_xi_model.
  *   2. Candidate grids: the 2,3,5,7-smooth sizes that the plan gives between
  *      0.75 xi* and 1.35 xi* (at most PSE_XI_GRIDS).  On a fixed grid the wave
  *      part costs the same for every xi it admits while the real part shrinks
@@ -253,7 +254,7 @@ typedef struct {
  *      for autotune bit 0, with the transforms that a sample of N takes) and
  *      its sample time predicted: the start context's, with that wave part in
  *      place of its own and the real part scaled by eq. work (~ xi^-d_f).
- *   3. The best predictions are timed as whole samples (up to seven), and the
+ *   3. The best predictions are timed as the start (up to seven), and the
  *      fastest trial, the start context included, is reported.
  * Every trial context is destroyed before the next is made; d_pos (3N
  * float32, device, caller order) is only read.  Synchronises `stream`.

@@ -1757,8 +1757,8 @@ pse_status pse_profile_stages(pse_ctx *c, int64_t N, const float *d_pos, uint64_
 }
 
 // ---------------------------------------------------------------- choice of xi
-// Mean device time of `reps` samples of a fresh context with parameters p
-// (two untimed samples first: graph capture and launch-shape tuning), its
+// Mean device time of `reps` samples of a fresh context with parameters p, the
+// fastest of three rounds (two untimed samples first: graph capture and launch-shape tuning), its
 // Lanczos count and grid; with `stage`, also the times of one staged sample's
 // neighbour list + matvecs and of its noise, FFT and node-major copy.
 static pse_status xi_trial(double L, double a, const pse_params &p, int64_t N, const float *d_pos, float *d_out,
@@ -1771,14 +1771,22 @@ static pse_status xi_trial(double L, double a, const pse_params &p, int64_t N, c
     for (int i = 0; st == PSE_OK && i < 2; ++i) st = pse_sample(c, N, d_pos, 1, 900000 + i, d_out, s);
     if (st == PSE_OK) st = pse_get_stats(c, &stats);
     if (st == PSE_OK && (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)) st = PSE_ECUDA;
-    if (st == PSE_OK && cudaEventRecord(e0, s) != cudaSuccess) st = PSE_ECUDA;
-    for (int i = 0; st == PSE_OK && i < reps; ++i) st = pse_sample(c, N, d_pos, 1, 900002 + i, d_out, s);
-    if (st == PSE_OK && (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess))
-        st = PSE_ECUDA;
-    if (st == PSE_OK) {
+    // the fastest of three rounds: neighbouring grids differ by a percent
+    // (N = 1e6: M = 240 1.164, 243 1.164, 256 1.156 ms), a first round by up
+    // to three (1.17 to 1.20)
+    float best = 1e30f;
+    for (int round = 0; round < 3 && st == PSE_OK; ++round) {
+        if (cudaEventRecord(e0, s) != cudaSuccess) st = PSE_ECUDA;
+        for (int i = 0; st == PSE_OK && i < reps; ++i) st = pse_sample(c, N, d_pos, 1, 900002 + i, d_out, s);
+        if (st == PSE_OK && (cudaEventRecord(e1, s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess))
+            st = PSE_ECUDA;
+        if (st != PSE_OK) break;
         float t = 0.f;
         cudaEventElapsedTime(&t, e0, e1);
-        *ms = t / reps;
+        best = t < best ? t : best;
+    }
+    if (st == PSE_OK) {
+        *ms = best / reps;
         st = pse_get_stats(c, &stats);
         *iters = stats.lanczos_iters;
         *M = c->plan.M;

@@ -17,6 +17,8 @@ static int ncost;
 static double now_ms;
 static long nmalloc, nlive;
 static int fail_plans, fail_malloc;
+static int slow_n, slow_seen; /* samples of a new context that take slow_ms more */
+static double slow_ms;
 static char last[128];
 static struct { dim3 g, b; size_t smem; void *s; } cfg;
 
@@ -43,6 +45,7 @@ void fake_cost(const char *part, double ms) {
     snprintf(cost[ncost % NCOST].name, sizeof(cost[0].name), "%s", part);
     cost[ncost++ % NCOST].ms = ms;
 }
+void fake_slow_start(int n, double ms) { slow_n = n; slow_ms = ms; }
 static void spend(const char *name) {
     for (int i = ncost - 1; i >= 0; --i)
         if (strstr(name, cost[i].name)) {
@@ -80,6 +83,7 @@ int __cudaLaunchKernel(void *k, dim3 g, dim3 b, void **args, size_t smem, void *
         if (fun[i].host == k) {
             ++fun[i].launches;
             spend(fun[i].name);
+            if (strstr(fun[i].name, "k_lz_final") && slow_seen++ < slow_n) now_ms += slow_ms;
             return 0;
         }
     return 98; /* invalid device function */
@@ -105,7 +109,11 @@ int cudaMalloc(void **p, size_t n) {
     return *p ? 0 : 2;
 }
 int cudaFree(void *p) { nlive -= p != NULL; free(p); return 0; }
-int cudaMallocHost(void **p, size_t n) { *p = calloc(n, 1); return *p ? 0 : 2; }
+int cudaMallocHost(void **p, size_t n) { /* once per context */
+    slow_seen = 0;
+    *p = calloc(n, 1);
+    return *p ? 0 : 2;
+}
 int cudaFreeHost(void *p) { free(p); return 0; }
 int cudaMemcpy(void *d, const void *s, size_t n, int k) { (void)k; memcpy(d, s, n); return 0; }
 int cudaMemcpyAsync(void *d, const void *s, size_t n, int k, void *st) { (void)k; (void)st; memcpy(d, s, n); return 0; }

@@ -18,6 +18,7 @@ lib = _lib.load()
 fake = ctypes.CDLL(None)
 fake.fake_mallocs.restype = fake.fake_live.restype = fake.fake_launches.restype = ctypes.c_long
 fake.fake_cost.argtypes = [ctypes.c_char_p, ctypes.c_double]
+fake.fake_slow_start.argtypes = [ctypes.c_int, ctypes.c_double]
 P = ctypes.c_void_p(64)  # kernels do not run: no position is read
 
 def params(**kw):
@@ -201,4 +202,18 @@ for k in range(1, out.n_tried):
     seen.add(own)
     assert abs(wave - (0.345 if own else 1.3)) < 1e-5, (M, wave)
 assert out.n_tried == 8 and True in seen
+""")
+
+
+def test_xi_tuning_keeps_the_fastest_of_three_rounds(child):
+    """A trial whose first samples run slow (clocks, a first round) counts
+    with its fastest round of `reps` samples."""
+    child("""
+fake.fake_cost(b"k_lz_matvec", 0.5)
+fake.fake_cost(b"k_wave_noise", 0.2)  # (no launch of the library's own transforms)
+fake.fake_slow_start(2 + 3 + 3, 2.0)  # the untimed samples and two rounds of three
+out = _lib.pse_xi_tuning()
+assert lib.pse_tune_xi(119.9 / per_length, 1.0, ctypes.byref(params(xi=0.5)), 50000, P, 3.0, 3, ctypes.byref(out), None) == 0
+assert out.n_tried == 8 and out.M_tried[0] == 120
+assert all(min(abs(t - 0.5), abs(t - 0.7)) < 1e-5 for t in out.ms_tried), list(out.ms_tried)
 """)
