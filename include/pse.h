@@ -100,8 +100,14 @@ typedef struct {
                             particles and neighbours (FP32; pse_get_stats
                             reports it), pair blocks evaluated once per sample
                             and streamed by every product (FP64; reported as
-                            shape 1, whose list they follow), or timed with
-                            autotune bit 2;
+                            shape 1, whose list they follow; where they would
+                            take over a quarter of the device memory that is
+                            free at the first call with this N, the products
+                            read the list instead: the same sums in another
+                            order, so the last bits of an FP64 sample depend
+                            on which it is, and a list shape asked for gives
+                            the same bits everywhere), or timed with autotune
+                            bit 2;
                             1..10 force threads x gathers, block size: 4x4
                             128, 8x2 128, 16x1 128, 4x2 128, 4x4 1024, 4x4
                             512, 8x2 1024, 4x2 1024, 1x4 1024, 2x4 1024;
@@ -273,7 +279,7 @@ pse_status pse_tune_xi(double L, double a, const pse_params *p, int64_t N, const
  * Real part: Lanczos on the sparse M_r (eq. Mreal, App. A) from a cell list,
  * stopped when ||x_j - x_{j-1}|| / ||x_j|| < lanczos_tol (Chow & Saad).
  * Wave part: Hermitian complex noise scaled per mode by eq. Mwave's
- * B^{1/2} and the Gaussian deconvolution, inverse FFT (cuFFT), Gaussian
+ * B^{1/2} and the Gaussian deconvolution, inverse FFT, Gaussian
  * interpolation at the particles (the Spectral-Ewald NUFFT of Sec. II B 2).
  * Returns once the work is queued; whether the Lanczos test passed is
  * reported by pse_get_stats (PSE_ENOTCONVERGED if the cap was hit, with the
