@@ -694,9 +694,10 @@ template <int P> __global__ void __launch_bounds__(128) k_interp4_batch(const BS
 
 // Spreading into the node-major grid, the interpolation's mirror image: a
 // group of P lanes per particle, lane c on the z-node c, one 16-byte vector
-// reduction (all three components) per node.  Bound by the reductions that L2
-// takes (2e5 particles, P = 5: 2.5e7 of them in 73 us, 5.5 TB/s); the tiles of
-// k_spread serialise on shared-memory atomics and their blocks pass through
+// reduction (all three components) per node.  Bound by the reductions on
+// their way through L1TEX and into L2 (2e5 particles, P = 5: 2.5e7 of them in
+// 73 us, 5.5 TB/s of values; L1TEX 84% and L2 70% busy, issue 22%); the tiles
+// of k_spread serialise on shared-memory atomics and their blocks pass through
 // memory twice more (146 us and 78 us for the gather).  Forces calls, tiles ->
 // reductions, us: 1e3 particles 117 -> 114, 1e5 369 -> 305, 2e5 664 -> 493,
 // 1e6 2657 -> 1999; P = 9, 1e5 dense 1393 -> 1115, 3e4 dilute 1912 -> 736; no
@@ -923,9 +924,12 @@ cudaError_t launch_spread(WaveGeom<T> w, Geom<T> g, SpreadTile st, const int *or
 // touch consecutive words in every pass whatever its stride; each pass is one
 // radix of a Stockham transform (natural order in and out), from one buffer
 // to the other.  A thread transforms two neighbouring lines at a time (one
-// 16-byte access, one set of indices and twiddles for both): the passes are
-// bound by instruction issue, and with one line per thread a point cost 39
-// instructions a pass (y pass at M = 200 67 us, of 30 at the memory's rate).
+// 16-byte access, one set of indices and twiddles for both): with one line per
+// thread a point cost 39 instructions a pass (y pass at M = 200 67 us; 48 now,
+// of 30 at the memory's rate).  Bound by issue and the latency between the
+// barriers of a few blocks: at M = 200 x, y and z issue on 60, 48 and 46% of
+// the cycles with a third of the warps resident, z with L1TEX at 71%, DRAM at
+// 6, 35 and 31%.
 constexpr int PSE_FFT_MAXM = 512;
 constexpr int PSE_FFT_TQ = 8;    // (y, kz) modes per block of the x pass
 constexpr int PSE_FFT_TX = 256;  // its threads
